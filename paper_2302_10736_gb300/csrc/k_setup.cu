@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(256) k_phasor(int nb, const double *__restrict
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nb) return;
     double s, c;
-    int_sincos(va[i], tab, &s, &c);
-    const double v = vm[i];
+    int_sincos(ld_after_wait(va + i), tab, &s, &c);
+    const double v = ld_after_wait(vm + i);
     U[i] = make_double4_32a(c, s, v, fast_rcp(v));
     V[i] = make_double2(v * c, v * s);
 }
@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(256) k_phasor_fix(int nb, const double *__rest
     __syncthreads();
     if (i >= nb) return;
     int64_t c, s;
-    int_sincos_q62(va[i], tab, &c, &s);
-    U[i] = make_double4_32a(__longlong_as_double(c), __longlong_as_double(s), vm[i], 0.0);
+    int_sincos_q62(ld_after_wait(va + i), tab, &c, &s);
+    U[i] = make_double4_32a(__longlong_as_double(c), __longlong_as_double(s), ld_after_wait(vm + i), 0.0);
 }
 
 // Upload the trig table once per device (synchronous, first use only).

@@ -64,6 +64,14 @@ __device__ __forceinline__ bool scen_value(const RowOutage &r, int i, int k, int
     return true;
 }
 
+// U[x], written by the phasor launch that the row kernels are dependents of
+__device__ __forceinline__ double4_32a load_u(const double4_32a *U)
+{
+    double4_32a u;
+    ld_after_wait(reinterpret_cast<const double *>(U), u.x, u.y, u.z, u.w);
+    return u;
+}
+
 // U[x] = {2^62 cos, 2^62 sin (64-bit integers stored bit for bit), v, -}
 __device__ __forceinline__ void unpack_u(const double4_32a &u, int64_t *C, int64_t *S)
 {
@@ -154,7 +162,7 @@ __global__ void __launch_bounds__(512) k_inj_ybus_b(int S, int nb, const int *__
         double4_32a uu[kChunkBW<W>];
 #pragma unroll
         for (int j = 0; j < kChunkBW<W>; ++j)
-            if (k0 + W * j < d) uu[j] = Us[jj[j]];
+            if (k0 + W * j < d) uu[j] = load_u(Us + jj[j]);
 #pragma unroll
         for (int j = 0; j < kChunkBW<W>; ++j) {
             const int k = k0 + W * j;
@@ -175,7 +183,7 @@ __global__ void __launch_bounds__(512) k_inj_ybus_b(int S, int nb, const int *__
         Ii += __shfl_xor_sync(0xffffffffu, Ii, off, W);
     }
     if (valid && lane == 0) {
-        const double4_32a ui = Us[i];
+        const double4_32a ui = load_u(Us + i);
         int64_t C, Sn;
         unpack_u(ui, &C, &Sn);
         const double cs = fix_q62_or_nan(C), sn = C == kFixNaN ? cs : q62_to_double(Sn);
@@ -249,7 +257,7 @@ __global__ void __launch_bounds__(512) k_jac_ybus_b(int S, int nb, int nnz, cons
     double dTr = 0.0, dTi = 0.0, dVr = 0.0, dVi = 0.0;   // diagonal partials (lane that owns it)
     int kd = -1;
     double4_32a ui = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-    if (valid) ui = Us[i];
+    if (valid) ui = load_u(Us + i);
     int64_t Crow, Srow;
     unpack_u(ui, &Crow, &Srow);
     const double cs = fix_q62_or_nan(Crow), sn = Crow == kFixNaN ? cs : q62_to_double(Srow);
@@ -271,7 +279,7 @@ __global__ void __launch_bounds__(512) k_jac_ybus_b(int S, int nb, int nnz, cons
         double4_32a uu[kChunkBW<W>];
 #pragma unroll
         for (int j = 0; j < kChunkBW<W>; ++j)
-            if (k0 + W * j < d) uu[j] = Us[jj[j]];
+            if (k0 + W * j < d) uu[j] = load_u(Us + jj[j]);
 #pragma unroll
         for (int j = 0; j < kChunkBW<W>; ++j) {
             const int k = k0 + W * j;

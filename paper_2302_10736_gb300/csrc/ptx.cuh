@@ -149,4 +149,22 @@ __device__ __forceinline__ bool grid_barrier(const GridBar &b, unsigned int *sta
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Loads of what an earlier kernel of the chain writes, to be used after
+// pdl_wait: a load through a const __restrict__ pointer counts as invariant over
+// the kernel, so the compiler may move it above the wait (or through the
+// non-coherent path) and read the values of the call before.
+__device__ __forceinline__ double ld_after_wait(const double *p)
+{
+    double x;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(x) : "l"(p));
+    return x;
+}
+// 32 bytes, 32-byte aligned
+__device__ __forceinline__ void ld_after_wait(const double *p, double &x, double &y, double &z, double &w)
+{
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(x), "=d"(y), "=d"(z), "=d"(w)
+                 : "l"(p));
+}
+
 }  // namespace pf

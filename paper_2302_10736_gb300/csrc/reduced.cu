@@ -116,7 +116,10 @@ __global__ void __launch_bounds__(256) k_reduce(int n, int npvpq, int nnz, const
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
             const long long i = base + u * stride;
-            if (i < total) val[u] = i < n ? (i < npvpq ? P[src[u]] - Ps[src[u]] : Q[src[u]] - Qs[src[u]]) : J[src[u]];
+            if (i < total) {
+                const double x = ld_after_wait((i < n ? (i < npvpq ? P : Q) : J) + src[u]);
+                val[u] = i < n ? x - (i < npvpq ? Ps : Qs)[src[u]] : x;
+            }
         }
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
