@@ -639,6 +639,7 @@ PF_API pf_status grid_set_config(pf_grid *grid, const pf_config *cfg, pf_stream 
         if (st) return st;
         PF_CUDA(cudaStreamSynchronize(s));
     }
+    if (cfg->ybus_lanes != g->cfg.ybus_lanes || cfg->ybus_block != g->cfg.ybus_block) g->ybus_shape_set = 1;
     g->cfg = *cfg;
     return PF_OK;
 }
@@ -758,6 +759,7 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
         }
     }
     st = grid_set_config(grid, &cfg, stream);
+    if (!st) g->ybus_shape_set = 1;
 out:
     if (st) g->cfg = keep;
     cudaFree(ctx.P);

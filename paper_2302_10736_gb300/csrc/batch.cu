@@ -87,6 +87,21 @@ pf_status batch_plan(const Grid *g, int nscen, int tb, int tfac, HostEw &E, bool
     return PF_OK;
 }
 
+// Launch shape of the batched Ybus row kernels for `rows` = scenarios x buses.
+// One lane per row issues the fewest instructions, but below about a thousand
+// rows per SM too few warps are in flight to hide its serial loop over the
+// row's entries, and more lanes per row shorten that loop.  jac_ybus_batched
+// on a GB300, us at 8 / 4 / 2 / 1 lanes (64-thread CTAs): 2,000 rows 5.4 / 6.2
+// / 8.7 / 13.6; 7,500 rows 8.5 / 8.2 / 9.0 / 12.1; 40,000 rows 20 / 15.2 /
+// 13.1 / 16.9; 120,000 rows - / 40 / 28.3 / 32.2; 320,000 rows - / 89 / 53.0 /
+// 51.9; 2.56 M rows - / 708 / 389 / 348.  CTAs of 64 threads leave the shortest
+// tail (2.56 M rows, one lane: 343 us at 32 threads, 348 at 64, 361 at 128).
+static void ybus_rows_shape(long long rows, pf_batch_config &c)
+{
+    c.ybus_lanes = rows <= 4096 ? 8 : rows <= 16384 ? 4 : rows <= 160000 ? 2 : 1;
+    c.ybus_block = 64;
+}
+
 // Upload a window plan, replacing the batch's previous one (synchronizes st).
 pf_status batch_upload(Batch *b, HostEw &E, bool ghost, cudaStream_t st)
 {
@@ -177,8 +192,10 @@ PF_API pf_status batch_create(pf_grid *grid, int32_t nscen, const int32_t *outag
     b->cfg.terminals_per_thread = 0;   // chosen by batch_plan
     b->cfg.ctas_per_sm = 0;
     b->cfg.adjoint_form = 0;
+    // the grid's row-kernel shape where the program chose one, else by size
     b->cfg.ybus_lanes = g->cfg.ybus_lanes;
     b->cfg.ybus_block = g->cfg.ybus_block;
+    if (!g->ybus_shape_set) ybus_rows_shape((long long)nscen * g->nb, b->cfg);
     cudaStream_t st = (cudaStream_t)stream;
     HostEw E;
     bool ghost = false;
