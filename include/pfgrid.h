@@ -95,12 +95,12 @@ typedef struct {
 
 /* Launch configuration (chosen by grid_autotune or set by hand). */
 typedef struct {
-    int32_t ybus_lanes;     /* lanes per Ybus row in the CSR kernels: 1, 2, 4, 8, 16 or 32 */
-    int32_t ybus_block;     /* threads per CTA of the CSR kernels (multiple of 32, <= 512) */
+    int32_t ybus_lanes;     /* lanes per Ybus row in the CSR row kernels: 1, 2, 4, 8, 16 or 32 */
+    int32_t ybus_block;     /* threads per CTA of the CSR row kernels (multiple of 32, <= 512) */
     int32_t ew_window;      /* threads per CTA of the element-wise kernels: 128 or 256; a CTA owns a
                                window of consecutive buses with at most that many buses and terminals */
-    int32_t ybus_fused;     /* Ybus method: 1 = the phasor step fused into the row kernel (one launch; each
-                               entry forms its column's phasor), 0 = the phasor step as its own launch */
+    int32_t ybus_fused;     /* Ybus method: 1 = one launch on the element-wise windows (ew_window), 0 = the
+                               phasor step as its own launch, then the CSR row kernel (ybus_lanes, ybus_block) */
 } pf_config;
 
 /* Human-readable name of a status code (static string). */
@@ -160,8 +160,9 @@ pf_status jac_pattern(const pf_grid *grid, int32_t *nnzJ, const int32_t **rowptr
 
 /*
  * Bus injections by the Ybus method (Eq. 1; Sec. IV-B.1 steps 1-3):
- * phasors U = e^{j theta}, V = vm U; I = Ybus V by a CSR SpMV with
- * config.ybus_lanes lanes per row; S = V . conj(I).
+ * phasors U = e^{j theta}, V = vm U; I = Ybus V row by row; S = V . conj(I)
+ * (config.ybus_fused = 1: the row's terms V_i conj(Y_ij V_j), summed; 0: a CSR
+ * SpMV with config.ybus_lanes lanes per row).
  * vm, va [nb] in; P, Q [nb] out (device, caller-owned).
  */
 pf_status inj_ybus(pf_grid *grid, const double *vm, const double *va, double *P, double *Q, pf_stream stream);
@@ -177,9 +178,9 @@ pf_status inj_elementwise(pf_grid *grid, const double *vm, const double *va, dou
 
 /*
  * Jacobian values by the Ybus method (Eqs. 2-4): per Ybus row, one sweep
- * forms Y_ij U_j, the off-diagonal entries and the row current I_i; the
- * diagonal entry is completed once I_i is known (the two passes of Alg. 1,
- * kept row-local).  Values land directly in the canonical layout (Alg. 2).
+ * forms the off-diagonal entries from Y_ij and the row sum (the current I_i, or
+ * V_i conj(I_i) term by term); the diagonal entry is completed once that is
+ * known (the two passes of Alg. 1, kept row-local).  Values land directly in the canonical layout (Alg. 2).
  * vm, va [nb] in; J [4 nnzY] out; P, Q [nb] out or NULL.
  */
 pf_status jac_ybus(pf_grid *grid, const double *vm, const double *va, double *P, double *Q, double *J,

@@ -172,6 +172,8 @@ static pf_status upload_topology(Grid *g, cudaStream_t s)
     PF_CUDA(a.alloc(&g->yv, (size_t)g->nnz));
     PF_CUDA(a.alloc(&g->yfx, (size_t)g->nnz));
     PF_CUDA(a.alloc(&g->yce, (size_t)g->nnz));
+    PF_CUDA(a.alloc(&g->ytfx, 2 * (size_t)g->nl));
+    PF_CUDA(a.alloc(&g->yte, 2 * (size_t)g->nl));
     PF_CUDA(a.alloc(&g->tself, (size_t)T));
     PF_CUDA(a.alloc(&g->tcoup, (size_t)T));
     PF_CUDA(a.alloc(&g->tcfx, (size_t)T));
@@ -436,9 +438,9 @@ PF_API pf_status inj_ybus(pf_grid *grid, const double *vm, const double *va, dou
     if (g->nb == 0) return PF_OK;
     if (!P || !Q) return set_error(PF_EINVAL, "inj_ybus: P or Q is NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    if (g->cfg.ybus_fused) {   // one launch: the phasors formed inside the row kernel
+    if (g->cfg.ybus_fused) {   // one launch on the element-wise windows
         TraceScope t(g, PF_K_INJ_YBUS, s);
-        PF_CUDA(launch_ybus_fused(g, false, vm, va, P, Q, nullptr, s));
+        PF_CUDA(launch_ybus_win(g, false, vm, va, P, Q, nullptr, s));
         return PF_OK;
     }
     {
@@ -479,9 +481,9 @@ PF_API pf_status jac_ybus(pf_grid *grid, const double *vm, const double *va, dou
     if (!J) return set_error(PF_EINVAL, "jac_ybus: J is NULL");
     if ((P == nullptr) != (Q == nullptr)) return set_error(PF_EINVAL, "jac_ybus: P and Q must both be set or both NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    if (g->cfg.ybus_fused) {   // one launch: the phasors formed inside the row kernel
+    if (g->cfg.ybus_fused) {   // one launch on the element-wise windows
         TraceScope t(g, PF_K_JAC_YBUS, s);
-        PF_CUDA(launch_ybus_fused(g, true, vm, va, P, Q, J, s));
+        PF_CUDA(launch_ybus_win(g, true, vm, va, P, Q, J, s));
         return PF_OK;
     }
     {
@@ -723,24 +725,29 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
     pf_config cfg = g->cfg, keep = g->cfg;
     float best_y = 1e30f, best_e = 1e30f;
     const int lanes[] = {1, 2, 4, 8, 16, 32}, blocks[] = {128, 256, 512};
-    for (int fused : {0, 1})
-        for (int w : lanes)
-            for (int bk : blocks) {
-                g->cfg.ybus_fused = fused;
-                g->cfg.ybus_lanes = w;
-                g->cfg.ybus_block = bk;
-                float ms;
-                if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
-                if (ms < best_y) {
-                    best_y = ms;
-                    cfg.ybus_fused = fused;
-                    cfg.ybus_lanes = w;
-                    cfg.ybus_block = bk;
-                }
+    // the row kernels' shape, then the windows (which have none) against it
+    g->cfg.ybus_fused = cfg.ybus_fused = 0;
+    for (int w : lanes)
+        for (int bk : blocks) {
+            g->cfg.ybus_lanes = w;
+            g->cfg.ybus_block = bk;
+            float ms;
+            if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
+            if (ms < best_y) {
+                best_y = ms;
+                cfg.ybus_lanes = w;
+                cfg.ybus_block = bk;
             }
-    g->cfg.ybus_fused = cfg.ybus_fused;
+        }
     g->cfg.ybus_lanes = cfg.ybus_lanes;
     g->cfg.ybus_block = cfg.ybus_block;
+    g->cfg.ybus_fused = 1;
+    {
+        float ms;
+        if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
+        cfg.ybus_fused = ms < best_y;
+    }
+    g->cfg.ybus_fused = cfg.ybus_fused;
     for (int win : {128, 256}) {
         pf_config c2 = g->cfg;
         c2.ew_window = win;

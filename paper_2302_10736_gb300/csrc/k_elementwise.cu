@@ -77,6 +77,10 @@ struct EwArgs {
     const int2 *binv;
     const double *Ps, *Qs;
     double *F, *Jr;
+    // the Ybus method's general row (ybus_row): terminals of every bus and
+    // their {other bus, slot position | flags}
+    const int *tp;
+    const int2 *tnbr;
 };
 
 #ifdef PF_PHASE_PROBE
@@ -116,11 +120,97 @@ __device__ __forceinline__ void store_range(double *x, const double *s, int b0, 
     if ((b1 - ge) & 1) x[b1 - 1] = s[b1 - 1 - b0 + par];
 }
 
+// ---- the Ybus method on the same windows (YBUS) ----
+// Its row sum I_i = sum_j Y_ij V_j enters S_i = V_i conj(I_i) and the diagonal
+// of the Jacobian only through products with V_i, so each entry's term
+// K_ij = V_i conj(Y_ij V_j) = v_j dS_i/dv_j, which the Jacobian needs anyway
+// (Eqs. 3-4), is formed once and summed over the row:
+//     S_i = v_i^2 conj(Y_ii) + sum K,   conj(I_i) U_i = S_i / v_i.
+// An entry of a parallel run holds the run's sum (k_ybus_values writes the
+// values in terminal order, zero for the run's later terminals).  Rows with a
+// magnitude whose products or quotient might leave the range of normal
+// doubles, or with a non-finite angle of their own, take the sum of currents
+// in FP64 instead (ybus_row).
+//
+// Why windows: with W lanes per CSR row and the sine and cosine per entry
+// (the earlier one-launch form) every bus was transformed 3.5 times and the
+// row's results left as scattered 8-byte stores; on windows it is 1.7 times,
+// and the results leave as bulk copies.  70,000 buses, Jacobian back to back:
+// 21.2 -> 9.9 us a call (k_ew: 9.1); 410,000: 98.9 -> 51.9; 25,000, injections,
+// on the device: 10.0 -> 6.0.
+constexpr int kYbusSlowRow = (int)0x80000000;
+
+// a biased exponent within 2^-300 .. 2^300
+__device__ __forceinline__ bool ybus_mid(int e) { return (unsigned)(e - 723) <= 600u; }
+
+// Y_oq of the entry whose parallel run starts at sorted terminal p (zero for a
+// later terminal of a run), summed as k_ybus_values sums it
+__device__ __noinline__ double2 ybus_entry(const EwArgs &a, int p, int kpos)
+{
+    double2 y = make_double2(0.0, 0.0);
+    if (kpos & EW_ACCUM) return y;
+    const int o = a.town[p], pe = a.tp[o + 1];
+    do {
+        const double2 c = a.tcoup[p];
+        y.x += c.x;
+        y.y += c.y;
+        ++p;
+    } while (p < pe && (a.tnbr[p].y & EW_ACCUM));
+    return y;
+}
+
+struct YbusRow {
+    double2 S, dT, dV;   // S_o, dS_o/dtheta_o, dS_o/dv_o
+};
+
+// Row o by its current I_o (Eqs. 1, 3, 4) in FP64, in the order of operations of
+// a row kernel's lane (k_jac_ybus_b)
+__device__ __noinline__ YbusRow ybus_row(const EwArgs &a, int o)
+{
+    double so, co;
+    int_sincos(a.va[o], a.trig, &so, &co);
+    const double v = a.vm[o], Vr = v * co, Vi = v * so;
+    double Ir = 0.0, Ii = 0.0;
+    YbusRow r;
+    const int pe = a.tp[o + 1];
+    bool diag = true;   // still to come
+    for (int p = a.tp[o]; p < pe || diag;) {
+        const int2 nq = p < pe ? a.tnbr[p] : make_int2(o + 1, 0);
+        const bool own = diag && nq.x > o;   // the diagonal's turn in column order
+        if (!own && (nq.y & EW_ACCUM)) {
+            ++p;
+            continue;
+        }
+        const int j = own ? o : nq.x;
+        const double2 y = own ? a.yd[o] : ybus_entry(a, p, nq.y);
+        double s, c;
+        int_sincos(a.va[j], a.trig, &s, &c);
+        const double vj = a.vm[j];
+        const double YUr = fma(y.x, c, -y.y * s), YUi = fma(y.x, s, y.y * c);
+        Ir = fma(vj, YUr, Ir);
+        Ii = fma(vj, YUi, Ii);
+        if (own) {
+            const double sVr = fma(Vr, YUr, Vi * YUi), sVi = fma(Vi, YUr, -Vr * YUi);   // V conj(YU)
+            r.dT = make_double2(vj * sVi, -vj * sVr);
+            r.dV = make_double2(sVr, sVi);
+            diag = false;
+        } else {
+            ++p;
+        }
+    }
+    r.S = make_double2(fma(Vr, Ir, Vi * Ii), fma(Vi, Ir, -Vr * Ii));
+    r.dT.x -= r.S.y;   // + j S
+    r.dT.y += r.S.x;
+    r.dV.x += fma(Ir, co, Ii * so);   // + conj(I) U
+    r.dV.y += fma(Ir, so, -Ii * co);
+    return r;
+}
+
 // One window per CTA; with PERSIST the CTAs loop over the windows
 // (grid-strided), so that the first windows' outputs leave while later
 // windows are evaluated (outputs in host memory, where the host link is the
 // bound).
-template <bool JAC, bool PERSIST, bool RED = false>
+template <bool JAC, bool PERSIST, bool RED = false, bool YBUS = false>
 __device__ __forceinline__ void ew_windows(const EwArgs &a)
 {
     extern __shared__ __align__(16) char smem[];
@@ -236,6 +326,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 int64_t ar, ai;
                 fix_phasor(C, S, v, &ar, &ai);
                 sA[j] = make_longlong2(ar, ai);
+                if (YBUS && (ar == kFixNaN || !ybus_mid(fix_vexp(v)))) bmo.z |= kYbusSlowRow;   // j = tid is the bus
             }
             if (JAC) {
                 // 1/v is read for the window's own buses only: warps of ghost
@@ -282,9 +373,13 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
             if (A.x == kFixNaN || uq.x == kFixNaN || ey == 0 ||
                 !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, yf.x, yf.y, ey, &Gr, &Gi)) {
                 const longlong2 uo = sU[ol];
-                const double2 yc = a.tcoup[t0 + i];
+                const double2 yc = YBUS ? ybus_entry(a, t0 + i, nq.y) : a.tcoup[t0 + i];
                 fix_G(A.x, A.y, vo, uo.x, uo.y, uq.x, uq.y, 0, 0, 0, yc.x, yc.y, &Gr, &Gi);
+                if (YBUS && (nq.y & EW_ACCUM)) Gr = Gi = 0.0;   // in the entry of its run's first terminal
             }
+            // magnitudes whose products might leave the doubles' range: the
+            // row's sums go the general way (ybus_row)
+            if (YBUS && !(ybus_mid(ey) && ybus_mid(fix_vexp(vq)))) sbm[ol].z |= kYbusSlowRow;
             const double Kr = vq * Gr, Ki = vq * Gi;   // K_t = v_q G
             if (JAC) {
                 skg[2 * i] = make_double2(Kr, Ki);
@@ -307,6 +402,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
 
         // ---- reduction: its terminals in sorted order onto every bus ----
         const int pqs = (int)sp.pqs, par = b0 & 1;
+        bool slow_row = false;
         if (JAC) {
             // two threads per bus: x = 2b' + im sums the real (im = 0) or imaginary
             // (im = 1) parts of K of bus b = sord[b'] and writes the entries that
@@ -327,7 +423,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 for (; i < tend; ++i) {
                     sK += kg[4 * i + im];
                     const int kp = skp[i];
-                    if (kp & EW_ACCUM) {   // later branch of a parallel run: add into the run's slot
+                    if (!YBUS && (kp & EW_ACCUM)) {   // later branch of a parallel run: add into the run's slot
                         const int pos = bm.x + (kp & EW_KMASK);
                         if (im) {
                             jst[pos] += kg[4 * i + 1];           // J11 += Re(-j K)
@@ -340,11 +436,23 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 }
                 const double2 dv = sW2[b], sv = sSv[b];   // 2 v conj(Yd), v^2 conj(Yd)
                 const double iv = sW[b].y;
-                const int pos = bm.x + bm.z;
+                const int pos = bm.x + (YBUS ? bm.z & ~kYbusSlowRow : bm.z);
                 jst[(im ? 0 : L) + pos] = neg_if(sK, im);                  // Re / Im of j sum K
                 jst[(im ? L : 0) + pos + d] = fma(sK, iv, im ? dv.y : dv.x);   // 2 v conj(Yd) + sum K / v
                 spq[(im ? pqs : 0) + b + par] = sK + (im ? sv.y : sv.x);      // S = v^2 conj(Yd) + sum K
+                if (YBUS) slow_row |= bm.z < 0;
             }
+            if (YBUS && slow_row)
+                for (int x = tid; x < 2 * nbus; x += TB) {
+                    const int b = sord[x >> 1], im = x & 1;
+                    const int4 bm = sbm[b];
+                    if (bm.z >= 0) continue;
+                    const YbusRow r = ybus_row(a, b0 + b);
+                    const int pos = bm.x + (bm.z & ~kYbusSlowRow);
+                    jst[(im ? 0 : L) + pos] = im ? r.dT.x : r.dT.y;
+                    jst[(im ? L : 0) + pos + bm.y] = im ? r.dV.y : r.dV.x;
+                    spq[(im ? pqs : 0) + b + par] = im ? r.S.y : r.S.x;
+                }
         } else {
             // two threads per bus as above; v^2 from the phasor phase
             const double *k1 = reinterpret_cast<const double *>(skg);   // K.x, K.y per terminal
@@ -359,7 +467,15 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 const double2 y = syd[b];
                 const double v2 = sW2[b].x;
                 spq[(im ? pqs : 0) + b + par] = fma(v2, im ? neg(y.y) : y.x, sK);   // S = v^2 conj(Yd) + sum K
+                if (YBUS) slow_row |= bm.z < 0;
             }
+            if (YBUS && slow_row)
+                for (int x = tid; x < 2 * nbus; x += TB) {
+                    const int b = sord[x >> 1], im = x & 1;
+                    if (sbm[b].z >= 0) continue;
+                    const YbusRow r = ybus_row(a, b0 + b);
+                    spq[(im ? pqs : 0) + b + par] = im ? r.S.y : r.S.x;
+                }
         }
 
         // ---- stores ----
@@ -449,6 +565,13 @@ __global__ void __launch_bounds__(256, 5) k_ew(EwArgs a)
     ew_windows<JAC, false>(a);
 }
 
+// the same by the Ybus method (one launch)
+template <bool JAC>
+__global__ void __launch_bounds__(256, 5) k_ybus_win(EwArgs a)
+{
+    ew_windows<JAC, false, false, true>(a);
+}
+
 // the Jacobian evaluation with its outputs in host memory (persistent CTAs)
 __global__ void __launch_bounds__(256, 5) k_ew_host(EwArgs a)
 {
@@ -467,7 +590,7 @@ static bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // persistent CTAs per SM of the host-output evaluation
 constexpr int kEwHostCtasPerSm = 2;
 
-enum class EwOut { device, host, reduced };
+enum class EwOut { device, host, reduced, ybus };
 
 template <bool JAC>
 static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double *P, double *Q, double *J,
@@ -484,13 +607,17 @@ static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double
     // over the windows, so the host link carries the first windows' outputs
     // while the later ones are evaluated
     const bool persist = out == EwOut::host && JAC;
-    const bool red = out == EwOut::reduced && JAC;
-    uint32_t &conf = persist ? g->ew_smem_host : red ? g->ew_smem_red : JAC ? g->ew_smem_jac : g->ew_smem_inj;
+    const bool red = out == EwOut::reduced && JAC, ybus = out == EwOut::ybus;
+    uint32_t &conf = persist ? g->ew_smem_host
+                     : red   ? g->ew_smem_red
+                     : ybus  ? (JAC ? g->yb_smem_jac : g->yb_smem_inj)
+                             : (JAC ? g->ew_smem_jac : g->ew_smem_inj);
     // conf: the largest size this grid has ensured (the process-wide limit
     // only grows, so a size ensured once stays valid)
     if (smem > 48u * 1024u && smem > conf) {
         cudaError_t e = ensure_dyn_smem(
-            reinterpret_cast<const void *>(persist ? k_ew_host : red ? k_ew_red : k_ew<JAC>), smem);
+            reinterpret_cast<const void *>(persist ? k_ew_host : red ? k_ew_red : ybus ? k_ybus_win<JAC> : k_ew<JAC>),
+            smem);
         if (e != cudaSuccess) return e;
         conf = smem;
     }
@@ -512,7 +639,7 @@ static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double
     a.max_L = L.max_L;
     a.max_nph = max_nph;
     // bulk (TMA) stores for device outputs; plain coalesced stores for host memory
-    a.aligned = out == EwOut::device && (!J || al16(J)) && (!P || (al16(P) && al16(Q)));
+    a.aligned = (out == EwOut::device || ybus) && (!J || al16(J)) && (!P || (al16(P) && al16(Q)));
     a.desc = L.desc;
     a.slotbus = L.slotbus;
     a.bmeta = L.bmeta;
@@ -520,8 +647,10 @@ static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double
     a.town = g->town;
     a.yd = g->bus_yd;
     a.tcoup = g->tcoup;
-    a.tcfx = g->tcfx;
-    a.tce = g->tce;
+    a.tcfx = ybus ? g->ytfx : g->tcfx;
+    a.tce = ybus ? g->yte : g->tce;
+    a.tp = g->tp;
+    a.tnbr = g->tnbr;
     a.trig = trig_table();
     a.tloc = L.tloc;
     a.vm = vm;
@@ -544,6 +673,7 @@ static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double
         return cudaGetLastError();
     }
     if (red) return launch_k(k_ew_red, grid, L.tb, smem, s, true, a);
+    if (ybus) return launch_k(k_ybus_win<JAC>, grid, L.tb, smem, s, true, a);
     return launch_k(k_ew<JAC>, grid, L.tb, smem, s, true, a);
 }
 
@@ -579,6 +709,13 @@ cudaError_t launch_jac_ew_mapped(Grid *g, const double *vm, const double *va, do
 cudaError_t launch_inj_ew(Grid *g, const double *vm, const double *va, double *P, double *Q, cudaStream_t s)
 {
     return launch_ew<false>(g, vm, va, P, Q, nullptr, s, EwOut::device);
+}
+
+cudaError_t launch_ybus_win(Grid *g, bool jac, const double *vm, const double *va, double *P, double *Q, double *J,
+                            cudaStream_t s)
+{
+    return jac ? launch_ew<true>(g, vm, va, P, Q, J, s, EwOut::ybus)
+               : launch_ew<false>(g, vm, va, P, Q, nullptr, s, EwOut::ybus);
 }
 
 }  // namespace pf

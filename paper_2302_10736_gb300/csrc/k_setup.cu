@@ -66,7 +66,8 @@ __global__ void k_branch_constants(int nl, const double *__restrict__ g, const d
 __global__ void k_ybus_values(int nnz, const int *__restrict__ ybeg, const int *__restrict__ yend,
                               const int *__restrict__ ydiag, const double2 *__restrict__ tself,
                               const double2 *__restrict__ tcoup, const double2 *__restrict__ bus_ysh,
-                              double2 *__restrict__ yv, longlong2 *__restrict__ yfx, int *__restrict__ yce)
+                              double2 *__restrict__ yv, longlong2 *__restrict__ yfx, int *__restrict__ yce,
+                              longlong2 *__restrict__ ytfx, int *__restrict__ yte)
 {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nnz) return;
@@ -80,8 +81,18 @@ __global__ void k_ybus_values(int nnz, const int *__restrict__ ybeg, const int *
     }
     yv[e] = acc;
     int64_t fr, fi;
-    yce[e] = fix_block(acc.x, acc.y, &fr, &fi);   // the fixed-point form of the Ybus kernels
+    const int ye = fix_block(acc.x, acc.y, &fr, &fi);   // the fixed-point form of the Ybus kernels
+    yce[e] = ye;
     yfx[e] = make_longlong2(fr, fi);
+    if (d >= 0) return;
+    // in terminal order: the entry at its run's first terminal, a zero with a
+    // representable exponent (no slow path) at the later ones
+    ytfx[ybeg[e]] = make_longlong2(fr, fi);
+    yte[ybeg[e]] = ye;
+    for (int p = ybeg[e] + 1; p < yend[e]; ++p) {
+        ytfx[p] = make_longlong2(0, 0);
+        yte[p] = 1023;
+    }
 }
 
 // Per-bus self sum Yd = y_sh + sum of the self constants of the bus's
@@ -195,7 +206,7 @@ cudaError_t launch_ybus_values(Grid *g, const double *gs, const double *bs, cuda
     if (g->nb > 0) k_bus_shunt<<<nblk(g->nb, 256), 256, 0, s>>>(g->nb, gs, bs, g->bus_ysh);
     if (g->nnz > 0)
         k_ybus_values<<<nblk(g->nnz, 256), 256, 0, s>>>(g->nnz, g->ybeg, g->yend, g->ydiag, g->tself, g->tcoup,
-                                                        g->bus_ysh, g->yv, g->yfx, g->yce);
+                                                        g->bus_ysh, g->yv, g->yfx, g->yce, g->ytfx, g->yte);
     if (g->nb > 0) k_bus_yd<<<nblk(g->nb, 256), 256, 0, s>>>(g->nb, g->tp, g->tself, g->bus_ysh, g->bus_yd);
     return cudaGetLastError();
 }

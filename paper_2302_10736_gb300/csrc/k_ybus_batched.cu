@@ -1,22 +1,29 @@
-// k_ybus_batched.cu - Ybus method (Sec. II-A, IV-B) over a batch of
-// scenarios, each of which may lose one branch (an N-1 contingency).
+// k_ybus_batched.cu - Ybus method (Sec. II-A, IV-B) on the CSR admittance matrix,
+// W lanes per row, over a batch of scenarios, each of which may lose one branch (an N-1 contingency).
 //
 // The base CSR Ybus is shared; scenario s's admittance matrix differs from
 // it only in the rows of the outage branch's two end buses h and k: the
 // branch's terminal constants are taken out of the diagonal entries
 // (Y_hh - Ys_h, Y_kk - Ys_k) and of the coupling entries (Y_hk - Yc_h,
 // Y_kh - Yc_k), and unless a parallel branch keeps it, the coupling pair
-// leaves the pattern altogether.  So W lanes per (scenario, row) run the
-// single-scenario kernels of k_ybus.cu with those corrections applied on the
-// fly, and write the Jacobian compacted onto scenario s's own pattern at
+// leaves the pattern altogether.  So W lanes per (scenario, row) apply those
+// corrections on the fly to the row's sweep,
+//     dS_i/dv_j     = V_i conj(Y_ij U_j)                         (Eq. 4)
+//     dS_i/dtheta_j = -j V_i conj(Y_ij V_j) = -j v_j dS_i/dv_j    (Eq. 3)
+//     I_i          += v_j Y_ij U_j
+// and on the diagonal additionally  +j V_i conj(I_i)  and  +conj(I_i) U_i by
+// the lane that holds it after a W-lane shuffle reduction (Alg. 1's two passes
+// kept row-local; Alg. 1 as printed carries the opposite sign on dS/dtheta;
+// Eq. 3 is used), and write the Jacobian compacted onto scenario s's own pattern at
 // J + joff[s] (the closed form of k_batched.cu):
 //   rowptr_s[i] = rowptr[i] - del ([h < i] + [k < i]),  d_s(i) = d(i) - del [i in {h, k}],
 //   k_s = k - del [k > position of the removed entry in row i].
 // Phasors of all scenarios come first, from the flat phasor kernel, in the
 // fixed-point form (2^62-scaled cosine and sine); the complex products of the
-// base entries run in fixed point on the integer pipe as in k_ybus_fused, the
+// base entries run in fixed point on the integer pipe (fixrot.cuh), the
 // entries an outage changes (and values the fixed-point form does not hold)
-// in FP64.
+// in FP64.  A single evaluation's separate form (pf_config.ybus_fused = 0) is a
+// batch of one scenario without outage.
 #include "fixrot.cuh"
 #include "pf_internal.h"
 #include "ptx.cuh"

@@ -244,6 +244,10 @@ struct Grid {
     // yce = 0 where a value is not representable (the kernels then take yv)
     longlong2 *yfx = nullptr;
     int *yce = nullptr;
+    // the off-diagonal ones again, in the order of the sorted terminals (an
+    // entry at its parallel run's first terminal, zero at the later ones)
+    longlong2 *ytfx = nullptr;
+    int *yte = nullptr;
     int *ybeg = nullptr, *yend = nullptr, *ydiag = nullptr;
     int *kd = nullptr;                     // [nb] diagonal position per row
     // J pattern (device)
@@ -263,7 +267,7 @@ struct Grid {
     double2 *bus_ysh = nullptr;            // [nb]
     double2 *bus_yd = nullptr;             // [nb] bus shunt + sum of the bus's terminal self constants
     EwDev ew;
-    uint32_t ew_smem_jac = 0, ew_smem_inj = 0, ew_smem_host = 0, ew_smem_red = 0;   // dynamic shared memory the kernels are configured for
+    uint32_t ew_smem_jac = 0, ew_smem_inj = 0, ew_smem_host = 0, ew_smem_red = 0, yb_smem_jac = 0, yb_smem_inj = 0;   // dynamic shared memory the kernels are configured for
     int nsm = 0;                                  // SM count (cached)
     int *tmir = nullptr;                   // [2nl] by sorted position: sorted position of the mirror terminal
     // device copies of the current parameters (branch gradients need them)
@@ -370,9 +374,9 @@ struct ScenOut;
 cudaError_t launch_ybus_rows(const Grid *g, int S, bool out, const ScenOut *sc, const long long *joff,
                              const double4_32a *U, bool jac, double *P, double *Q, double *J, int lanes, int blk,
                              cudaStream_t s);
-// the Ybus method with the phasor step fused into the row kernel (one launch)
-cudaError_t launch_ybus_fused(const Grid *g, bool jac, const double *vm, const double *va, double *P, double *Q,
-                              double *J, cudaStream_t s);
+// the Ybus method in one launch on the element-wise windows (k_elementwise.cu)
+cudaError_t launch_ybus_win(Grid *g, bool jac, const double *vm, const double *va, double *P, double *Q, double *J,
+                            cudaStream_t s);
 // element-wise: one CTA per window (phasors of its own and ghost buses, evaluation, reduction)
 cudaError_t ew_blocks_per_sm(int tb, size_t smem, int *per_sm);   // CTAs of k_ew<true> that fit on one SM
 cudaError_t launch_inj_ew(Grid *g, const double *vm, const double *va, double *P, double *Q, cudaStream_t s);
