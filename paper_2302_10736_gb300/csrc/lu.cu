@@ -10,63 +10,44 @@
 //     which keeps the factor close to the matrix on power grids (about 1.5
 //     times its entries on the synthetic grids), and a bus's unknowns stay
 //     adjacent (theta, then v).
-//   * Symbolic factorization of the permuted pattern: the elimination tree and
-//     the pattern of L by row subtrees; U has the transposed pattern, so one
-//     index structure (CSC of L) serves both factors: Lx[p] = L(Li[p], j) and
-//     Ux[p] = U(j, Li[p]) for p in Lp[j] .. Lp[j+1].
-//   * The columns grouped by height in the elimination tree: a column depends
-//     only on its descendants, which are all lower.
+//   * The elimination tree of the buses and its columns' patterns; chains of
+//     the tree whose patterns nest are merged into fronts (supernodes), also
+//     where that adds a bounded share of zeros (merge_fronts), and the unknowns
+//     renumbered so that a front's pivots are consecutive and follow its
+//     subtree's (postorder).
 //
-// Numeric phase (GPU), left-looking Crout factorization without pivoting in
-// gather form: the analysis lists, for every factor slot (i, j), the pairs of
-// slots (L(i, k), U(k, j)) - and for the mirrored U(j, i) the pairs
-// (L(j, k), U(k, i)) - over the k below j that update it, ascending, so every
-// slot is one independent sum:
-//   d   = A(j, j) - sum_k L(j, k) U(k, j)          U(j, j) = d
-//   y_j = F_j    - sum_k L(j, k) y_k               (forward solve, fused)
-//   L(i, j) = (A(i, j) - sum_k L(i, k) U(k, j)) / d,  U(j, i) = A(j, i) - sum_k L(j, k) U(k, i)
-// then the backward solve x_j = (y_j - sum_i U(j, i) x_i) / U(j, j) from the
-// root down.
+// Numeric phase (GPU), multifrontal LU without pivoting (Duff & Reid 1983): a
+// front of p pivots and r border unknowns is a dense (p + r) x (p + r + 1)
+// matrix (the last column the right-hand side) that sums the entries of A whose
+// first unknown it owns and its children's updates; eliminating its pivots
+// leaves the pivot rows of U and y and an r x (r + 1) update for its parent:
+//     l_i = m_ik / m_kk,   m_ij -= l_i m_kj     (k < p; i, j > k, y with it)
+// Backward, x_p = U_pp^-1 (y - U_pr x_r) from the root down.
 //
-// The dynamic schedule (k_lu_solve, a cooperative launch).  No barrier
-// separates the levels: a column depends only on its descendants in the
-// elimination tree, so every work item waits for its column's children to be
-// finished (per-column counters, bounded waits) and the work runs as soon as
-// its inputs exist, along the tree's critical path rather than level by level.
-// Work items are in level order and the warps take them in that order from a
-// shared counter, so the lowest unfinished item has a warp and its inputs, and
-// can always run (all CTAs are resident: cooperative launch).  Wide levels
-// give a warp to a column (a lane per slot); on the upper levels (those with
-// no more slots than the launch has warps) every slot of a column gets a warp
-// of its own (its lanes splitting the slot's sum; each warp forms its
-// column's pivot itself, the same way); the backward solve gives a warp to a
-// column, which waits for its own factorization and then for its parent.
-// What an item needs that no other item writes - its index lists and its own
-// slots' values of A and F - is loaded before its wait, and after the wait all
-// its loads of other columns' factor values are in flight at once (four terms
-// per lane), so a level of the tree costs one round trip to L2 for the values,
-// one for the release of the results and one for the next item's acquire.
-// Values written by other CTAs are read with L1-bypassing loads after an
-// acquire load of the counter that announced them.
+// What bounds it.  The arithmetic is small (1.3 M FMAs at 10,000 buses, 2.5 us
+// of the GPU's FP64 rate); the solve is the latency of the tree's longest path,
+// so it is built around few, cheap dependent steps.  Fronts halve the levels
+// against columns twice over (197 column levels are 22 front levels at 10,000
+// buses), a front's work stays in one warp's or CTA's shared memory, and its
+// only global round trips are its children's updates in and its own out.  A
+// warp that finishes a front counts itself at the parent, and the last child to
+// arrive goes on with the parent (no polling, no schedule).  A warp-wide FP64
+// instruction occupies the SM's FP64 pipe for about 19 cycles whatever its
+// active lanes, so loops are flattened over a front's elements and what is
+// uniform (a pivot's reciprocal) is formed by one warp.
+//   k_mf_small: fronts of at most kMfSmall unknowns with such subtrees, a warp each.
+//   k_mf_big:   the rest (the top of the tree), a CTA each.
+//   k_mf_back_big, k_mf_back_small: the backward solve; a CTA or warp follows
+//     one heavy path of the tree down and waits (bounded) only at its head.
+// One solve, start of this form -> now, back to back: see launch_lu_solve.
 //
-// The tail (k_lu_tail, one thread-block cluster).  At the top of the tree the
-// levels hold one or two columns each, and the schedule above would pay a
-// chain of round trips per column.  The longest run of final columns T0 .. n-1
-// on such levels (closed under the tree's ancestors) is factored as a dense
-// block in the cluster's shared memory; the dynamic launch computes only its
-// entries' terms over the columns outside it (parallel items, after the tail's
-// frontier is finished), and a second dynamic launch solves backward below it.
-// Without a tail (fewer than kLuTailMin such columns) one launch does it all.
-//
-// Every sum has a fixed order (sequential, or lane-strided partial sums joined
-// by a fixed shuffle tree): the results are bitwise repeatable.  A zero or
-// non-finite pivot sets the grid's error word (no trap); a wait that runs out
-// (2 s) sets it to a time-out and ends the warp.
+// Every sum has a fixed order (children in order of their pivots, lane-strided
+// partial sums joined by a fixed shuffle tree): the results are bitwise
+// repeatable.  A zero or non-finite pivot sets the grid's error word (no trap);
+// a wait that runs out (2 s) sets it to a time-out and ends the warp or CTA.
 #include <algorithm>
 #include <set>
 #include <vector>
-
-#include <cooperative_groups.h>
 
 #include "fastmath.cuh"
 #include "pf_internal.h"
@@ -76,30 +57,36 @@ namespace pf {
 
 namespace {
 
-constexpr uint64_t kLuBarrierNs = 2000000000ull;   // bounded grid-barrier wait (2 s)
-constexpr int kLuThreads = 384;
-// the tail: the top of the elimination tree factored as a dense block by one
-// thread-block cluster (shared memory spread over its CTAs)
-constexpr int kLuTailCtas = 8;
-constexpr int kLuTailThreads = 512;
-constexpr int kLuTailMax = 384;   // columns: 48 rows of 384 doubles per CTA
-constexpr int kLuTailMin = 16;    // a shorter top chain stays in the dynamic schedule
-constexpr int kLuTailWidth = 2;   // the tail holds columns of levels at most this wide
+constexpr uint64_t kLuWaitNs = 2000000000ull;   // bounded waits (2 s)
+// classes of fronts, by who eliminates them (kMfClasses): a warp, a CTA, a
+// cluster of CTAs, and, beyond those, a CTA with the front in global memory
+constexpr int kMfSmall = 12, kMfMid = 63, kMfWide = 255;   // most unknowns of a front of the first three
+constexpr int kMfNone = (int)0x80000000;   // no source
+constexpr int kMfSmallLd = 13;        // row stride of a small front (odd: no bank conflicts down a column)
+constexpr int kMfSmallWarps = 16;     // warps per CTA of k_mf_small and k_mf_back_small
+constexpr int kMfMidWarps = 8;        // warps per CTA of the second class
+constexpr int kMfWideWarps = 8, kMfWideCtas = 8;           // of the third
+constexpr int kMfHugeThreads = 512, kMfBackThreads = 512;
+constexpr int kMfBackRows = 160;      // most pivots of a front whose pivot block the backward solve copies to shared memory
+constexpr int kMfMidRows = kMfMid;    // pivot rows kept in shared memory at a time: all of a front of the second class
+constexpr size_t kMfWideRowBytes = 200u * 1024u;           // ... and what fits, of the third
+constexpr size_t kMfMaxSmem = 220u * 1024u;
 
-struct LuArgs {
-    int n, nnzA, nfitems, nbcols;
-    int T0, LpT0;   // the tail's first column and first factor slot (n, nnz(L): no tail)
-    int fr0, fr1;   // the tail's frontier in cidx: the columns outside it whose parent is in it
-    int mode;       // 0 the whole solve; 1 zero, scatter, factorization (the tail's outside terms only); 2 the backward solve outside the tail
-    const int *Lp, *Li, *Rp, *Rk, *Rq, *perm, *amap, *gptr;
-    const int *need, *cptr, *cidx, *parent, *bcols;
-    const int2 *gsrc;     // per update term of a slot: {L(i, k) slot, U(k, j) slot}
-    const int2 *fitems;   // {column, -2 (whole column) or slot or -1 (pivot only)}, level order
+struct MfArgs {
+    int n, nf, nnzA;
+    int backmax;            // unknowns of the largest front but the small ones
+    int nleaf[kMfClasses];  // fronts without children of their class
+    int npath[2];           // backward paths of the small fronts, of the others
+    const MfFront *fr;
+    const int *leaf[kMfClasses];   // longest remaining path first
+    const int *path[2];            // heads, top down
+    const int2 *el;         // per element of a front: {its first source (mf_source; kMfNone), its further ones in ext (-1: none)}
+    const int4 *ext;        // {how many, the first three}, then the others
+    const int *bidx;        // per border unknown: its number
+    const int *perm;        // unknown -> reduced index
     const double *A, *F;
-    double *Lx, *Ux, *D, *y, *dx;
-    double *piv;          // [n] the pivots U(j, j) (D keeps A(j, j): every item of a column reads it)
-    int *done;            // [2n + 2]: finished items of column j at j, x_j written at n + j, the item counters
-    unsigned int *bar;
+    double *U, *cb, *x, *dx, *mat;   // pivot rows and y; updates; solution; fronts beyond shared memory
+    int *cnt;               // [nf] children arrived; [nf] x written; item counters
     int *err;
 };
 
@@ -110,55 +97,39 @@ __device__ __forceinline__ int ld_acquire(const int *p)
     return v;
 }
 
-__device__ __forceinline__ unsigned long long lu_gtimer()
+// wait until *p != 0, at most kLuWaitNs; false (and the grid's error word set
+// to a time-out) if it stays 0
+__device__ __forceinline__ bool mf_wait(const MfArgs &a, const int *p)
 {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// wait until *p >= target, at most kLuBarrierNs; false (and the grid's error
-// word set to a time-out) if it never gets there
-__device__ __forceinline__ bool lu_wait(const LuArgs &a, const int *p, int target)
-{
-    if (ld_acquire(p) >= target) return true;
-    const unsigned long long t0 = lu_gtimer();
+    if (ld_acquire(p)) return true;
+    const uint64_t t0 = global_timer_ns();
     for (;;) {
         __nanosleep(20);
-        if (ld_acquire(p) >= target) return true;
-        if (lu_gtimer() - t0 > kLuBarrierNs) {
+        if (ld_acquire(p)) return true;
+        if (global_timer_ns() - t0 > kLuWaitNs) {
             atomicExch(a.err, DEV_TIMEOUT);
             return false;
         }
     }
 }
 
-// every child of column j in the elimination tree finished (the lanes wait for
-// different children); false on a time-out (all lanes agree)
-__device__ __forceinline__ bool lu_wait_children(const LuArgs &a, int j, int lane)
+// wait for a pivot row's slot (phase 0 of its mbarrier), bounded in the same way;
+// no sleep between the polls: the slot's arrival is on the critical path
+__device__ __forceinline__ bool mf_wait_slot(const MfArgs &a, uint64_t *bar)
 {
-    bool ok = true;
-    // a column of the tail reads the outside columns of its whole subtree: it
-    // waits for the tail's frontier
-    const int c0 = j >= a.T0 ? a.fr0 : a.cptr[j], c1 = j >= a.T0 ? a.fr1 : a.cptr[j + 1];
-    for (int t = c0 + lane; t < c1; t += 32) {
-        const int c = a.cidx[t];
-        ok = ok && lu_wait(a, a.done + c, a.need[c]);
+    uint64_t t0 = 0;
+    for (uint32_t i = 1;; ++i) {
+        if (mbar_try_wait(bar, 0)) return true;
+        if (i % 1024 == 0) {
+            const uint64_t t = global_timer_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > kLuWaitNs) {
+                atomicExch(a.err, DEV_TIMEOUT);
+                return false;
+            }
+        }
     }
-    ok = __all_sync(0xffffffffu, ok);
-    __syncwarp();   // orders the waiting lanes' acquires before every lane's reads
-    return ok;
 }
-
-// the warp's writes visible, then one more finished item of column j
-__device__ __forceinline__ void lu_finish(const LuArgs &a, int *cnt, int lane)
-{
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) atomicAdd(cnt, 1);
-}
-
-__device__ __forceinline__ double ldcg(const double *p) { return __ldcg(p); }
 
 __device__ __forceinline__ double warp_sum_d(double x)
 {
@@ -166,449 +137,696 @@ __device__ __forceinline__ double warp_sum_d(double x)
     return x;
 }
 
-__device__ __forceinline__ void pivot_check(const LuArgs &a, double d)
+// 1 / v: the hardware's approximate reciprocal y, 1 / v = y (1 + e + e^2 + ...) with
+// e = 1 - v y exact to rounding and below 2^-19, so the series may stop at e^2:
+// three dependent FP64 operations (64 cycles each) where fast_rcp's two Newton
+// steps take four
+__device__ __forceinline__ double mf_rcp(double v)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    const double e = fma(-v, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+__device__ __forceinline__ void pivot_check(const MfArgs &a, double d)
 {
     if (!(fabs(d) > 0.0) || !isfinite(d)) atomicExch(a.err, DEV_SINGULAR);
 }
 
-// The static part of a work item - index lists fixed by the analysis, and the
-// values of A and F in the item's own slots, which no other item writes - is
-// loaded before the item's wait, so that after it only the factor values of
-// its descendants remain to be read (one round trip instead of three).
+// t / w for 0 <= t < w^2 and 1 <= w <= 2^10 (rw = 1 / w): t + 1/2 is exact and
+// at least 1/2 from every multiple of w, and the quotient, below 2^10, is off by
+// less than 2^-22 of itself, below 1 / (2 w)
+__device__ __forceinline__ int fast_div(int t, float rw) { return (int)(((float)t + 0.5f) * rw); }
 
-// row j's (slot, column) pairs, the first 128 (four per lane, lane-strided)
-struct LuRow {
-    int r, r1;   // the next entry after the loaded ones, the row's end
-    int q[4], k[4];
-};
+// ------------------------------------------------------- factorization ----
 
-__device__ __forceinline__ void lu_row_load(const LuArgs &a, int j, int lane, LuRow &w)
+// a front's source: an element of an update, or (negative) an entry of A or F
+__device__ __forceinline__ double mf_source(const MfArgs &a, int k)
 {
-    const int r0 = a.Rp[j] + lane;
-    w.r1 = a.Rp[j + 1];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int r = r0 + 32 * u;
-        w.k[u] = r < w.r1 ? a.Rk[r] : 0;
-        w.q[u] = r < w.r1 && w.k[u] < a.T0 ? a.Rq[r] : -1;   // k in the tail: the dense phase's term
-    }
-    w.r = r0 + 128;
+    if (k >= 0) return __ldcg(a.cb + k);
+    k = ~k;
+    return k < a.nnzA ? a.A[k] : a.F[k - a.nnzA];
 }
 
-// a slot's update pairs {L(i, k) slot, U(k, j) slot}, the first four of the
-// lane's share: lane-strided (`stride` 32, a warp per slot) or consecutive
-// (`stride` 1, a lane per slot)
-struct LuSlot {
-    int g, g1;
-    int2 s[4];
-};
-
-__device__ __forceinline__ void lu_slot_load(const LuArgs &a, int p, int g0, int stride, LuSlot &w)
+// N elements from their sources, in order (A's entry, then the children's): the
+// first sources and the lists of the further ones are in flight together, then
+// three further ones of each.  The (few) elements with more are left marked in
+// `rest` for mf_gather_rest, so that no loop keeps the next elements' loads back.
+template <int N>
+__device__ __forceinline__ void mf_gather(const MfArgs &a, const int2 (&e)[N], double (&x)[N], uint32_t &rest)
 {
-    w.g1 = a.gptr[p + 1];
+    int4 q[N];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int g = g0 + stride * u;
-        w.s[u] = g < w.g1 ? a.gsrc[g] : make_int2(-1, -1);
-        if (w.s[u].y >= a.LpT0) w.s[u] = make_int2(-1, -1);   // k in the tail: the dense phase's term
+    for (int u = 0; u < N; ++u) q[u] = e[u].y >= 0 ? a.ext[e[u].y] : make_int4(0, 0, 0, 0);
+#pragma unroll
+    for (int u = 0; u < N; ++u) x[u] = e[u].x != kMfNone ? mf_source(a, e[u].x) : 0.0;
+    double v[N][3];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        v[u][0] = q[u].x > 0 ? mf_source(a, q[u].y) : 0.0;
+        v[u][1] = q[u].x > 1 ? mf_source(a, q[u].z) : 0.0;
+        v[u][2] = q[u].x > 2 ? mf_source(a, q[u].w) : 0.0;
     }
-    w.g = g0 + 4 * stride;
-}
-
-// the values of the loaded pairs (after the wait)
-struct LuRowVal {
-    double l[4], uu[4], yk[4];
-};
-struct LuSlotVal {
-    double lx[4], uy[4], ly[4], ux[4];
-};
-
-// (a term the lane does not have reads as 0 x 0, which leaves a sum unchanged
-// but for the sign of a zero; the indices are not needed after the loads)
-__device__ __forceinline__ void lu_row_fetch(const LuArgs &a, const LuRow &w, bool fwd, LuRowVal &v)
-{
+    rest = 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const bool h = w.q[u] >= 0;
-        v.l[u] = h ? ldcg(a.Lx + w.q[u]) : 0.0;
-        v.uu[u] = h ? ldcg(a.Ux + w.q[u]) : 0.0;
-        v.yk[u] = h && fwd ? ldcg(a.y + w.k[u]) : 0.0;
+    for (int u = 0; u < N; ++u) {
+        if (q[u].x > 0) x[u] += v[u][0];
+        if (q[u].x > 1) x[u] += v[u][1];
+        if (q[u].x > 2) x[u] += v[u][2];
+        if (q[u].x > 3) rest |= 1u << u;
     }
 }
 
-__device__ __forceinline__ void lu_slot_fetch(const LuArgs &a, const LuSlot &w, LuSlotVal &v)
+// an element with more than four sources: the fifth on
+__device__ __forceinline__ double mf_gather_rest(const MfArgs &a, int list, double x)
 {
+    for (int n = a.ext[list].x - 3, t = list + 1; n > 0; n -= 8, t += 2) {
+        int4 r[2];
+        double v[8];
+        r[0] = a.ext[t];
+        r[1] = n > 4 ? a.ext[t + 1] : make_int4(0, 0, 0, 0);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const bool h = w.s[u].x >= 0;
-        v.lx[u] = h ? ldcg(a.Lx + w.s[u].x) : 0.0;
-        v.uy[u] = h ? ldcg(a.Ux + w.s[u].y) : 0.0;
-        v.ly[u] = h ? ldcg(a.Lx + w.s[u].y) : 0.0;
-        v.ux[u] = h ? ldcg(a.Ux + w.s[u].x) : 0.0;
-    }
-}
-
-// the lane's part of sum_k L(j, k) U(k, j) and sum_k L(j, k) y_k: the fetched
-// four (first), then the rest of its share of row j, four in flight (rest);
-// lane-strided, so every lane adds its terms in ascending order
-__device__ __forceinline__ double2 lu_row_first(const LuRowVal &v)
-{
-    double dd = 0.0, yy = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        dd = fma(v.l[u], v.uu[u], dd);
-        yy = fma(v.l[u], v.yk[u], yy);
-    }
-    return make_double2(dd, yy);
-}
-
-__device__ __forceinline__ double2 lu_row_rest(const LuArgs &a, const LuRow &w, double2 t)
-{
-    double dd = t.x, yy = t.y;
-    #pragma unroll 1
-    for (int r = w.r; r < w.r1; r += 128) {
-        int q[4], k[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            k[u] = r + 32 * u < w.r1 ? a.Rk[r + 32 * u] : 0;
-            q[u] = r + 32 * u < w.r1 && k[u] < a.T0 ? a.Rq[r + 32 * u] : -1;
+        for (int h = 0; h < 2; ++h) {
+            v[4 * h] = n > 4 * h ? mf_source(a, r[h].x) : 0.0;
+            v[4 * h + 1] = n > 4 * h + 1 ? mf_source(a, r[h].y) : 0.0;
+            v[4 * h + 2] = n > 4 * h + 2 ? mf_source(a, r[h].z) : 0.0;
+            v[4 * h + 3] = n > 4 * h + 3 ? mf_source(a, r[h].w) : 0.0;
         }
-        double l[4], uu[4], yk[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (q[u] >= 0) {
-                l[u] = ldcg(a.Lx + q[u]);
-                uu[u] = ldcg(a.Ux + q[u]);
-                yk[u] = ldcg(a.y + k[u]);
-            }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (q[u] >= 0) {
-                dd = fma(l[u], uu[u], dd);
-                yy = fma(l[u], yk[u], yy);
-            }
+        for (int u = 0; u < 8; ++u)
+            if (n > u) x += v[u];
     }
-    return make_double2(dd, yy);
+    return x;
 }
 
-// sl - sum L(i, k) U(k, j) and su - sum L(j, k) U(k, i) over the lane's share
-// of a slot's pairs: the fetched four (first), then the rest (`stride` as
-// loaded), four in flight, in ascending order (rest)
-__device__ __forceinline__ double2 lu_slot_first(const LuSlotVal &v, double sl, double su)
+// a small front's elements, a lane's share
+constexpr int kMfSmallEl = (kMfSmall * (kMfSmall + 1) + 31) / 32;
+__device__ __forceinline__ void mf_small_el(const MfArgs &a, const MfFront &fr, int2 (&e)[kMfSmallEl], int lane)
 {
+    const int n = fr.f * (fr.f + 1);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        sl = fma(-v.lx[u], v.uy[u], sl);
-        su = fma(-v.ly[u], v.ux[u], su);
-    }
-    return make_double2(sl, su);
+    for (int u = 0; u < kMfSmallEl; ++u)
+        e[u] = lane + 32 * u < n ? a.el[fr.s0 + lane + 32 * u] : make_int2(kMfNone, -1);
 }
 
-__device__ __forceinline__ double2 lu_slot_rest(const LuArgs &a, const LuSlot &w, int stride, double2 t)
+// One small front by one warp, in its shared memory S
+__device__ __forceinline__ void mf_small_front(const MfArgs &a, const MfFront &fr, const int2 (&e)[kMfSmallEl], double *S,
+                                               int lane)
 {
-    double sl = t.x, su = t.y;
-    #pragma unroll 1
-    for (int g = w.g; g < w.g1; g += 4 * stride) {
-        int2 s4[4];
+    const int p = fr.p, f = fr.f, ld = (f + 1) | 1, r = f - p;
+    {
+        double x[kMfSmallEl];
+        uint32_t rest;
+        mf_gather(a, e, x, rest);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            s4[u] = g + stride * u < w.g1 ? a.gsrc[g + stride * u] : make_int2(-1, -1);
-            if (s4[u].y >= a.LpT0) s4[u] = make_int2(-1, -1);
-        }
-        double lx[4], uy[4], ly[4], ux[4];
+        for (int u = 0; u < kMfSmallEl; ++u)
+            if (rest >> u & 1) x[u] = mf_gather_rest(a, e[u].y, x[u]);
+        const float rw = 1.0f / (float)(f + 1);
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (s4[u].x >= 0) {
-                lx[u] = ldcg(a.Lx + s4[u].x);
-                uy[u] = ldcg(a.Ux + s4[u].y);
-                ly[u] = ldcg(a.Lx + s4[u].y);
-                ux[u] = ldcg(a.Ux + s4[u].x);
-            }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (s4[u].x >= 0) {
-                sl = fma(-lx[u], uy[u], sl);
-                su = fma(-ly[u], ux[u], su);
-            }
-    }
-    return make_double2(sl, su);
-}
-
-// A factorization item's static part: its row (the pivot and forward terms),
-// and either the lane's first slot of column j (a warp per column: p0 = -2)
-// or the slot's first pairs (a warp per slot p0 = p >= 0; -1: no slot), with
-// A(j, j), F_j's place in y and the slot's values of A
-struct LuItem {
-    LuRow row;
-    LuSlot slot;
-    int j, p, pfirst, pend;   // column; the lane's (column warp) or the item's slot (-1: none); column j's slots
-    bool colwarp;
-    double d0, y0, l0, u0;    // A(j, j), y_j before the update, the slot's A values (the lane sums' start)
-};
-
-__device__ __forceinline__ void lu_item_load(const LuArgs &a, int j, int p0, int lane, LuItem &it)
-{
-    it.j = j;
-    it.colwarp = p0 == -2;
-    lu_row_load(a, j, lane, it.row);
-    it.pfirst = a.Lp[j];
-    it.pend = a.Lp[j + 1];
-    it.d0 = ldcg(a.D + j);
-    it.y0 = ldcg(a.y + j);
-    it.p = it.colwarp ? (it.pfirst + lane < it.pend ? it.pfirst + lane : -1) : p0;
-    it.l0 = it.u0 = 0.0;
-    it.slot.g = it.slot.g1 = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) it.slot.s[u] = make_int2(-1, -1);
-    if (it.p >= 0) {
-        const int g0 = a.gptr[it.p];
-        lu_slot_load(a, it.p, it.colwarp ? g0 : g0 + lane, it.colwarp ? 1 : 32, it.slot);
-        it.l0 = ldcg(a.Lx + it.p);
-        it.u0 = ldcg(a.Ux + it.p);
-    }
-}
-
-// One factorization item by one warp, after its wait.  A whole column (wide
-// levels, `it.colwarp`): its pivot, then a lane per slot, each slot's update
-// terms in order, four in flight.  One slot of a narrow level's column (p < 0:
-// the column has no slot below the diagonal): the lanes split the slot's
-// terms; every item of a column forms its pivot the same way, and the
-// column's first item also writes the pivot and y_j.  A column of the tail
-// (j >= T0) takes only the terms of columns outside it and keeps its
-// numerators, pivot and y_j unfinished for the dense phase.
-__device__ __forceinline__ void lu_factor(const LuArgs &a, const LuItem &it, int lane)
-{
-    const bool tail = it.j >= a.T0;
-    // y_j is formed by a column warp and by a column's first item only
-    const bool fwd = it.colwarp || it.p < 0 || it.p == it.pfirst;
-    LuRowVal rv;
-    LuSlotVal sv;
-    lu_row_fetch(a, it.row, fwd, rv);
-    lu_slot_fetch(a, it.slot, sv);
-    double2 t = lu_row_first(rv);
-    // a lane's own slot (column warp) starts from A's values, the lane sums of
-    // a warp's slot from 0
-    double2 s = lu_slot_first(sv, it.colwarp ? it.l0 : 0.0, it.colwarp ? it.u0 : 0.0);
-    t = lu_row_rest(a, it.row, t);
-    s = lu_slot_rest(a, it.slot, it.colwarp ? 1 : 32, s);
-    const double d = it.d0 - warp_sum_d(t.x), yj = it.y0 - warp_sum_d(t.y);
-    const double inv = fast_rcp(d);
-    if (it.colwarp) {
-        if (it.p >= 0) {
-            a.Lx[it.p] = s.x * inv;
-            a.Ux[it.p] = s.y;
-            // slots beyond the warp's first 32
-#pragma unroll 1
-            for (int p = it.p + 32; p < it.pend; p += 32) {
-                LuSlot w;
-                w.g = a.gptr[p];
-                w.g1 = a.gptr[p + 1];
-                const double2 s2 = lu_slot_rest(a, w, 1, make_double2(ldcg(a.Lx + p), ldcg(a.Ux + p)));
-                a.Lx[p] = s2.x * inv;
-                a.Ux[p] = s2.y;
-            }
-        }
-    } else if (it.p >= 0) {
-        // the lane sums were formed as 0 - terms: their warp sum is minus the
-        // slot's sum
-        const double sx = warp_sum_d(s.x), sy = warp_sum_d(s.y);
-        if (lane == 0) {
-            a.Lx[it.p] = tail ? it.l0 + sx : (it.l0 + sx) * inv;
-            a.Ux[it.p] = it.u0 + sy;
+        for (int u = 0; u < kMfSmallEl; ++u) {
+            const int t = lane + 32 * u, i = fast_div(t, rw);
+            if (i < f) S[i * ld + (t - i * (f + 1))] = x[u];
         }
     }
-    if (lane == 0 && fwd) {
-        if (!tail) pivot_check(a, d);
-        a.piv[it.j] = d;
-        a.y[it.j] = yj;
-    }
-}
-
-// x_j of the backward solve, in place of y_j (one warp): the column's rows are
-// loaded before any wait, its U values, y_j and pivot once its own
-// factorization is finished, the x of its rows (its ancestors) once its
-// parent's x is written; false on a time-out (all lanes agree)
-__device__ __forceinline__ bool lu_back(const LuArgs &a, int j, int lane)
-{
-    const int p0 = a.Lp[j] + lane, p1 = a.Lp[j + 1], pj = a.parent[j], need = a.need[j], pm = a.perm[j];
-    int li[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) li[u] = p0 + 32 * u < p1 ? a.Li[p0 + 32 * u] : -1;
-    if (!__all_sync(0xffffffffu, lu_wait(a, a.done + j, need))) return false;
     __syncwarp();
-    double ux[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (li[u] >= 0) ux[u] = ldcg(a.Ux + p0 + 32 * u);
-    const double yj = ldcg(a.y + j), pv = ldcg(a.piv + j);
-    if (pj >= 0) {
-        if (!__all_sync(0xffffffffu, lu_wait(a, a.done + a.n + pj, 1))) return false;
+    for (int k = 0; k < p; ++k) {
+        const double dk = S[k * ld + k], inv = mf_rcp(dk);
+        if (k + 1 + lane <= f) S[k * ld + k + 1 + lane] *= inv;
+        if (lane == 31) pivot_check(a, dk);
+        __syncwarp();
+        const int w = f - k, m = f - k - 1;   // columns k + 1 .. f, rows k + 1 .. f - 1
+        const float rw = 1.0f / (float)w;
+        const double *Sk = S + k * ld + k + 1;
+        double *Sb = S + (k + 1) * ld + k;
+        for (int t = lane; t < m * w; t += 32) {
+            const int i = fast_div(t, rw), j = t - i * w;
+            Sb[i * ld + 1 + j] = fma(-Sb[i * ld], Sk[j], Sb[i * ld + 1 + j]);
+        }
         __syncwarp();
     }
-    double s = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (li[u] >= 0) s = fma(ux[u], ldcg(a.y + li[u]), s);
-    #pragma unroll 1
-    for (int p = p0 + 128; p < p1; p += 32) s = fma(ldcg(a.Ux + p), ldcg(a.y + a.Li[p]), s);
-    s = warp_sum_d(s);
-    if (lane == 0) {
-        const double x = (yj - s) * fast_rcp(pv);
-        a.y[j] = x;
-        a.dx[pm] = x;
+    // the pivot rows and y, then the update
+    double *U = a.U + fr.u0;
+    {
+        const float rf = 1.0f / (float)f;
+        for (int t = lane; t < p * f; t += 32) {
+            const int i = fast_div(t, rf), j = t - i * f;
+            U[t] = S[i * ld + j];
+        }
     }
-    return true;
+    if (lane < p) U[p * f + lane] = S[lane * ld + f];
+    {
+        const float rr = 1.0f / (float)(r + 1);
+        for (int t = lane; t < r * (r + 1); t += 32) {
+            const int i = fast_div(t, rr), j = t - i * (r + 1);
+            a.cb[fr.c0 + t] = S[(p + i) * ld + p + j];
+        }
+    }
+    __syncwarp();   // S is read before the next front overwrites it
 }
 
-__global__ void __launch_bounds__(kLuThreads) k_lu_solve(LuArgs a)
+__global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_small(MfArgs a)
 {
-    const GridBar gbar = a.mode != 2 ? grid_barrier_begin(a.bar) : GridBar{nullptr, 0u};
+    extern __shared__ __align__(16) double msm[];
     const int lane = threadIdx.x & 31;
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gthreads = (long long)gridDim.x * blockDim.x;
-    const int nnzL = a.Lp[a.n];
-    unsigned int bk = 0;
-    if (a.mode != 2) {
-        // ---- the factor storage and the counters zeroed, then A and the
-        // right-hand side scattered in ----
-        for (long long t = gtid; t < nnzL; t += gthreads) {
-            a.Lx[t] = 0.0;
-            a.Ux[t] = 0.0;
-        }
-        for (long long t = gtid; t < 2LL * a.n + 2; t += gthreads) a.done[t] = 0;   // and the item counters
-        if (!grid_barrier(gbar, a.bar, gridDim.x, bk++, a.err, DEV_TIMEOUT, kLuBarrierNs)) return;
-        for (long long e = gtid; e < a.nnzA; e += gthreads) {
-            const int code = a.amap[e], slot = code >> 2;
-            const double v = a.A[e];
-            if ((code & 3) == 0)
-                a.Lx[slot] = v;
-            else if ((code & 3) == 1)
-                a.Ux[slot] = v;
-            else
-                a.D[slot] = v;
-        }
-        for (long long j = gtid; j < a.n; j += gthreads) a.y[j] = a.F[a.perm[j]];
-        if (!grid_barrier(gbar, a.bar, gridDim.x, bk++, a.err, DEV_TIMEOUT, kLuBarrierNs)) return;
-    }
-    // ---- every warp takes the next item (factorization and forward solve in
-    // level order, then the backward solve from the root down) from a shared
-    // counter, waits for what the item depends on, and runs it ----
-    int *next = a.done + 2LL * a.n + (a.mode == 2 ? 1 : 0);
-    const int nf = a.mode == 2 ? 0 : a.nfitems;
-    const int nall = nf + (a.mode == 1 ? 0 : a.nbcols);
+    double *S = msm + (size_t)(threadIdx.x >> 5) * (kMfSmall * kMfSmallLd);
+    int *next = a.cnt + 2 * a.nf;
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(next, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= nall) break;
-        if (t < nf) {   // once the column's children are finished
-            const int2 fi = a.fitems[t];
-            LuItem it;
-            lu_item_load(a, fi.x, fi.y, lane, it);
-            if (!lu_wait_children(a, fi.x, lane)) return;
-            lu_factor(a, it, lane);
-            lu_finish(a, a.done + fi.x, lane);
-        } else {   // x_j once its own factorization is finished and its parent's x is written
-            const int j = a.bcols[t - nf];
-            if (!lu_back(a, j, lane)) return;
-            lu_finish(a, a.done + a.n + j, lane);
+        if (t >= a.nleaf[0]) break;
+        MfFront fr = a.fr[a.leaf[0][t]];
+        int2 e[kMfSmallEl];
+        mf_small_el(a, fr, e, lane);
+        for (;;) {
+            // the parent's plan is in flight while this front is eliminated, in
+            // case this warp is the last child to arrive and goes on with it
+            const bool up = fr.parent_need > 0;   // 0: a root, or the parent is of another class
+            const MfFront nx = a.fr[up ? fr.parent : 0];
+            mf_small_front(a, fr, e, S, lane);
+            if (!up) break;
+            mf_small_el(a, nx, e, lane);
+            int arrived = 0;
+            if (lane == 0) {
+                __threadfence();
+                arrived = atomicAdd(a.cnt + fr.parent, 1);
+                __threadfence();
+            }
+            arrived = __shfl_sync(0xffffffffu, arrived, 0);
+            if (arrived + 1 != fr.parent_need) break;
+            __syncwarp();   // lane 0's fence before every lane's reads of the other children's updates
+            fr = nx;
         }
     }
 }
 
-// The tail (columns T0 .. n-1, the top of the elimination tree, where the
-// dynamic schedule would pay a chain of L2 round trips per column) as a dense
-// block of m = n - T0 rows and columns, by one cluster of kLuTailCtas CTAs:
-// row i of the block lives in the shared memory of CTA i mod C (row-cyclic,
-// so every step's rows are spread over all CTAs), and the CTAs read the
-// current pivot row, y_k and x_k from each other's shared memory.  On entry
-// the tail's slots hold A's values less the terms of the columns outside the
-// tail (L numerators, U values, the pivots' and y's partial sums); the kernel
-// finishes them right-looking in the same order of terms as a column of the
-// dynamic schedule (k ascending, one fused multiply-add per term), solving
-// L y = F on the way, then solves U x = y backward, writes x_j into y_j and
-// dx, and marks the tail's x written for the backward solve below it.  One
-// cluster barrier per step (a warp per row in the factorization, a thread per
-// row in the backward solve, so that no other barrier is needed there).
-// Cluster barriers are hardware barriers every CTA passes the same number of
-// times.
-__global__ void __cluster_dims__(kLuTailCtas, 1, 1) __launch_bounds__(kLuTailThreads, 1) k_lu_tail(LuArgs a)
-{
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    extern __shared__ __align__(16) double tsm[];
-    constexpr int C = kLuTailCtas;
-    const int rank = (int)cl.block_rank();
-    const int T0 = a.T0, m = a.n - T0, R = (m + C - 1) / C;
-    const int tid = threadIdx.x, TB = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = TB >> 5;
-    double *S = tsm;                        // [R][m]: block rows rank, rank + C, rank + 2C, ...
-    double *yv = S + (size_t)R * m;         // [R] y, then the right-hand side of the backward solve
-    double *xl = yv + R;                    // [R] x
-    double *prow = xl + R;                  // [m + 1] the current pivot row (columns k .. m-1) and y_k
-    const int nown = rank < m ? (m - 1 - rank) / C + 1 : 0;   // rows of this CTA
-    // ---- the block: column jj's slots give L(ii, jj) to row ii's CTA and
-    // U(jj, ii) to row jj's ----
-    for (int t = tid; t < R * m; t += TB) S[t] = 0.0;
-    __syncthreads();
-    for (int jj = wid; jj < m; jj += nw) {
-        const int j = T0 + jj;
-        for (int p = a.Lp[j] + lane; p < a.Lp[j + 1]; p += 32) {
-            const int ii = a.Li[p] - T0;
-            if (ii % C == rank) S[(size_t)(ii / C) * m + jj] = __ldcg(a.Lx + p);
-            if (jj % C == rank) S[(size_t)(jj / C) * m + ii] = __ldcg(a.Ux + p);
-        }
-        if (lane == 0 && jj % C == rank) {
-            S[(size_t)(jj / C) * m + jj] = __ldcg(a.piv + j);
-            yv[jj / C] = __ldcg(a.y + j);
+// ---- fronts in registers ----
+//
+// A CTA's (NC = 1) or cluster's warps hold the front in registers: a warp holds a
+// row, a column per lane and 32-column block, and the rows go round the warps
+// (warp gw has rows gw, gw + NW, ...).  The warp that
+// owns row k scales it by its pivot's reciprocal (so that U has a unit diagonal
+// and the multipliers are the plain column: no other FP64 instruction is
+// uniform) and puts it into slot k of every CTA's shared memory, where an
+// mbarrier per slot announces it; every warp then takes row k out of its rows.
+// No barrier joins the warps: the owner of row k + 1 updates that row first and
+// sends it on while the others still work on row k, so a step costs the chain
+// wait - multiply-add - reciprocal - scale - send or the FP64 time of the rows,
+// whichever is longer.  Slots are not reused within a batch of rows; a batch
+// ends with a barrier of all warps, writes its rows to U and starts afresh.
+template <int NC>
+struct MfGroup {
+    uint64_t *bar;      // [rows] mbarriers
+    double *row;        // [rows][32 C2] pivot rows
+    int rank;           // this CTA in the cluster
+    int gw;             // this warp among the group's
+    bool dead;          // a wait ran out: no further waits
+    uint32_t rrow[NC], rbar[NC];   // row and bar in every CTA of a cluster
+
+    __device__ __forceinline__ MfGroup(uint64_t *bar_, double *row_, int rank_, int gw_)
+        : bar(bar_), row(row_), rank(rank_), gw(gw_), dead(false)
+    {
+        if (NC > 1)
+            for (int q = 0; q < NC; ++q) {
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rrow[q]) : "r"(smem_addr(row)), "r"(q));
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar[q]) : "r"(smem_addr(bar)), "r"(q));
+            }
+    }
+
+    __device__ __forceinline__ void sync() const
+    {
+        if (NC == 1) {
+            __syncthreads();
+        } else {
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         }
     }
-    cl.sync();
-    // ---- factorization and forward solve, one pivot per step: the pivot row
-    // copied in, then a warp per row below it ----
-    for (int k = 0; k < m; ++k) {
-        const int own = k % C, kr = k / C;
-        const double *Sk = cl.map_shared_rank(S, own) + (size_t)kr * m;
-        for (int c = k + tid; c < m; c += TB) prow[c] = Sk[c];
-        if (tid == TB - 1) prow[m] = *cl.map_shared_rank(yv + kr, own);
-        __syncthreads();
-        const double d = prow[k], inv = fast_rcp(d), yk = prow[m];
-        if (rank == own && tid == 0) pivot_check(a, d);
-        for (int r = (k + C - rank) / C + wid; r < nown; r += nw) {   // this CTA's rows below k
-            double *Sr = S + (size_t)r * m;
-            const double l = Sr[k] * inv;
-            for (int c = k + 1 + lane; c < m; c += 32) Sr[c] = fma(-l, prow[c], Sr[c]);
-            __syncwarp();
-            if (lane == 0) {
-                Sr[k] = l;
-                yv[r] = fma(-l, yk, yv[r]);
+};
+
+// the slots of rows k0 .. k1 - 1 ready to receive (every thread; ends with a
+// barrier of the group)
+template <int NC, int C2>
+__device__ __forceinline__ void mf_slots(const MfGroup<NC> &g, int k0, int k1)
+{
+    for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) mbar_init(g.bar + (k - k0), 1);
+    mbar_fence_init();
+    if (NC > 1) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x)
+            mbar_arrive_expect_tx(g.bar + (k - k0), 256u * (uint32_t)(C2 - k / 32));
+    }
+    g.sync();
+}
+
+// a column of a pivot row into slot `slot` of every CTA
+template <int NC, int C2>
+__device__ __forceinline__ void mf_send(const MfGroup<NC> &g, int slot, int col, double u)
+{
+    const uint32_t at = (uint32_t)slot * (32 * C2) + (uint32_t)col;
+    if (NC == 1) {
+        g.row[at] = u;
+    } else {
+#pragma unroll
+        for (int q = 0; q < NC; ++q)
+            asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(
+                             g.rrow[q] + 8 * at),
+                         "d"(u), "r"(g.rbar[q] + 8 * (uint32_t)slot)
+                         : "memory");
+    }
+}
+
+// rows k0 .. k1 - 1 of the batch from their slots to U and y (the CTAs of a group
+// in turn, a warp per row), and the end of their mbarriers
+template <int NC, int C2>
+__device__ __forceinline__ void mf_rows_out(const MfArgs &a, const MfFront &fr, const MfGroup<NC> &g, int k0, int k1)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, f = fr.f;
+    double *U = a.U + fr.u0;
+    for (int k = k0 + wid * NC + g.rank; k < k1; k += nw * NC) {
+        const double *rw = g.row + (size_t)(k - k0) * (32 * C2);
+        for (int j = k + 1 + lane; j < f; j += 32) U[(size_t)k * f + j] = rw[j];
+        if (lane == 0) U[(size_t)fr.p * f + k] = rw[f];
+    }
+    for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) mbar_inval(g.bar + (k - k0));   // as initialised
+}
+
+// a word of shared memory of every CTA of the group (one thread)
+template <int NC>
+__device__ __forceinline__ void mf_tell(int *word, int value)
+{
+    if (NC == 1) {
+        *(volatile int *)word = value;
+    } else {
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+            uint32_t d;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(smem_addr(word)), "r"(q));
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(d), "r"(value) : "memory");
+        }
+    }
+}
+
+// row k (in mr; block C0, already free of rows 0 .. k - 1) scaled and sent by its warp
+template <int NC, int C2, int C0>
+__device__ __forceinline__ void mf_publish(const MfArgs &a, const MfGroup<NC> &g, const double (&mr)[C2], int k, int slot)
+{
+    const int lane = threadIdx.x & 31;
+    const double d = __shfl_sync(0xffffffffu, mr[C0], k & 31);
+    const double inv = mf_rcp(d);
+#pragma unroll
+    for (int c = C0; c < C2; ++c) mf_send<NC, C2>(g, slot, 32 * c + lane, mr[c] * inv);
+    if (NC == 1) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(g.bar + slot);
+    }
+    if (lane == 0) pivot_check(a, d);
+}
+
+// row k (its columns from block C0 on in u) out of a row
+template <int C2, int C0>
+__device__ __forceinline__ void mf_take(double (&mr)[C2], const double (&u)[C2], int k)
+{
+    const double x = -__shfl_sync(0xffffffffu, mr[C0], k & 31);
+#pragma unroll
+    for (int c = C0; c < C2; ++c) mr[c] = fma(x, u[c], mr[c]);
+}
+
+// the pivots from K0 on: of one column block (the blocks before it are done, their
+// registers are not touched any more) and of one row per warp, so that the
+// registers of a pivot row are known when this is compiled
+template <int NC, int NW, int R, int C2, int K0>
+__device__ __forceinline__ void mf_pivots(const MfArgs &a, const MfFront &fr, MfGroup<NC> &g, int rows, int &kb,
+                                          double (&m)[R][C2])
+{
+    constexpr int N = NW < 32 ? NW : 32, C0 = K0 / 32, Q = K0 / NW;
+    constexpr bool same = (K0 + N) % 32 != 0;   // the next pivots are of the same block
+    const int p = fr.p, gw = g.gw, lane = threadIdx.x & 31;
+    const int last = gw < fr.f ? gw + (fr.f - 1 - gw) / NW * NW : -1;   // this warp's last row
+    const int k1 = min(p, K0 + N);
+    for (int k = K0; k < k1; ++k) {
+        if (k == kb + rows) {   // the batch's slots are used up
+            g.sync();
+            mf_rows_out<NC, C2>(a, fr, g, kb, k);
+            g.sync();
+            kb = k;
+            mf_slots<NC, C2>(g, kb, min(p, kb + rows));
+        }
+        const int slot = k - kb;
+        // a row that its owner could not send ahead: the first of a batch or block
+        if ((slot == 0 || k == 32 * C0) && k % NW == gw) mf_publish<NC, C2, C0>(a, g, m[Q], k, slot);
+        if (last <= k) continue;   // no rows left
+        if (!g.dead) g.dead = !__all_sync(0xffffffffu, mf_wait_slot(a, g.bar + slot));
+        double u[C2];
+        const double *rw = g.row + (size_t)slot * (32 * C2) + lane;
+#pragma unroll
+        for (int c = C0; c < C2; ++c) u[c] = rw[32 * c];
+        // the next pivot row first, and on its way at once
+        const int kn = k + 1;
+        const bool mine = kn < p && kn < kb + rows && kn % NW == gw;
+        const bool here = mine && kn < K0 + N, next = mine && same && kn == K0 + N;
+        if (here) {
+            mf_take<C2, C0>(m[Q], u, k);
+            mf_publish<NC, C2, C0>(a, g, m[Q], kn, slot + 1);
+        }
+        if constexpr (Q + 1 < R)
+            if (next) {
+                mf_take<C2, C0>(m[Q + 1], u, k);
+                mf_publish<NC, C2, C0>(a, g, m[Q + 1], kn, slot + 1);
+            }
+#pragma unroll
+        for (int q = Q; q < R; ++q) {
+            const int i = gw + NW * q;
+            if (!(q == Q && here) && !(q == Q + 1 && next) && i <= last && i > k) mf_take<C2, C0>(m[q], u, k);
+        }
+    }
+    if constexpr ((K0 + N) / 32 < C2 && (K0 + N) / NW < R)
+        if (p > K0 + N) mf_pivots<NC, NW, R, C2, K0 + N>(a, fr, g, rows, kb, m);
+}
+
+template <int NC, int NW, int R, int C2>
+__device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr, MfGroup<NC> &g, int rows)
+{
+    const int p = fr.p, f = fr.f, w = f + 1, r = f - p;
+    const int lane = threadIdx.x & 31, gw = g.gw;
+    // ---- the front's elements: their plan while the slots are made ready, then
+    // their sources, a few at a time ----
+    int2 e[R * C2];
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int c = 0; c < C2; ++c) {
+            const int i = gw + NW * q, j = 32 * c + lane;
+            e[q * C2 + c] = i < f && j < w ? a.el[fr.s0 + i * w + j] : make_int2(kMfNone, -1);
+        }
+    mf_slots<NC, C2>(g, 0, min(p, rows));
+    double m[R][C2];
+    constexpr int G = R * C2 % 4 == 0 ? 4 : 3;   // elements at a time
+    uint32_t rest = 0;
+#pragma unroll
+    for (int t = 0; t < R * C2; t += G) {
+        int2 es[G];
+        double x[G];
+        uint32_t more;
+#pragma unroll
+        for (int u = 0; u < G; ++u) es[u] = e[t + u];
+        mf_gather(a, es, x, more);
+        rest |= more << t;
+#pragma unroll
+        for (int u = 0; u < G; ++u) m[(t + u) / C2][(t + u) % C2] = x[u];
+    }
+    if (rest)
+#pragma unroll
+        for (int t = 0; t < R * C2; ++t)
+            if (rest >> t & 1) m[t / C2][t % C2] = mf_gather_rest(a, e[t].y, m[t / C2][t % C2]);
+    int kb = 0;   // first row of the batch
+    mf_pivots<NC, NW, R, C2, 0>(a, fr, g, rows, kb, m);
+    // ---- the update ----
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int i = gw + NW * q;
+        if (i >= p && i < f) {
+            double *cb = a.cb + fr.c0 + (size_t)(i - p) * (r + 1) - p;
+#pragma unroll
+            for (int c = 0; c < C2; ++c) {
+                const int j = 32 * c + lane;
+                if (j >= p && j <= f) cb[j] = m[q][c];
             }
         }
-        cl.sync();
     }
-    // ---- backward solve: thread r keeps row r's right-hand side; x_k by the
-    // thread of row k, then every row above k takes its term out ----
-    for (int k = m - 1; k >= 0; --k) {
-        const int own = k % C, kr = k / C;
-        if (rank == own && tid == kr) xl[kr] = yv[kr] * fast_rcp(S[(size_t)kr * m + k]);
-        cl.sync();
-        if (tid < nown && tid * C + rank < k)
-            yv[tid] = fma(-S[(size_t)tid * m + k], *cl.map_shared_rank(xl + kr, own), yv[tid]);
-    }
-    // ---- x out, and the tail's x marked written ----
-    for (int r = tid; r < nown; r += TB) {
-        const int j = T0 + r * C + rank;
-        a.y[j] = xl[r];
-        a.dx[a.perm[j]] = xl[r];
-        a.done[a.n + j] = 1;
-    }
-    cl.sync();   // no CTA leaves while another may still read its shared memory
+    g.sync();
+    mf_rows_out<NC, C2>(a, fr, g, kb, p);
 }
 
-// shared memory of k_lu_tail for a tail of m columns
-size_t lu_tail_smem(int m)
+// after a group's front: whether it goes on with the parent (its last child to
+// arrive does).  Every thread; contains barriers of the group.
+template <int NC>
+__device__ __forceinline__ bool mf_climb(const MfArgs &a, const MfFront &fr, const MfGroup<NC> &g, int *s_next)
 {
-    const size_t R = (size_t)(m + kLuTailCtas - 1) / kLuTailCtas;
-    return sizeof(double) * (R * (size_t)m + 2 * R + (size_t)m + 1);
+    g.sync();   // the group's writes, before its arrival
+    if (g.rank == 0 && threadIdx.x == 0) {
+        __threadfence();
+        const int go = atomicAdd(a.cnt + fr.parent, 1) + 1 == fr.parent_need;
+        __threadfence();
+        mf_tell<NC>(s_next, go);
+    }
+    g.sync();
+    return *(volatile int *)s_next != 0;
+}
+
+// the next front of the group's class without children there (-1: none left)
+template <int NC>
+__device__ __forceinline__ int mf_next(const MfArgs &a, int cls, const MfGroup<NC> &g, int *s_next)
+{
+    g.sync();
+    if (g.rank == 0 && threadIdx.x == 0) mf_tell<NC>(s_next, atomicAdd(a.cnt + 2 * a.nf + cls, 1));
+    g.sync();
+    const int t = *(volatile int *)s_next;
+    return t < a.nleaf[cls] ? a.leaf[cls][t] : -1;
+}
+
+__global__ void __launch_bounds__(32 * kMfMidWarps, 2) k_mf_mid(MfArgs a)
+{
+    __shared__ __align__(16) double row[kMfMidRows * 64];
+    __shared__ uint64_t bar[kMfMidRows];
+    __shared__ int s_next;
+    MfGroup<1> g(bar, row, 0, (int)threadIdx.x >> 5);
+    for (int s; (s = mf_next(a, 1, g, &s_next)) >= 0;)
+        for (;;) {
+            const MfFront fr = a.fr[s];
+            if (fr.f < 32)
+                mf_tile_front<1, kMfMidWarps, 4, 1>(a, fr, g, kMfMidRows);
+            else
+                mf_tile_front<1, kMfMidWarps, 8, 2>(a, fr, g, kMfMidRows);
+            if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
+            s = fr.parent;
+        }
+}
+
+__global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWideWarps, 1) k_mf_wide(MfArgs a)
+{
+    extern __shared__ __align__(16) double msm[];
+    __shared__ int s_next;
+    uint32_t rank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    constexpr int NW = kMfWideWarps * kMfWideCtas;
+    // consecutive rows on different SMs
+    MfGroup<kMfWideCtas> g(reinterpret_cast<uint64_t *>(msm), msm + (kMfWide + 1), (int)rank,
+                           ((int)threadIdx.x >> 5) * kMfWideCtas + (int)rank);
+    for (int s; (s = mf_next(a, 2, g, &s_next)) >= 0;)
+        for (;;) {
+            const MfFront fr = a.fr[s];
+            if (fr.f < 128)
+                mf_tile_front<kMfWideCtas, NW, 2, 4>(a, fr, g, (int)(kMfWideRowBytes / 1024));
+            else if (fr.f < 192)
+                mf_tile_front<kMfWideCtas, NW, 3, 6>(a, fr, g, (int)(kMfWideRowBytes / 1536));
+            else
+                mf_tile_front<kMfWideCtas, NW, 4, 8>(a, fr, g, (int)(kMfWideRowBytes / 2048));
+            if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
+            s = fr.parent;
+        }
+    g.sync();   // no CTA leaves while another may still send to it
+}
+
+// One front by one CTA in global memory M: any size
+__device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr, double *M)
+{
+    const int p = fr.p, f = fr.f, ld = (f + 1) | 1, r = f - p;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = kMfHugeThreads >> 5;
+    for (int t = tid; t < f * (f + 1); t += kMfHugeThreads) {
+        const int2 e[1] = {a.el[fr.s0 + t]};
+        double x[1];
+        uint32_t rest;
+        mf_gather(a, e, x, rest);
+        if (rest) x[0] = mf_gather_rest(a, e[0].y, x[0]);
+        M[(size_t)(t / (f + 1)) * ld + t % (f + 1)] = x[0];
+    }
+    __syncthreads();
+    for (int k = 0; k < p; ++k) {
+        double *Mk = M + (size_t)k * ld;
+        const double d = Mk[k], inv = mf_rcp(d);
+        __syncthreads();
+        for (int j = k + 1 + tid; j <= f; j += kMfHugeThreads) Mk[j] *= inv;
+        if (tid == 0) pivot_check(a, d);
+        __syncthreads();
+        for (int i = k + 1 + wid; i < f; i += nw) {
+            double *Mi = M + (size_t)i * ld;
+            const double x = -Mi[k];
+            for (int j = k + 1 + lane; j <= f; j += 32) Mi[j] = fma(x, Mk[j], Mi[j]);
+        }
+        __syncthreads();
+    }
+    double *U = a.U + fr.u0;
+    for (int i = wid; i < p; i += nw) {
+        for (int j = i + 1 + lane; j < f; j += 32) U[(size_t)i * f + j] = M[(size_t)i * ld + j];
+        if (lane == 0) U[(size_t)p * f + i] = M[(size_t)i * ld + f];
+    }
+    for (int i = wid; i < r; i += nw)
+        for (int j = lane; j <= r; j += 32)
+            a.cb[fr.c0 + (size_t)i * (r + 1) + j] = M[(size_t)(p + i) * ld + p + j];
+}
+
+__global__ void __launch_bounds__(kMfHugeThreads) k_mf_huge(MfArgs a)
+{
+    __shared__ int s_next;
+    const MfGroup<1> g(nullptr, nullptr, 0, 0);
+    for (int s; (s = mf_next(a, 3, g, &s_next)) >= 0;)
+        for (;;) {
+            const MfFront fr = a.fr[s];
+            mf_huge_front(a, fr, a.mat + fr.m0);
+            if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
+            s = fr.parent;
+        }
+}
+
+// ------------------------------------------------------ backward solve ----
+
+// The other fronts: x_p of the fronts of one path, from its head down, by one CTA.
+// t = y - U_pr x_r (a warp per row), then U_pp x_p = t (unit diagonal) from the
+// bottom in blocks of 32 rows: a block's triangle by one warp (a lane per row), its
+// terms out of the rows above by a thread per row.  U_pp is copied to shared
+// memory before the wait.
+__global__ void __launch_bounds__(kMfBackThreads) k_mf_back_big(MfArgs a)
+{
+    extern __shared__ __align__(16) double msm[];
+    __shared__ int s_next, s_ok;
+    // the border's x, the pivots' right-hand side, U_pp (of at most kMfBackRows pivots)
+    double *xr = msm, *tv = msm + a.backmax, *T = tv + a.backmax;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int TB = kMfBackThreads, nw = TB / 32;
+    int *next = a.cnt + 2 * a.nf + kMfClasses + 1, *done = a.cnt + a.nf;
+    for (;;) {
+        if (tid == 0) s_next = atomicAdd(next, 1);
+        __syncthreads();
+        const int t = s_next;
+        __syncthreads();
+        if (t >= a.npath[1]) break;
+        int s = a.path[1][t];
+        bool head = true;
+        while (s >= 0) {
+            const MfFront fr = a.fr[s];
+            const int p = fr.p, f = fr.f, r = f - p, ldt = p | 1;
+            const double *U = a.U + fr.u0;
+            const bool whole = p <= kMfBackRows;
+            const int bj = tid < r ? a.bidx[fr.b0 + tid] : 0;
+            if (whole)
+                for (int i = wid; i < p; i += nw)
+                    for (int j = i + 1 + lane; j < p; j += 32) T[i * ldt + j] = U[(size_t)i * f + j];
+            if (head && fr.wait) {
+                if (tid == 0) s_ok = mf_wait(a, done + fr.parent);
+                __syncthreads();
+                if (!s_ok) return;
+            }
+            head = false;
+            for (int j = tid; j < r; j += TB) xr[j] = __ldcg(a.x + (j == tid ? bj : a.bidx[fr.b0 + j]));
+            __syncthreads();
+            for (int i = wid; i < p; i += 2 * nw) {   // two rows at a time
+                const int i2 = i + nw < p ? i + nw : i;
+                double s0 = 0.0, s1 = 0.0;
+#pragma unroll 2
+                for (int j = lane; j < r; j += 32) {
+                    const double x = xr[j];
+                    s0 = fma(U[(size_t)i * f + p + j], x, s0);
+                    s1 = fma(U[(size_t)i2 * f + p + j], x, s1);
+                }
+                s0 = warp_sum_d(s0);
+                s1 = warp_sum_d(s1);
+                if (lane == 0) {
+                    tv[i] = U[(size_t)p * f + i] - s0;
+                    if (i2 != i) tv[i2] = U[(size_t)p * f + i2] - s1;
+                }
+            }
+            __syncthreads();
+            for (int b1 = p; b1 > 0; b1 -= 32) {
+                const int b0 = b1 > 32 ? b1 - 32 : 0, w = b1 - b0;
+                if (wid == 0) {
+                    const double *Ti = whole ? T + (size_t)(b0 + lane) * ldt + b0 : U + (size_t)(b0 + lane) * f + b0;
+                    double x = lane < w ? tv[b0 + lane] : 0.0;
+                    for (int k = w - 1; k > 0; --k) {
+                        const double uk = lane < k ? Ti[k] : 0.0;
+                        const double xk = __shfl_sync(0xffffffffu, x, k);
+                        if (lane < k) x = fma(-uk, xk, x);
+                    }
+                    if (lane < w) {
+                        tv[b0 + lane] = x;
+                        a.x[fr.e0 + b0 + lane] = x;
+                        a.dx[a.perm[fr.e0 + b0 + lane]] = x;
+                    }
+                }
+                __syncthreads();
+                for (int i = tid; i < b0; i += TB) {
+                    const double *Ti = whole ? T + (size_t)i * ldt + b0 : U + (size_t)i * f + b0;
+                    double y = tv[i];
+#pragma unroll 4
+                    for (int k = 0; k < w; ++k) y = fma(-Ti[k], tv[b0 + k], y);
+                    tv[i] = y;
+                }
+                __syncthreads();
+            }
+            if (tid == 0 && fr.light) {   // someone waits for this front
+                __threadfence();
+                atomicExch(done + s, 1);
+            }
+            s = fr.heavy;
+        }
+    }
+}
+
+// Small fronts: the same by one warp; the lanes are (row, part) pairs that split
+// the row's border terms, joined by a shuffle tree.  What does not depend on the
+// fronts above is loaded before the wait.
+__global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_back_small(MfArgs a)
+{
+    extern __shared__ __align__(16) double msm[];
+    const int lane = threadIdx.x & 31;
+    double *W = msm + (size_t)(threadIdx.x >> 5) * (kMfSmall * kMfSmall + kMfSmall);   // pivot rows and y
+    int *next = a.cnt + 2 * a.nf + kMfClasses, *done = a.cnt + a.nf;
+    for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(next, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= a.npath[0]) break;
+        int s = a.path[0][t];
+        bool head = true;
+        while (s >= 0) {
+            const MfFront fr = a.fr[s];
+            const int p = fr.p, f = fr.f, r = f - p;
+            for (int q = lane; q < p * f + p; q += 32) W[q] = a.U[fr.u0 + q];
+            const int bj = lane < r ? a.bidx[fr.b0 + lane] : 0;
+            const int pm = lane < p ? a.perm[fr.e0 + lane] : 0;
+            // the head of a path waits for its parent unless an earlier launch wrote it
+            if (head && fr.wait && !__all_sync(0xffffffffu, mf_wait(a, done + fr.parent))) return;
+            head = false;
+            __syncwarp();
+            const double xb = lane < r ? __ldcg(a.x + bj) : 0.0;
+            // lane = row i + p2 * part g
+            const int p2 = p <= 1 ? 1 : 1 << (32 - __clz(p - 1)), g = lane / p2, i = lane & (p2 - 1), ng = 32 / p2;
+            double sum = 0.0;
+            for (int j0 = 0; j0 < r; j0 += ng) {
+                const int j = j0 + g;
+                const double xj = __shfl_sync(0xffffffffu, xb, j & 31);
+                if (j < r && i < p) sum = fma(W[i * f + p + j], xj, sum);
+            }
+            for (int off = p2; off < 32; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            double x = 0.0;
+            if (i < p) x = W[p * f + i] - sum;
+            for (int k = p - 1; k > 0; --k) {
+                const double xk = __shfl_sync(0xffffffffu, x, k);
+                if (i < k) x = fma(-W[i * f + k], xk, x);
+            }
+            if (lane < p) {
+                a.x[fr.e0 + lane] = x;
+                a.dx[pm] = x;
+            }
+            __syncwarp();
+            if (lane == 0 && fr.light) {   // someone waits for this front
+                __threadfence();
+                atomicExch(done + s, 1);
+            }
+            s = fr.heavy;
+        }
+    }
 }
 
 // ------------------------------------------------------------ analysis ----
@@ -645,10 +863,135 @@ std::vector<int> min_degree_order(std::vector<std::vector<int>> adj)
     return order;
 }
 
+// The fronts of an elimination tree on the buses: node j starts as a front of
+// its own (pivots wt[j] unknowns, border bw[j] unknowns) and takes in a child
+// k's front while that adds few zeros: none at all (the border of k is j and
+// the border of j), or at most 40 % of the merged front's pivot rows and
+// columns up to 16 unknowns (a level of the tree costs 2-3 us, more than the
+// added arithmetic of a small front; 10,000 buses: 9,409 fronts on 29 levels ->
+// 4,209 on 22), and 2 % above.
+struct FrontTree {
+    std::vector<int> top;                     // front -> its top node
+    std::vector<std::vector<int>> members;    // front -> its nodes, ascending
+    std::vector<int> parent;                  // front -> parent front (-1: a root)
+};
+
+FrontTree merge_fronts(const std::vector<int> &par, const std::vector<int> &wt, const std::vector<int> &bw)
+{
+    const int B = (int)par.size();
+    std::vector<std::vector<int>> ch(B), mem(B);
+    std::vector<int> p(wt), owner(B);
+    std::vector<double> zeros(B, 0.0);
+    for (int j = 0; j < B; ++j)
+        if (par[j] >= 0) ch[par[j]].push_back(j);
+    std::vector<char> gone(B, 0);
+    for (int j = 0; j < B; ++j) {
+        mem[j] = {j};
+        for (;;) {
+            int best = -1;
+            double bz = 0.0;
+            for (int k : ch[j]) {
+                const double z = 2.0 * p[k] * (p[j] + bw[j] - bw[k]);
+                if (best < 0 || z < bz) {
+                    best = k;
+                    bz = z;
+                }
+            }
+            if (best < 0) break;
+            const double fn = (double)p[best] + p[j] + bw[j], tot = fn * fn - (double)bw[j] * bw[j];
+            const double z = bz + zeros[best] + zeros[j];
+            if (bz > 0.0 && z > (fn <= 12.0 ? 0.4 : 0.02) * tot) break;
+            zeros[j] = z;
+            p[j] += p[best];
+            gone[best] = 1;
+            mem[j].insert(mem[j].end(), mem[best].begin(), mem[best].end());
+            ch[j].erase(std::find(ch[j].begin(), ch[j].end(), best));
+            ch[j].insert(ch[j].end(), ch[best].begin(), ch[best].end());
+            std::vector<int>().swap(mem[best]);
+            std::vector<int>().swap(ch[best]);
+        }
+    }
+    // postorder of the fronts (children before parents, a subtree consecutive)
+    FrontTree T;
+    std::vector<int> id(B, -1), stack;
+    std::vector<std::pair<int, size_t>> st;
+    for (int j = 0; j < B; ++j) {
+        if (gone[j] || par[j] >= 0) continue;   // a root's top node has no parent
+        st.push_back({j, 0});
+        while (!st.empty()) {
+            auto &[u, c] = st.back();
+            if (c < ch[u].size()) {
+                const int v = ch[u][c++];
+                st.push_back({v, 0});
+                continue;
+            }
+            id[u] = (int)T.top.size();
+            T.top.push_back(u);
+            std::sort(mem[u].begin(), mem[u].end());
+            T.members.push_back(std::move(mem[u]));
+            st.pop_back();
+        }
+    }
+    T.parent.assign(T.top.size(), -1);
+    for (int u : T.top)
+        for (int v : ch[u]) T.parent[id[v]] = id[u];
+    return T;
+}
+
+// The class of every front: the smallest that its size allows, and its subtree's.
+// The classes run one launch after the other, so a long chain of fronts that one
+// class could take holds up the next class's other fronts: chains are cut where
+// the model's time of all three launches is least (rough us of a front, fitted to
+// timestamps of the kernels; 25,000 buses: the small fronts' launch ends after 27
+// instead of 52 us and the next one's after 70 instead of 110).
+void plan_classes(std::vector<MfFront> &fr)
+{
+    const int nf = (int)fr.size();
+    std::vector<int> best(nf), cls(nf);
+    std::vector<double> t[3], cost[3];
+    for (auto &v : cost) v.resize(nf);
+    for (int s = 0; s < nf; ++s) {
+        const int p = fr[s].p, f = fr[s].f;
+        cost[0][s] = 4.5 + 0.6 * p;
+        cost[1][s] = f < 32 ? 3.2 + 0.4 * p : 7.0 + 0.8 * p;
+        cost[2][s] = 6.0 + (f < 128 ? 0.7 : 1.0) * p;
+    }
+    double least = 1e300;
+    for (double lim0 : {15.0, 25.0, 40.0, 1e9})
+        for (double lim1 : {25.0, 40.0, 60.0, 90.0, 1e9}) {
+            for (auto &v : t) v.assign(nf, 0.0);
+            std::fill(cls.begin(), cls.end(), 0);
+            double end[3] = {0.0, 0.0, 0.0}, work[3] = {0.0, 0.0, 0.0};
+            for (int s = 0; s < nf; ++s) {   // t[c][s], cls[s]: so far from its children
+                const int f = fr[s].f;
+                int c = std::max(cls[s], f <= kMfSmall ? 0 : f <= kMfMid ? 1 : f <= kMfWide ? 2 : 3);
+                if (c == 0 && t[0][s] + cost[0][s] > lim0) c = 1;
+                if (c == 1 && t[1][s] + cost[1][s] > lim1) c = 2;
+                cls[s] = c;
+                const int k = std::min(c, 2);
+                t[k][s] += cost[k][s];
+                end[k] = std::max(end[k], t[k][s]);
+                work[k] += cost[k][s];
+                if (const int q = fr[s].parent; q >= 0) {
+                    cls[q] = std::max(cls[q], c);
+                    t[k][q] = std::max(t[k][q], t[k][s]);
+                }
+            }
+            // at least the work over what runs at once (warps, CTAs, clusters of 148 SMs)
+            const double total = std::max(end[0], work[0] / (148 * 16.0)) + std::max(end[1], work[1] / (148 * 2.0)) +
+                                 std::max(end[2], work[2] / 18.0);
+            if (total < least) {
+                least = total;
+                best = cls;
+            }
+        }
+    for (int s = 0; s < nf; ++s) fr[s].cls = best[s];
+}
+
 }  // namespace
 
 pf_status host_lu(int nb, int n, int npvpq, const std::vector<int> &colptr, const std::vector<int> &rowidx,
-                  const std::vector<int> &fmap, int slot_warps, HostLu &L)
+                  const std::vector<int> &fmap, HostLu &L)
 {
     L = HostLu{};
     L.n = n;
@@ -673,188 +1016,211 @@ pf_status host_lu(int nb, int n, int npvpq, const std::vector<int> &colptr, cons
         std::sort(a.begin(), a.end());
         a.erase(std::unique(a.begin(), a.end()), a.end());
     }
-    const std::vector<int> border = min_degree_order(adj);
-    // unknowns in elimination order: each bus's theta, then its v
-    std::vector<int> vidx(nb, -1);
-    for (int k = npvpq; k < n; ++k) vidx[fmap[k]] = k;
-    L.perm.reserve(n);
-    std::vector<int> tidx(nb, -1);
+    std::vector<int> tidx(nb, -1), vidx(nb, -1);
     for (int k = 0; k < npvpq; ++k) tidx[fmap[k]] = k;
-    for (int u : border) {
-        const int b = bus_of[u];
-        L.perm.push_back(tidx[b]);
-        if (vidx[b] >= 0) L.perm.push_back(vidx[b]);
+    for (int k = npvpq; k < n; ++k) vidx[fmap[k]] = k;
+    const std::vector<int> order = min_degree_order(adj);
+    std::vector<int> pos(B);
+    for (int i = 0; i < B; ++i) pos[order[i]] = i;
+    // elimination tree of the ordered buses and the patterns of its columns, by
+    // row subtrees (rows ascending: every column's come out ascending)
+    std::vector<int> par(B, -1), flag(B, -1), wt(B), bw(B, 0);
+    std::vector<std::vector<int>> col(B);
+    for (int i = 0; i < B; ++i) {
+        wt[i] = vidx[bus_of[order[i]]] >= 0 ? 2 : 1;
+        flag[i] = i;
+        for (int u : adj[order[i]]) {
+            int k = pos[u];
+            if (k > i) continue;
+            while (k != -1 && flag[k] != i) {
+                if (par[k] == -1) par[k] = i;
+                col[k].push_back(i);
+                flag[k] = i;
+                k = par[k];
+            }
+        }
+    }
+    for (int i = 0; i < B; ++i)
+        for (int x : col[i]) bw[i] += wt[x];
+    FrontTree T = merge_fronts(par, wt, bw);
+    const int nf = (int)T.top.size();
+    // unknowns renumbered front by front
+    L.perm.reserve(n);
+    std::vector<int> first(B), front_of(B);   // a node's first unknown, its front
+    L.fr.resize(nf);
+    for (int s = 0; s < nf; ++s) {
+        MfFront &f = L.fr[s];
+        f.e0 = (int)L.perm.size();
+        for (int i : T.members[s]) {
+            first[i] = (int)L.perm.size();
+            front_of[i] = s;
+            const int b = bus_of[order[i]];
+            L.perm.push_back(tidx[b]);
+            if (vidx[b] >= 0) L.perm.push_back(vidx[b]);
+        }
+        f.p = (int)L.perm.size() - f.e0;
+        f.parent = T.parent[s];
     }
     if ((int)L.perm.size() != n) return set_error(PF_EINVAL, "jac_reduced_solve: unknowns do not match buses");
-    std::vector<int> iperm(n);
+    std::vector<int> iperm(n), sn(n);
     for (int i = 0; i < n; ++i) iperm[L.perm[i]] = i;
-    // lower pattern of the permuted (symmetrised) matrix, row by row
-    std::vector<std::vector<int>> low(n);
-    for (int c = 0; c < n; ++c)
-        for (int p = colptr[c]; p < colptr[c + 1]; ++p) {
-            const int i = iperm[rowidx[p]], j = iperm[c];
-            if (i > j) low[i].push_back(j);
-            if (j > i) low[j].push_back(i);
-        }
-    for (auto &r : low) {
-        std::sort(r.begin(), r.end());
-        r.erase(std::unique(r.begin(), r.end()), r.end());
+    // borders, update and pivot-row storage
+    long long u0 = 0, c0 = 0, b0 = 0, s0 = 0;
+    std::vector<int> tmp;
+    for (int s = 0; s < nf; ++s) {
+        MfFront &f = L.fr[s];
+        for (int i = 0; i < f.p; ++i) sn[f.e0 + i] = s;
+        tmp.clear();
+        for (int x : col[T.top[s]])
+            for (int w = 0; w < wt[x]; ++w) tmp.push_back(first[x] + w);
+        std::sort(tmp.begin(), tmp.end());
+        const int r = (int)tmp.size();
+        f.f = f.p + r;
+        f.b0 = (int)b0;
+        f.u0 = (int)u0;
+        f.c0 = (int)c0;
+        f.s0 = (int)s0;
+        L.bidx.insert(L.bidx.end(), tmp.begin(), tmp.end());
+        b0 += r;
+        u0 += (long long)f.p * f.f + f.p;
+        c0 += (long long)r * (r + 1);
+        s0 += (long long)f.f * (f.f + 1);
+        if (u0 >= (1LL << 31) || c0 >= (1LL << 31) || s0 >= (1LL << 31) || f.f > 46000)
+            return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: factor too large");
     }
-    // elimination tree and the rows of L by row subtrees
-    std::vector<int> parent(n, -1), flag(n, -1), cnt(n, 0);
-    std::vector<std::vector<int>> lrow(n);
-    for (int i = 0; i < n; ++i) {
-        flag[i] = i;
-        for (int k : low[i]) {
-            while (k != -1 && flag[k] != i) {
-                if (parent[k] == -1) parent[k] = i;
-                lrow[i].push_back(k);
-                cnt[k]++;
-                flag[k] = i;
-                k = parent[k];
-            }
-        }
-        std::sort(lrow[i].begin(), lrow[i].end());
-    }
-    L.Lp.assign(n + 1, 0);
-    for (int j = 0; j < n; ++j) L.Lp[j + 1] = L.Lp[j] + cnt[j];
-    const long long nnzL = L.Lp[n];
-    if (nnzL >= (1LL << 29)) return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: factor too large");
-    L.Li.assign(nnzL, 0);
-    L.Rp.assign(n + 1, 0);
-    L.Rk.reserve(nnzL);
-    L.Rq.reserve(nnzL);
-    std::vector<int> fill(L.Lp.begin(), L.Lp.end() - 1);
-    for (int i = 0; i < n; ++i) {   // rows ascending: every column's rows come out ascending
-        for (int k : lrow[i]) {
-            L.Rk.push_back(k);
-            L.Rq.push_back(fill[k]);
-            L.Li[fill[k]++] = i;
-        }
-        L.Rp[i + 1] = (int)L.Rk.size();
-        std::vector<int>().swap(lrow[i]);
-    }
-    // the update terms of every slot p = (i, j) of column j: for each k of row j
-    // (ascending), the pairs {slot of L(i, k), slot of L(j, k)} over the rows i of
-    // column k below j (all of them are in column j's pattern)
-    auto slot_of = [&](int col, int row) {
-        const auto b = L.Li.begin() + L.Lp[col], e = L.Li.begin() + L.Lp[col + 1];
-        return (int)(std::lower_bound(b, e, row) - L.Li.begin());
+    L.nU = u0;
+    L.nC = c0;
+    // the place of unknown x in front s
+    auto place = [&](int s, int x) {
+        const MfFront &f = L.fr[s];
+        if (x < f.e0 + f.p) return x - f.e0;
+        const auto b = L.bidx.begin() + f.b0, e = b + (f.f - f.p);
+        return f.p + (int)(std::lower_bound(b, e, x) - b);
     };
-    L.gptr.assign(nnzL + 1, 0);
-    for (int j = 0; j < n; ++j)
-        for (int r = L.Rp[j]; r < L.Rp[j + 1]; ++r) {
-            const int k = L.Rk[r], q = L.Rq[r];
-            for (int pp = q + 1; pp < L.Lp[k + 1]; ++pp) L.gptr[slot_of(j, L.Li[pp]) + 1]++;
-        }
-    for (long long p = 0; p < nnzL; ++p) L.gptr[p + 1] += L.gptr[p];
-    if (L.gptr[nnzL] >= (1LL << 30)) return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: factorization too large");
-    L.gsrc.assign(L.gptr[nnzL], make_int2(0, 0));
-    {
-        std::vector<int> gf(L.gptr.begin(), L.gptr.end() - 1);
-        for (int j = 0; j < n; ++j)
-            for (int r = L.Rp[j]; r < L.Rp[j + 1]; ++r) {
-                const int k = L.Rk[r], q = L.Rq[r];
-                for (int pp = q + 1; pp < L.Lp[k + 1]; ++pp) L.gsrc[gf[slot_of(j, L.Li[pp])]++] = make_int2(pp, q);
+    // the place of every border unknown in the parent (both borders ascend)
+    std::vector<int> rel(std::max<long long>(b0, 1), 0);
+    std::vector<std::vector<int>> kids(nf);
+    for (int s = 0; s < nf; ++s) {
+        const MfFront &f = L.fr[s];
+        if (f.parent < 0) continue;
+        kids[f.parent].push_back(s);
+        const MfFront &q = L.fr[f.parent];
+        int at = 0;
+        for (int j = 0; j < f.f - f.p; ++j) {
+            const int x = L.bidx[f.b0 + j];
+            if (x < q.e0 + q.p) {
+                rel[f.b0 + j] = x - q.e0;
+            } else {
+                while (L.bidx[q.b0 + at] != x) ++at;
+                rel[f.b0 + j] = q.p + at;
             }
-    }
-    // levels by height in the tree
-    std::vector<int> height(n, 0);
-    for (int j = 0; j < n; ++j)
-        if (parent[j] >= 0) height[parent[j]] = std::max(height[parent[j]], height[j] + 1);
-    L.H = n ? *std::max_element(height.begin(), height.end()) + 1 : 0;
-    L.lvl_ptr.assign(L.H + 1, 0);
-    for (int j = 0; j < n; ++j) L.lvl_ptr[height[j] + 1]++;
-    for (int h = 0; h < L.H; ++h) L.lvl_ptr[h + 1] += L.lvl_ptr[h];
-    L.lvl_col.assign(n, 0);
-    std::vector<int> lf(L.lvl_ptr.begin(), L.lvl_ptr.end() - 1);
-    for (int j = 0; j < n; ++j) L.lvl_col[lf[height[j]]++] = j;
-    // From the top down, every level whose columns have at most as many slots
-    // as the launch has warps (the widest level's width, or the warps of one
-    // CTA per SM if fewer): every slot of its columns is a work item of its own
-    // (a column without slots below the diagonal still needs its pivot: slot
-    // -1), whose lanes split the slot's update terms, so that a slot costs one
-    // round of loads however many terms it has; below them (wide levels of
-    // short columns) a column is one item, a lane per slot.
-    int widest = 1;
-    for (int h = 0; h < L.H; ++h) widest = std::max(widest, L.lvl_ptr[h + 1] - L.lvl_ptr[h]);
-    const long long budget = std::min<long long>(widest, (long long)slot_warps);
-    auto level_items = [&](int h) {
-        long long c = 0;
-        for (int t = L.lvl_ptr[h]; t < L.lvl_ptr[h + 1]; ++t) {
-            const int j = L.lvl_col[t];
-            c += std::max(1, L.Lp[j + 1] - L.Lp[j]);
         }
-        return c;
-    };
-    L.chain = L.H;
-    while (L.chain > 0 && level_items(L.chain - 1) <= budget) --L.chain;
-    // the tail for the dense phase: the longest run of columns n-1, n-2, ...
-    // (closed under the tree's ancestors, like every final run) on levels at
-    // most kLuTailWidth wide, at most kLuTailMax columns; none below kLuTailMin
-    int T0 = n;
-    while (T0 > 0 && n - T0 < kLuTailMax) {
-        const int h = height[T0 - 1];
-        if (L.lvl_ptr[h + 1] - L.lvl_ptr[h] > kLuTailWidth) break;
-        --T0;
     }
-    if (n - T0 < kLuTailMin) T0 = n;
-    L.T0 = T0;
-    // (the tail's items last: they wait for its whole frontier, and every item
-    // waits only for items before it in the list)
-    L.need.assign(n, 0);
-    for (int pass = 0; pass < 2; ++pass)
-        for (int h = 0; h < L.H; ++h)
-            for (int t = L.lvl_ptr[h]; t < L.lvl_ptr[h + 1]; ++t) {
-                const int j = L.lvl_col[t];
-                if ((j >= T0) != (pass == 1)) continue;
-                if (h < L.chain && j < T0) {
-                    L.fitems.push_back(make_int2(j, -2));
-                } else {
-                    if (L.Lp[j + 1] == L.Lp[j]) L.fitems.push_back(make_int2(j, -1));
-                    for (int p = L.Lp[j]; p < L.Lp[j + 1]; ++p) L.fitems.push_back(make_int2(j, p));
-                }
-                L.need[j] = h < L.chain && j < T0 ? 1 : std::max(1, L.Lp[j + 1] - L.Lp[j]);
-            }
-    // the elimination tree's children (CSR) and parents
-    L.parent = parent;
-    // (outside the tail; the tail's columns wait for its frontier, the columns
-    // outside it whose parent is in it, listed after the children)
-    L.cptr.assign(n + 1, 0);
-    for (int j = 0; j < n; ++j)
-        if (parent[j] >= 0 && parent[j] < T0) L.cptr[parent[j] + 1]++;
-    for (int j = 0; j < n; ++j) L.cptr[j + 1] += L.cptr[j];
-    L.cidx.assign(L.cptr[n], 0);
-    {
-        std::vector<int> cf(L.cptr.begin(), L.cptr.end() - 1);
-        for (int j = 0; j < n; ++j)
-            if (parent[j] >= 0 && parent[j] < T0) L.cidx[cf[parent[j]]++] = j;
-    }
-    L.fr0 = (int)L.cidx.size();
-    for (int j = 0; j < T0; ++j)
-        if (parent[j] >= T0) L.cidx.push_back(j);
-    L.fr1 = (int)L.cidx.size();
-    if (L.cidx.empty()) L.cidx.push_back(0);
-    // the backward solve's columns outside the tail from the highest level down
-    L.bcols.reserve(n);
-    for (int h = L.H - 1; h >= 0; --h)
-        for (int t = L.lvl_ptr[h]; t < L.lvl_ptr[h + 1]; ++t)
-            if (L.lvl_col[t] < T0) L.bcols.push_back(L.lvl_col[t]);
-    // every entry of J_r (CSC order) to its factor slot: 4 slot + {0: L, 1: U, 2: diagonal}
+    // the sources of every element, by counting: A's entries and F first, then
+    // the children's updates in order
     const int nnzA = colptr[n];
-    L.amap.assign(nnzA, 0);
-    const auto &pos = slot_of;
+    std::vector<int> aplace(nnzA);
+    auto each = [&](auto &&take) {   // take(element, source)
+        for (int p = 0; p < nnzA; ++p) take(aplace[p], ~p);
+        for (int s = 0; s < nf; ++s) {
+            const MfFront &f = L.fr[s];
+            const int w = f.f + 1;
+            for (int i = 0; i < f.p; ++i) take(f.s0 + i * w + f.f, ~(nnzA + L.perm[f.e0 + i]));
+            for (int c : kids[s]) {
+                const MfFront &q = L.fr[c];
+                const int r = q.f - q.p, *rl = rel.data() + q.b0;
+                for (int i = 0; i < r; ++i) {
+                    const int row = f.s0 + rl[i] * w, cb = q.c0 + i * (r + 1);
+                    for (int j = 0; j < r; ++j) take(row + rl[j], cb + j);
+                    take(row + f.f, cb + r);
+                }
+            }
+        }
+    };
     for (int c = 0; c < n; ++c)
         for (int p = colptr[c]; p < colptr[c + 1]; ++p) {
-            const int i = iperm[rowidx[p]], j = iperm[c];
-            if (i == j)
-                L.amap[p] = 4 * j + 2;
-            else if (i > j)
-                L.amap[p] = 4 * pos(j, i) + 0;
-            else
-                L.amap[p] = 4 * pos(i, j) + 1;
+            const int i = iperm[rowidx[p]], j = iperm[c], s = sn[std::min(i, j)];
+            aplace[p] = L.fr[s].s0 + place(s, i) * (L.fr[s].f + 1) + place(s, j);
         }
+    if (nnzA + n >= INT32_MAX / 2) return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: system too large");
+    L.el.assign(std::max<long long>(s0, 1), make_int2(kMfNone, -1));
+    std::vector<int> more(std::max<long long>(s0, 1), -1);   // further sources of an element, then how many are placed
+    each([&](int e, int) { more[e]++; });
+    long long next = 0;
+    for (long long e = 0; e < s0; ++e)
+        if (more[e] > 0) {
+            L.el[e].y = (int)next;
+            next += 1 + more[e] / 4;
+        }
+    if (next >= INT32_MAX / 4) return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: factor too large");
+    L.ext.assign(std::max<long long>(next, 1), make_int4(0, 0, 0, 0));
+    each([&](int e, int k) {
+        if (L.el[e].x == kMfNone) {
+            L.el[e].x = k;
+            return;
+        }
+        int *rec = &L.ext[L.el[e].y].x;   // the count, then the sources
+        rec[1 + rec[0]++] = k;
+    });
+    std::vector<int> need(nf, 0);
+    std::vector<double> rem(nf, 0.0), down(nf, 0.0);
+    plan_classes(L.fr);
+    for (int s = 0; s < nf; ++s)
+        for (int c : kids[s]) need[s] += L.fr[c].cls == L.fr[s].cls;
+    // the longest remaining path to the root and down to a leaf, in rough us
+    for (int s = nf - 1; s >= 0; --s) {
+        const MfFront &f = L.fr[s];
+        double fl = 0.0;
+        for (int k = 0; k < f.p; ++k) fl += (double)(f.f - k) * (f.f - k);
+        rem[s] = 3.0 + 0.2 * f.p + fl / 3500.0 + (f.parent >= 0 ? rem[f.parent] : 0.0);
+    }
+    for (int s = 0; s < nf; ++s) {
+        down[s] += 1.0 + 0.05 * L.fr[s].p;
+        if (L.fr[s].parent >= 0) down[L.fr[s].parent] = std::max(down[L.fr[s].parent], down[s]);
+    }
+    // backward paths: the small fronts with small subtrees a warp each, the others
+    // a CTA each (a path goes on with the child that reaches furthest down among
+    // those of its launch), and the order of the leaves and heads
+    std::vector<char> cont(nf, 0), large(nf, 0);
+    for (int s = 0; s < nf; ++s) {
+        large[s] = L.fr[s].f > kMfSmall;
+        for (int c : kids[s]) large[s] |= large[c];
+    }
+    for (int s = 0; s < nf; ++s) {
+        MfFront &f = L.fr[s];
+        f.parent_need = f.parent >= 0 && L.fr[f.parent].cls == f.cls ? need[f.parent] : 0;
+        f.heavy = -1;
+        for (int c : kids[s])
+            if (large[c] == large[s] && (f.heavy < 0 || down[c] > down[f.heavy])) f.heavy = c;
+        f.light = f.wait = 0;
+        f.m0 = -1;
+        if (f.heavy >= 0) cont[f.heavy] = 1;
+        if (large[s]) L.bigp = std::max(L.bigp, f.p), L.backmax = std::max(L.backmax, f.f);
+        if (need[s] == 0) L.leaf[f.cls].push_back(s);
+    }
+    for (int s = 0; s < nf; ++s) {
+        MfFront &f = L.fr[s];
+        if (cont[s]) continue;
+        L.path[large[s]].push_back(s);
+        if (f.parent >= 0 && large[f.parent] == large[s]) {
+            f.wait = 1;
+            L.fr[f.parent].light = 1;
+        }
+    }
+    auto by = [](const std::vector<double> &key) {
+        return [&key](int x, int y) { return key[x] > key[y]; };
+    };
+    for (auto &v : L.leaf) std::stable_sort(v.begin(), v.end(), by(rem));
+    // (a parent reaches further down than its children: parents' paths come first)
+    for (auto &v : L.path) std::stable_sort(v.begin(), v.end(), by(down));
     return PF_OK;
+}
+
+// shared memory of the backward solve
+static size_t back_smem(int fmax, int pmax)
+{
+    const size_t p = (size_t)std::min(pmax, kMfBackRows);
+    return sizeof(double) * (2 * (size_t)fmax + p * (p | 1));
 }
 
 // Upload the plan of the grid's current bus types and size its workspace.
@@ -862,144 +1228,121 @@ pf_status lu_prepare(Grid *g, cudaStream_t s)
 {
     if (g->lu_ready) return PF_OK;
     HostLu L;
-    // the warps of one CTA per SM: an upper bound of the launch's warps
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return cuda_error(cudaGetLastError(), "jac_reduced_solve: device attributes");
-    if (pf_status st = host_lu(g->nb, g->red_n, g->red_npvpq, g->red_h_colptr, g->red_h_rowidx, g->red_h_fmap,
-                               std::max(1, nsm) * (kLuThreads / 32), L))
+    if (pf_status st = host_lu(g->nb, g->red_n, g->red_npvpq, g->red_h_colptr, g->red_h_rowidx, g->red_h_fmap, L))
         return st;
-    const size_t nnzL = (size_t)L.Lp[L.n];
-    auto up = [&](int **dst, const std::vector<int> &v) -> cudaError_t {
-        cudaError_t e = g->arena.alloc(dst, std::max<size_t>(v.size(), 1));
-        if (e == cudaSuccess && !v.empty())
-            e = cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice, s);
-        return e;
+    size_t nmat = 0;
+    for (MfFront &f : L.fr)
+        if (f.cls == 3) {
+            f.m0 = (long long)nmat;
+            nmat += (size_t)f.f * ((f.f + 1) | 1);
+        }
+    if (back_smem(L.backmax, L.bigp) > kMfMaxSmem)
+        return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: a front of %d unknowns exceeds shared memory", L.backmax);
+    const int nf = (int)L.fr.size();
+    cudaError_t e = cudaSuccess;
+    auto up = [&](auto **dst, const auto &v) -> cudaError_t {
+        cudaError_t r = g->arena.alloc(dst, std::max<size_t>(v.size(), 1));
+        if (r == cudaSuccess && !v.empty())
+            r = cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, s);
+        return r;
     };
-    cudaError_t e;
-    if ((e = up(&g->lu_Lp, L.Lp)) || (e = up(&g->lu_Li, L.Li)) || (e = up(&g->lu_Rp, L.Rp)) ||
-        (e = up(&g->lu_Rk, L.Rk)) || (e = up(&g->lu_Rq, L.Rq)) || (e = up(&g->lu_lvl_ptr, L.lvl_ptr)) ||
-        (e = up(&g->lu_lvl_col, L.lvl_col)) || (e = up(&g->lu_perm, L.perm)) || (e = up(&g->lu_amap, L.amap)) ||
-        (e = up(&g->lu_gptr, L.gptr)) || (e = up(&g->lu_need, L.need)) || (e = up(&g->lu_cptr, L.cptr)) ||
-        (e = up(&g->lu_cidx, L.cidx)) || (e = up(&g->lu_parent, L.parent)) || (e = up(&g->lu_bcols, L.bcols)) ||
-        (e = g->arena.alloc(&g->lu_done, 2 * (size_t)L.n + 2)) ||
-        (e = g->arena.alloc(&g->lu_fitems, std::max<size_t>(L.fitems.size(), 1))) ||
-        (!L.fitems.empty() && (e = cudaMemcpyAsync(g->lu_fitems, L.fitems.data(), L.fitems.size() * sizeof(int2),
-                                                   cudaMemcpyHostToDevice, s))) ||
-        (e = g->arena.alloc(&g->lu_gsrc, std::max<size_t>(L.gsrc.size(), 1))) ||
-        (!L.gsrc.empty() && (e = cudaMemcpyAsync(g->lu_gsrc, L.gsrc.data(), L.gsrc.size() * sizeof(int2),
-                                                 cudaMemcpyHostToDevice, s))) ||
-        (e = g->arena.alloc(&g->lu_Lx, std::max<size_t>(nnzL, 1))) ||
-        (e = g->arena.alloc(&g->lu_Ux, std::max<size_t>(nnzL, 1))) ||
-        (e = g->arena.alloc(&g->lu_D, std::max(2 * L.n, 1))) || (e = g->arena.alloc(&g->lu_y, std::max(L.n, 1))) ||
-        (e = cudaStreamSynchronize(s)))
+    if ((e = up(&g->lu_fr, L.fr)) || (e = up(&g->lu_leaf[0], L.leaf[0])) || (e = up(&g->lu_leaf[1], L.leaf[1])) ||
+        (e = up(&g->lu_leaf[2], L.leaf[2])) || (e = up(&g->lu_leaf[3], L.leaf[3])) || (e = up(&g->lu_path[0], L.path[0])) ||
+        (e = up(&g->lu_path[1], L.path[1])) || (e = up(&g->lu_el, L.el)) || (e = up(&g->lu_ext, L.ext)) ||
+        (e = up(&g->lu_bidx, L.bidx)) || (e = up(&g->lu_perm, L.perm)) ||
+        (e = g->arena.alloc(&g->lu_U, (size_t)std::max<long long>(L.nU, 1))) ||
+        (e = g->arena.alloc(&g->lu_cb, (size_t)std::max<long long>(L.nC, 1))) ||
+        (e = g->arena.alloc(&g->lu_x, (size_t)std::max(L.n, 1))) ||
+        (e = g->arena.alloc(&g->lu_mat, std::max<size_t>(nmat, 1))) ||
+        (e = g->arena.alloc(&g->lu_cnt, 2 * (size_t)nf + kMfClasses + 2)) || (e = cudaStreamSynchronize(s))) {
+        lu_release(g);
         return cuda_error(e, "jac_reduced_solve: set-up");
+    }
     g->lu_n = L.n;
-    g->lu_H = L.H;
-    g->lu_chain = L.chain;
-    g->lu_nfitems = (int)L.fitems.size();
-    g->lu_nbcols = (int)L.bcols.size();
-    g->lu_T0 = L.T0;
-    g->lu_LpT0 = L.Lp[L.T0];
-    g->lu_fr0 = L.fr0;
-    g->lu_fr1 = L.fr1;
-    g->lu_widest = 1;
-    for (int h = 0; h < L.H; ++h) g->lu_widest = std::max(g->lu_widest, L.lvl_ptr[h + 1] - L.lvl_ptr[h]);
-    g->lu_nnzL = (long long)nnzL;
+    g->lu_nf = nf;
+    for (int c = 0; c < kMfClasses; ++c) g->lu_nleaf[c] = (int)L.leaf[c].size();
+    for (int c = 0; c < 2; ++c) g->lu_npath[c] = (int)L.path[c].size();
+    g->lu_backmax = L.backmax;
+    g->lu_bigp = L.bigp;
     g->lu_ready = 1;
     return PF_OK;
 }
 
 void lu_release(Grid *g)
 {
-    for (void *p : {(void *)g->lu_Lp, (void *)g->lu_Li, (void *)g->lu_Rp, (void *)g->lu_Rk, (void *)g->lu_Rq,
-                    (void *)g->lu_lvl_ptr, (void *)g->lu_lvl_col, (void *)g->lu_perm, (void *)g->lu_amap,
-                    (void *)g->lu_Lx, (void *)g->lu_Ux, (void *)g->lu_D, (void *)g->lu_y, (void *)g->lu_gptr,
-                    (void *)g->lu_gsrc, (void *)g->lu_need, (void *)g->lu_cptr, (void *)g->lu_cidx,
-                    (void *)g->lu_parent, (void *)g->lu_bcols, (void *)g->lu_done, (void *)g->lu_fitems})
+    for (void *p : {(void *)g->lu_fr, (void *)g->lu_leaf[0], (void *)g->lu_leaf[1], (void *)g->lu_leaf[2], (void *)g->lu_leaf[3],
+                    (void *)g->lu_path[0], (void *)g->lu_path[1], (void *)g->lu_el, (void *)g->lu_ext,
+                    (void *)g->lu_bidx, (void *)g->lu_perm, (void *)g->lu_U, (void *)g->lu_cb, (void *)g->lu_x,
+                    (void *)g->lu_mat, (void *)g->lu_cnt})
         g->arena.release(p);
-    g->lu_Lp = g->lu_Li = g->lu_Rp = g->lu_Rk = g->lu_Rq = g->lu_lvl_ptr = g->lu_lvl_col = g->lu_perm = g->lu_amap =
-        g->lu_gptr = nullptr;
-    g->lu_need = g->lu_cptr = g->lu_cidx = g->lu_parent = g->lu_bcols = g->lu_done = nullptr;
-    g->lu_gsrc = g->lu_fitems = nullptr;
-    g->lu_Lx = g->lu_Ux = g->lu_D = g->lu_y = nullptr;
+    g->lu_fr = nullptr;
+    for (int *&p : g->lu_leaf) p = nullptr;
+    for (int *&p : g->lu_path) p = nullptr;
+    g->lu_el = nullptr;
+    g->lu_ext = nullptr;
+    g->lu_bidx = g->lu_perm = g->lu_cnt = nullptr;
+    g->lu_U = g->lu_cb = g->lu_x = g->lu_mat = nullptr;
     g->lu_ready = 0;
 }
 
 cudaError_t launch_lu_solve(Grid *g, const double *Jr, const double *F, double *dx, cudaStream_t s)
 {
     if (g->lu_n == 0) return cudaSuccess;
-    LuArgs a{};
+    MfArgs a{};
     a.n = g->lu_n;
+    a.nf = g->lu_nf;
     a.nnzA = (int)g->red_nnz;
-    a.nfitems = g->lu_nfitems;
-    a.nbcols = g->lu_nbcols;
-    a.T0 = g->lu_T0;
-    a.LpT0 = g->lu_LpT0;
-    a.fr0 = g->lu_fr0;
-    a.fr1 = g->lu_fr1;
-    a.Lp = g->lu_Lp;
-    a.Li = g->lu_Li;
-    a.Rp = g->lu_Rp;
-    a.Rk = g->lu_Rk;
-    a.Rq = g->lu_Rq;
+    a.backmax = g->lu_backmax;
+    for (int c = 0; c < kMfClasses; ++c) {
+        a.nleaf[c] = g->lu_nleaf[c];
+        a.leaf[c] = g->lu_leaf[c];
+    }
+    for (int c = 0; c < 2; ++c) {
+        a.npath[c] = g->lu_npath[c];
+        a.path[c] = g->lu_path[c];
+    }
+    a.fr = g->lu_fr;
+    a.el = g->lu_el;
+    a.ext = g->lu_ext;
+    a.bidx = g->lu_bidx;
     a.perm = g->lu_perm;
-    a.amap = g->lu_amap;
-    a.gptr = g->lu_gptr;
-    a.gsrc = g->lu_gsrc;
-    a.need = g->lu_need;
-    a.cptr = g->lu_cptr;
-    a.cidx = g->lu_cidx;
-    a.parent = g->lu_parent;
-    a.bcols = g->lu_bcols;
-    a.fitems = g->lu_fitems;
-    a.done = g->lu_done;
     a.A = Jr;
     a.F = F;
-    a.Lx = g->lu_Lx;
-    a.Ux = g->lu_Ux;
-    a.D = g->lu_D;
-    a.piv = g->lu_D + g->lu_n;
-    a.y = g->lu_y;
+    a.U = g->lu_U;
+    a.cb = g->lu_cb;
+    a.x = g->lu_x;
     a.dx = dx;
-    a.bar = g->bar;
+    a.mat = g->lu_mat;
+    a.cnt = g->lu_cnt;
     a.err = g->err;
-    if (g->lu_resident == 0) {
-        int per_sm = 0, dev = 0, nsm = 0;
-        cudaError_t e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lu_solve, kLuThreads, 0)) ||
-            (e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)))
+    cudaError_t e;
+    if (g->nsm == 0) {
+        int dev = 0;
+        if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&g->nsm, cudaDevAttrMultiProcessorCount, dev)))
             return e;
-        // one CTA per SM at most: the widest levels have a few thousand columns,
-        // and more CTAs make every grid barrier dearer
-        g->lu_resident = std::max(1, std::min(per_sm, 1) * nsm);
     }
-    // a warp per column of the widest level (the leaves) at most
-    const int ctas = std::max(1, (g->lu_widest + kLuThreads / 32 - 1) / (kLuThreads / 32));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::max(1, std::min(g->lu_resident, ctas)));
-    cfg.blockDim = dim3(kLuThreads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (a.T0 >= a.n) {   // no tail: one launch
-        a.mode = 0;
-        return cudaLaunchKernelEx(&cfg, k_lu_solve, a);
-    }
-    // the factorization outside the tail and the tail's outside terms; the
-    // tail by one cluster; the backward solve outside the tail
-    a.mode = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_lu_solve, a);
-    if (e != cudaSuccess) return e;
-    const size_t tsm = lu_tail_smem(a.n - a.T0);
-    if ((e = ensure_dyn_smem(reinterpret_cast<const void *>(k_lu_tail), tsm))) return e;
-    k_lu_tail<<<kLuTailCtas, kLuTailThreads, tsm, s>>>(a);
-    if ((e = cudaGetLastError())) return e;
-    a.mode = 2;
-    return cudaLaunchKernelEx(&cfg, k_lu_solve, a);
+    const size_t sm_small = sizeof(double) * kMfSmallWarps * kMfSmall * kMfSmallLd;
+    const size_t sm_bsmall = sizeof(double) * kMfSmallWarps * (kMfSmall * kMfSmall + kMfSmall);
+    const size_t sm_wide = sizeof(double) * (kMfWide + 1) + kMfWideRowBytes;
+    const size_t sm_bbig = back_smem(g->lu_backmax, g->lu_bigp);
+    if ((e = ensure_dyn_smem(reinterpret_cast<const void *>(k_mf_wide), sm_wide)) ||
+        (e = ensure_dyn_smem(reinterpret_cast<const void *>(k_mf_back_big), sm_bbig)))
+        return e;
+    // arrivals, written marks and item counters
+    if ((e = cudaMemsetAsync(a.cnt, 0, (2 * (size_t)a.nf + kMfClasses + 2) * sizeof(int), s))) return e;
+    auto ctas = [&](int items, int per_cta, int per_sm) {
+        return std::max(1, std::min(per_sm * g->nsm, (items + per_cta - 1) / per_cta));
+    };
+    if (a.nleaf[0] > 0)
+        k_mf_small<<<ctas(a.nleaf[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_small, s>>>(a);
+    if (a.nleaf[1] > 0) k_mf_mid<<<ctas(a.nleaf[1], 1, 6), 32 * kMfMidWarps, 0, s>>>(a);
+    if (a.nleaf[2] > 0)
+        k_mf_wide<<<kMfWideCtas * std::min(a.nleaf[2], std::max(1, g->nsm / kMfWideCtas)), 32 * kMfWideWarps, sm_wide, s>>>(a);
+    if (a.nleaf[3] > 0) k_mf_huge<<<ctas(a.nleaf[3], 1, 1), kMfHugeThreads, 0, s>>>(a);
+    if (a.npath[1] > 0) k_mf_back_big<<<ctas(a.npath[1], 1, 2), kMfBackThreads, sm_bbig, s>>>(a);
+    if (a.npath[0] > 0)
+        k_mf_back_small<<<ctas(a.npath[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_bsmall, s>>>(a);
+    return cudaGetLastError();
 }
 
 }  // namespace pf

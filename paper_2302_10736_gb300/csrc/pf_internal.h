@@ -227,6 +227,18 @@ struct EwDev {
     int2 *tloc = nullptr;     // [T] {phasor slot of the other bus, slot position | flags}
 };
 
+// A front of the multifrontal LU (lu.cu): p pivots e0 .. e0 + p - 1 and f - p
+// border unknowns (bidx[b0 ...]), both in elimination numbers
+constexpr int kMfClasses = 4;   // by who eliminates it (lu.cu)
+struct alignas(16) MfFront {
+    int p, f, e0, parent;              // parent: its front (-1: a root)
+    int s0, u0, c0, b0;                // its elements' sources, pivot rows and y, update, border
+    int parent_need, cls, heavy, light;   // children of its class the parent waits for (0: other class); class; the
+                                       // child its backward path goes on with; other paths wait for it
+    int wait, pad[3];                  // heads a path whose parent is written in the same launch
+    long long m0, pad2;                // place in global memory (the last class)
+};
+
 struct Grid {
     int nb = 0, nl = 0, nnz = 0;
     pf_config cfg{};
@@ -304,19 +316,16 @@ struct Grid {
     // Newton-Raphson workspace (powerflow_newton): F, J_r (CSC), step, max |F|
     double *nt_F = nullptr, *nt_J = nullptr, *nt_dx = nullptr;
     unsigned long long *nt_max = nullptr;
-    // sparse LU of the reduced system (lu.cu): plan of the current bus types
-    // (CSC of L's pattern, row structures, levels, permutation, value map) and
-    // the factor storage
-    int lu_ready = 0, lu_n = 0, lu_H = 0, lu_chain = 0, lu_resident = 0, lu_widest = 0;
-    long long lu_nnzL = 0;
-    int *lu_Lp = nullptr, *lu_Li = nullptr, *lu_Rp = nullptr, *lu_Rk = nullptr, *lu_Rq = nullptr;
-    int *lu_lvl_ptr = nullptr, *lu_lvl_col = nullptr, *lu_perm = nullptr, *lu_amap = nullptr, *lu_gptr = nullptr;
-    int *lu_need = nullptr, *lu_cptr = nullptr, *lu_cidx = nullptr, *lu_parent = nullptr, *lu_bcols = nullptr;
-    int *lu_done = nullptr;   // [2n + 1] per column: finished factorization items, backward solve done; the item counter
-    int lu_nfitems = 0, lu_nbcols = 0, lu_T0 = 0, lu_LpT0 = 0;   // items; the tail's first column and slot
-    int lu_fr0 = 0, lu_fr1 = 0;                                  // the tail's frontier in lu_cidx
-    int2 *lu_gsrc = nullptr, *lu_fitems = nullptr;
-    double *lu_Lx = nullptr, *lu_Ux = nullptr, *lu_D = nullptr, *lu_y = nullptr;
+    // sparse LU of the reduced system (lu.cu): the plan of the current bus types
+    // (HostLu), its pivot rows, updates, solution and counters
+    int lu_ready = 0, lu_n = 0, lu_nf = 0, lu_backmax = 0, lu_bigp = 0;
+    int lu_nleaf[kMfClasses] = {}, lu_npath[2] = {};
+    MfFront *lu_fr = nullptr;
+    int *lu_leaf[kMfClasses] = {}, *lu_path[2] = {};
+    int2 *lu_el = nullptr;
+    int4 *lu_ext = nullptr;
+    int *lu_bidx = nullptr, *lu_perm = nullptr, *lu_cnt = nullptr;
+    double *lu_U = nullptr, *lu_cb = nullptr, *lu_x = nullptr, *lu_mat = nullptr;
     // tracer: events [2 * capacity], kernel id per record
     std::vector<cudaEvent_t> tr_ev;
     std::vector<int> tr_kernel;
@@ -395,27 +404,18 @@ cudaError_t launch_reduce(Grid *g, const int *map, const double *Pspec, const do
                           cudaStream_t s);
 
 // sparse LU of the reduced system (lu.cu): the host analysis of a reduced
-// pattern (permutation new -> reduced index, CSC of L's pattern, per column the
-// (k, position of L(j, k)) pairs of its row, columns by tree height, the top
-// levels narrow enough for one CTA from `chain` on, and each reduced entry's
-// factor slot 4 slot + {0 L, 1 U, 2 diagonal}), its upload, and the solve
+// pattern, its upload, and the solve
 struct HostLu {
-    int n = 0, H = 0, chain = 0;
-    int T0 = 0;             // the tail (columns T0 .. n-1) factored as a dense block; n: none
-    int fr0 = 0, fr1 = 0;   // the tail's frontier (the columns outside it whose parent is in it) in cidx
-    std::vector<int> perm, Lp, Li, Rp, Rk, Rq, lvl_ptr, lvl_col, amap;
-    std::vector<int> gptr;    // [nnzL + 1] update terms of every factor slot
-    std::vector<int2> gsrc;   // {slot of L(i, k), slot of L(j, k)}, k ascending per slot
-    // dependency-driven schedule: the factorization's work items in level order
-    // ({column, -2}: the whole column by one warp; {column, slot or -1}: one slot
-    // of a column of the narrow top), the items of every column, the columns'
-    // children in the elimination tree (CSR) and parents, and the columns of the
-    // backward solve from the root down
-    std::vector<int2> fitems;
-    std::vector<int> need, cptr, cidx, parent, bcols;
+    int n = 0, backmax = 0, bigp = 0;
+    long long nU = 0, nC = 0;
+    std::vector<MfFront> fr;
+    std::vector<int> perm, bidx;
+    std::vector<int2> el;
+    std::vector<int4> ext;
+    std::vector<int> leaf[kMfClasses], path[2];
 };
 pf_status host_lu(int nb, int n, int npvpq, const std::vector<int> &colptr, const std::vector<int> &rowidx,
-                  const std::vector<int> &fmap, int slot_warps, HostLu &L);
+                  const std::vector<int> &fmap, HostLu &L);
 pf_status lu_prepare(Grid *g, cudaStream_t s);
 void lu_release(Grid *g);
 cudaError_t launch_lu_solve(Grid *g, const double *Jr, const double *F, double *dx, cudaStream_t s);
