@@ -606,19 +606,15 @@ pf_status jac_target(pf_grid *grid, int32_t method, const double *vm, const doub
  * Solve J_r dx = F for the reduced Newton system of the grid's bus types
  * (the step the paper hands to a sparse direct solver, KLU): Jr [nnz] holds
  * the reduced Jacobian's values in jac_reduced's CSC order, F [n] the right-hand
- * side, dx [n] receives the solution (device pointers).  Sparse LU without
- * pivoting on a fill-reducing order: the first call after grid_set_bus_types
- * analyses the pattern on the host (minimum-degree order of the buses,
- * symbolic factorization, the dependency schedule of the elimination tree),
- * allocates the factor storage and synchronizes; make it before any stream
- * capture.  Every later call is asynchronous: a cooperative launch for the
- * numeric factorization with the forward solve, each column started when the
- * columns it depends on are done (bounded waits); where the top of the
- * elimination tree is a run of at least 16 narrow levels, a launch of one
- * 8-CTA thread-block cluster for it (a dense block in shared memory, both
- * triangular solves), then a cooperative launch for the backward solve below
- * it (otherwise the backward solve ends the first launch).  Bitwise
- * repeatable.  A zero
+ * side, dx [n] receives the solution (device pointers).  Multifrontal sparse LU
+ * without pivoting on a fill-reducing order: the first call after
+ * grid_set_bus_types analyses the pattern on the host (minimum-degree order of
+ * the buses, symbolic factorization, fronts), allocates the factor storage and
+ * synchronizes; make it before any stream capture.  Every later call is
+ * asynchronous: a memset of the counters and up to six plain launches (fronts
+ * eliminated by a warp, a CTA, a cluster of 8 CTAs, or a CTA in global memory,
+ * the forward solve with them; then the backward solve, by CTAs and by warps),
+ * fewer where a size does not occur.  Bitwise repeatable.  A zero
  * or non-finite pivot sets the grid's device error word (grid_check_error
  * reports PF_EDEVICE), a wait that runs out (2 s) sets it to a time-out
  * (grid_check_error reports PF_ETIMEOUT and clears it); no pivoting

@@ -24,22 +24,35 @@
 //     l_i = m_ik / m_kk,   m_ij -= l_i m_kj     (k < p; i, j > k, y with it)
 // Backward, x_p = U_pp^-1 (y - U_pr x_r) from the root down.
 //
-// What bounds it.  The arithmetic is small (1.3 M FMAs at 10,000 buses, 2.5 us
-// of the GPU's FP64 rate); the solve is the latency of the tree's longest path,
-// so it is built around few, cheap dependent steps.  Fronts halve the levels
-// against columns twice over (197 column levels are 22 front levels at 10,000
-// buses), a front's work stays in one warp's or CTA's shared memory, and its
-// only global round trips are its children's updates in and its own out.  A
-// warp that finishes a front counts itself at the parent, and the last child to
-// arrive goes on with the parent (no polling, no schedule).  A warp-wide FP64
-// instruction occupies the SM's FP64 pipe for about 19 cycles whatever its
-// active lanes, so loops are flattened over a front's elements and what is
-// uniform (a pivot's reciprocal) is formed by one warp.
-//   k_mf_small: fronts of at most kMfSmall unknowns with such subtrees, a warp each.
-//   k_mf_big:   the rest (the top of the tree), a CTA each.
-//   k_mf_back_big, k_mf_back_small: the backward solve; a CTA or warp follows
-//     one heavy path of the tree down and waits (bounded) only at its head.
-// One solve, start of this form -> now, back to back: see launch_lu_solve.
+// What bounds it.  The arithmetic is small (5.5 M FMAs at 25,000 buses, 10 us of
+// the GPU's FP64 rate); the solve is the latency of the tree's longest path, so it
+// is built around few, cheap dependent steps:
+//   * Fronts instead of columns: 105 levels of buses are 22 of fronts at 10,000
+//     buses, and a front's only global round trips are its children's updates in
+//     and its own out.
+//   * No schedule and no polling on the way up: a warp, CTA or cluster that
+//     finishes a front counts itself at the parent, and the last child to arrive
+//     goes on with the parent.
+//   * A sub-partition's FP64 unit takes a warp instruction in 64 cycles, whatever
+//     its active lanes and however independent the next one (measured: 64.1
+//     cycles per FMA for 1 to 64 threads of an SM, dependent or 8 chains; 76 with
+//     all four sub-partitions busy).  So a row of a front lies across a whole
+//     warp, rows go round the sub-partitions and, for large fronts, the SMs of a
+//     cluster, and nothing uniform is computed more than once: pivot rows are
+//     scaled by the reciprocal (unit-diagonal U), so that multipliers and the
+//     backward solve need no FP64 operation of their own.
+// The kernels, by the size of a front (plan_classes): k_mf_small, a warp per front
+// in shared memory; k_mf_mid, a CTA, and k_mf_wide, a cluster of 8 CTAs, with the
+// front in registers; k_mf_huge, a CTA in global memory.  k_mf_back_big,
+// k_mf_back_small: the backward solve; a CTA or warp follows one heavy path of the
+// tree down and waits (bounded) only at its head.
+//
+// One solve (CUDA-profiled kernels, us): 2,000 buses 378 -> 172, 10,000 962 -> 350,
+// 25,000 1,752 -> 560, 70,000 3,111 -> 937, against a left-looking factorization
+// by columns whose every level cost a chain of L2 round trips, with the top of the
+// tree as one dense block of a cluster and an FP64 reciprocal in each of its warps.
+// Of the 560 us at 25,000 buses, small 34, mid 88, wide 295 (0.75 us per pivot row
+// of the top ten fronts), backward 130.
 //
 // Every sum has a fixed order (children in order of their pivots, lane-strided
 // partial sums joined by a fixed shuffle tree): the results are bitwise

@@ -5,7 +5,7 @@
 // loop on the GPU.  Iteration k: the mismatch F and the reduced Jacobian J_r
 // in CSC order (jac_reduced: one launch by the element-wise method), max |F|
 // to the host (the only host round trip), then J_r dx = F by the library's
-// sparse LU (lu.cu, one cooperative launch) and x <- x - dx, with x the
+// sparse LU (lu.cu) and x <- x - dx, with x the
 // angles of the PV and PQ buses and the magnitudes of the PQ buses.
 #include <algorithm>
 #include <cstring>
