@@ -179,7 +179,6 @@ static pf_status upload_topology(Grid *g, cudaStream_t s)
     PF_CUDA(a.alloc(&g->tcfx, (size_t)T));
     PF_CUDA(a.alloc(&g->tce, (size_t)T));
     PF_CUDA(a.alloc(&g->br_aux, (size_t)g->nl));
-    PF_CUDA(a.alloc(&g->bus_ysh, (size_t)nb));
     PF_CUDA(a.alloc(&g->ph_u, (size_t)nb));
     PF_CUDA(a.alloc(&g->ph_v, (size_t)nb));
     PF_CUDA(a.alloc(&g->err, 1));
@@ -252,16 +251,7 @@ static pf_status build_ew_layout(Grid *g, int tb, cudaStream_t s)
 pf_status refresh_values(Grid *g, const double *gg, const double *gb, const double *gbsh, const double *gtap,
                          const double *gshift, const double *gs, const double *bs, cudaStream_t s)
 {
-    PF_CUDA(launch_branch_constants(g, gg, gb, gbsh, gtap, gshift, s));
-    PF_CUDA(launch_ybus_values(g, gs, bs, s));
-    const size_t bytes = (size_t)g->nl * sizeof(double);
-    if (bytes) {
-        PF_CUDA(cudaMemcpyAsync(g->p_g, gg, bytes, cudaMemcpyDeviceToDevice, s));
-        PF_CUDA(cudaMemcpyAsync(g->p_b, gb, bytes, cudaMemcpyDeviceToDevice, s));
-        PF_CUDA(cudaMemcpyAsync(g->p_bsh, gbsh, bytes, cudaMemcpyDeviceToDevice, s));
-        PF_CUDA(cudaMemcpyAsync(g->p_tap, gtap, bytes, cudaMemcpyDeviceToDevice, s));
-        PF_CUDA(cudaMemcpyAsync(g->p_shift, gshift, bytes, cudaMemcpyDeviceToDevice, s));
-    }
+    PF_CUDA(launch_params(g, gg, gb, gbsh, gtap, gshift, gs, bs, s));
     return PF_OK;
 }
 

@@ -276,7 +276,6 @@ struct Grid {
     int2 *tnbr = nullptr;                  // {other bus, kpos | EW_ACCUM}
     int *town = nullptr;                   // owner bus
     int *tpos = nullptr;                   // [2nl] sorted position of terminal t
-    double2 *bus_ysh = nullptr;            // [nb]
     double2 *bus_yd = nullptr;             // [nb] bus shunt + sum of the bus's terminal self constants
     EwDev ew;
     uint32_t ew_smem_jac = 0, ew_smem_inj = 0, ew_smem_host = 0, ew_smem_red = 0, yb_smem_jac = 0, yb_smem_inj = 0;   // dynamic shared memory the kernels are configured for
@@ -372,9 +371,8 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), int grid, int block, size_
 }
 
 // kernel launchers (k_*.cu); each returns the status of its launch(es)
-cudaError_t launch_branch_constants(Grid *g, const double *gg, const double *gb, const double *gbsh,
-                                    const double *gtap, const double *gshift, cudaStream_t s);
-cudaError_t launch_ybus_values(Grid *g, const double *gs, const double *bs, cudaStream_t s);
+cudaError_t launch_params(Grid *g, const double *gg, const double *gb, const double *gbsh, const double *gtap,
+                          const double *gshift, const double *gs, const double *bs, cudaStream_t s);
 cudaError_t ensure_trig_table();   // once per device, synchronous
 const ITrig *trig_table();         // device address of the (cos, sin) table of isincos.cuh
 cudaError_t launch_phasor(int nb, const double *vm, const double *va, double4_32a *U, double2 *V, cudaStream_t s);
