@@ -189,10 +189,25 @@ static pf_status upload_topology(Grid *g, cudaStream_t s)
     return PF_OK;
 }
 
+// How many windows to cut at equal estimated cost when the plain cut (as many
+// buses and terminals as a CTA's threads) gives n0; 0: the plain cut as it is.
+//   * All of it fits one CTA per SM: one per SM.  More, emptier CTAs only cost
+//     their launch, and leave the next evaluation of a stream no room to start:
+//     9,241 buses 4.42 us at 5 CTAs per SM, 3.92 at one; 2,736 buses 4.06 / 3.59;
+//     300 buses 3.35 / 3.13 (jac_elementwise, back to back).
+//   * More than that: the whole wave of CTAs that fit (25,000 buses: 5.13 us at
+//     760, 5.40 at 608, 7.12 at 304).
+//   * Several waves: nothing is gained by more windows, each with its ghost
+//     buses (410,000 buses 43.3 us in 4,256, 44.8 in six whole waves).
+static int ew_target_windows(int n0, int nsm, long long wave)
+{
+    if (n0 <= nsm) return nsm;
+    if (n0 > wave) return 0;
+    return (int)std::min<long long>(wave, INT32_MAX);
+}
+
 // Build (host), check and upload the element-wise windows for CTAs of `tb`
-// threads (at most tb buses and tb terminals per window).  The windows are cut
-// at equal estimated cost into a whole number of waves of the CTAs that fit
-// on the GPU at once, so that every SM gets the same work.
+// threads (at most tb buses and tb terminals per window).
 static pf_status ew_fits(const HostEw &E, size_t *smem)
 {
     const EwSmem plan = ew_smem_plan(E.max_nbus, E.max_nt, E.max_L, true, E.max_nph);
@@ -215,7 +230,8 @@ static pf_status build_ew_layout(Grid *g, int tb, cudaStream_t s)
     PF_CUDA(ew_blocks_per_sm(tb, smem, &per_sm));
     for (int pass = 0; pass < 2 && per_sm > 0 && E.nwin > 1; ++pass) {
         const long long wave = (long long)nsm * per_sm;
-        const int target = (int)std::min<long long>(wave * ((E.nwin + wave - 1) / wave), INT32_MAX);
+        const int target = ew_target_windows(E.nwin, nsm, wave);
+        if (target == 0) break;
         HostEw B;
         size_t smem_b = 0;
         if ((st = host_ew(g->topo, tb, B, 1, target)) || (st = ew_fits(B, &smem_b))) return st;
