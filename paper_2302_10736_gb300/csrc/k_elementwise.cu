@@ -216,8 +216,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
     extern __shared__ __align__(16) char smem[];
     const EwSmem sp = ew_smem_plan(a.max_nbus, a.max_nt, JAC ? a.max_L : 0, JAC, a.max_nph);
     int4 *sbm = reinterpret_cast<int4 *>(smem + sp.bm);
-    double2 *syd = reinterpret_cast<double2 *>(smem + sp.yd);
-    double2 *sSv = syd;   // the Jacobian kernels keep v^2 conj(Yd) where the others keep Yd
+    double2 *syd = reinterpret_cast<double2 *>(smem + sp.yd);   // Yd, or (Jacobian) v conj(Yd)
     double2 *skg = reinterpret_cast<double2 *>(smem + sp.kg);
     int *skp = reinterpret_cast<int *>(smem + sp.kp);
     double *jst = reinterpret_cast<double *>(smem + sp.jst);
@@ -225,7 +224,6 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
     longlong2 *sA = reinterpret_cast<longlong2 *>(smem + sp.ph);             // own buses: V in block floating point
     longlong2 *sU = sA + a.max_nph;                                          // 2^62 (cos, sin)
     double2 *sW = reinterpret_cast<double2 *>(sU + a.max_nph);               // (v, 1/v)
-    double2 *sW2 = reinterpret_cast<double2 *>(smem + sp.w2);               // own buses: (v^2, 2 v)
     int *sord = reinterpret_cast<int *>(smem + sp.ord);                     // reduction thread -> bus
     ITrig *tab = reinterpret_cast<ITrig *>(smem + sp.total);
     const int tid = threadIdx.x, TB = blockDim.x;
@@ -331,20 +329,14 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
             if (JAC) {
                 // 1/v is read for the window's own buses only: warps of ghost
                 // slots skip it (a warp-uniform branch), mixed warps form it
-                // for all lanes; and the parameter-and-magnitude terms of the
-                // reduction, 2 v conj(Yd) and v^2 conj(Yd), formed once per bus
-                // here (where the FP64 pipe is idle) instead of by both threads
-                // of its pair (slot j < nbus is bus j, whose Yd thread j holds)
+                // for all lanes; and v conj(Yd) of the reduction, formed once per
+                // bus here (where the FP64 pipe is idle) instead of by both
+                // threads of its pair (slot j < nbus is bus j, whose Yd thread j
+                // holds)
                 if (__any_sync(__activemask(), j < nbus)) {
                     iv = fast_rcp(v);
-                    if (j < nbus) {
-                        const double tv = fix_twice(v), v2 = v * v;
-                        sW2[j] = make_double2(__dmul_rn(tv, ydo.x), neg(__dmul_rn(tv, ydo.y)));   // 2 v conj(Yd)
-                        sSv[j] = make_double2(__dmul_rn(v2, ydo.x), neg(__dmul_rn(v2, ydo.y)));   // v^2 conj(Yd)
-                    }
+                    if (j < nbus) syd[j] = make_double2(v * ydo.x, neg(v * ydo.y));   // v conj(Yd)
                 }
-            } else if (j < nbus) {
-                sW2[j].x = v * v;
             }
             sW[j] = make_double2(v, iv);
         }
@@ -434,12 +426,12 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                         }
                     }
                 }
-                const double2 dv = sW2[b], sv = sSv[b];   // 2 v conj(Yd), v^2 conj(Yd)
-                const double iv = sW[b].y;
+                const double2 vy = syd[b], vw = sW[b];   // v conj(Yd); v, 1/v
+                const double vc = im ? vy.y : vy.x;
                 const int pos = bm.x + (YBUS ? bm.z & ~kYbusSlowRow : bm.z);
                 jst[(im ? 0 : L) + pos] = neg_if(sK, im);                  // Re / Im of j sum K
-                jst[(im ? L : 0) + pos + d] = fma(sK, iv, im ? dv.y : dv.x);   // 2 v conj(Yd) + sum K / v
-                spq[(im ? pqs : 0) + b + par] = sK + (im ? sv.y : sv.x);      // S = v^2 conj(Yd) + sum K
+                jst[(im ? L : 0) + pos + d] = fma(sK, vw.y, fix_twice(vc));   // 2 v conj(Yd) + sum K / v
+                spq[(im ? pqs : 0) + b + par] = fma(vw.x, vc, sK);            // S = v^2 conj(Yd) + sum K
                 if (YBUS) slow_row |= bm.z < 0;
             }
             if (YBUS && slow_row)
@@ -454,7 +446,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                     spq[(im ? pqs : 0) + b + par] = im ? r.S.y : r.S.x;
                 }
         } else {
-            // two threads per bus as above; v^2 from the phasor phase
+            // two threads per bus as above
             const double *k1 = reinterpret_cast<const double *>(skg);   // K.x, K.y per terminal
             for (int x = tid; x < 2 * nbus; x += TB) {
                 const int b = sord[x >> 1], im = x & 1;
@@ -465,8 +457,8 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 if (i < tend) sK = k1[2 * i++ + im];
                 for (; i < tend; ++i) sK += k1[2 * i + im];
                 const double2 y = syd[b];
-                const double v2 = sW2[b].x;
-                spq[(im ? pqs : 0) + b + par] = fma(v2, im ? neg(y.y) : y.x, sK);   // S = v^2 conj(Yd) + sum K
+                const double v = sW[b].x;
+                spq[(im ? pqs : 0) + b + par] = fma(v, v * (im ? neg(y.y) : y.x), sK);   // S = v^2 conj(Yd) + sum K
                 if (YBUS) slow_row |= bm.z < 0;
             }
             if (YBUS && slow_row)

@@ -150,18 +150,6 @@ __device__ __forceinline__ double warp_sum_d(double x)
     return x;
 }
 
-// 1 / v: the hardware's approximate reciprocal y, 1 / v = y (1 + e + e^2 + ...) with
-// e = 1 - v y exact to rounding and below 2^-19, so the series may stop at e^2:
-// three dependent FP64 operations (64 cycles each) where fast_rcp's two Newton
-// steps take four
-__device__ __forceinline__ double mf_rcp(double v)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    const double e = fma(-v, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
 __device__ __forceinline__ void pivot_check(const MfArgs &a, double d)
 {
     if (!(fabs(d) > 0.0) || !isfinite(d)) atomicExch(a.err, DEV_SINGULAR);
@@ -264,7 +252,7 @@ __device__ __forceinline__ void mf_small_front(const MfArgs &a, const MfFront &f
     }
     __syncwarp();
     for (int k = 0; k < p; ++k) {
-        const double dk = S[k * ld + k], inv = mf_rcp(dk);
+        const double dk = S[k * ld + k], inv = fast_rcp(dk);
         if (k + 1 + lane <= f) S[k * ld + k + 1 + lane] *= inv;
         if (lane == 31) pivot_check(a, dk);
         __syncwarp();
@@ -447,7 +435,7 @@ __device__ __forceinline__ void mf_publish(const MfArgs &a, const MfGroup<NC> &g
 {
     const int lane = threadIdx.x & 31;
     const double d = __shfl_sync(0xffffffffu, mr[C0], k & 31);
-    const double inv = mf_rcp(d);
+    const double inv = fast_rcp(d);
 #pragma unroll
     for (int c = C0; c < C2; ++c) mf_send<NC, C2>(g, slot, 32 * c + lane, mr[c] * inv);
     if (NC == 1) {
@@ -658,7 +646,7 @@ __device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr
     __syncthreads();
     for (int k = 0; k < p; ++k) {
         double *Mk = M + (size_t)k * ld;
-        const double d = Mk[k], inv = mf_rcp(d);
+        const double d = Mk[k], inv = fast_rcp(d);
         __syncthreads();
         for (int j = k + 1 + tid; j <= f; j += kMfHugeThreads) Mk[j] *= inv;
         if (tid == 0) pivot_check(a, d);

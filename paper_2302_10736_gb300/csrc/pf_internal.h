@@ -145,20 +145,19 @@ pf_status host_window_branches(const HostTopo &H, const HostEw &E, std::vector<i
 
 // Shared-memory plan of the element-wise kernels (byte offsets, 16-aligned):
 //   bm  int4    [max_nbus]   per bus {J-slice row offset, row length, diagonal position, first terminal}
-//   yd  double2 [max_nbus]   per bus self sum
+//   yd  double2 [max_nbus]   per bus self sum (the single evaluation's Jacobian: v conj of it)
 //   kg  double2 [2 max_nt]   per terminal K and G (injection kernel: K only)
 //   kp  int     [max_nt]     per terminal slot position | EW_ACCUM (Jacobian kernel)
 //   jst double  [2 max_L]    the window's J slice (P half, then Q half)
 //   pq  double  [2 pqs]      P then Q of the window, parity-aligned with global memory
 //   ph                       phasor table (below)
 //   ord int     [max_nbus]   the reduction's thread-to-bus map (HostEw::rorder)      (max_nph > 0)
-//   w2  double2 [max_nbus]   (v^2, 2 v) of the window's own buses                     (max_nph > 0)
 struct EwSmem {
-    uint32_t bm, yd, kg, kp, jst, pq, pqs, ph, ord, w2, total;
+    uint32_t bm, yd, kg, kp, jst, pq, pqs, ph, ord, total;
 };
 // max_nph > 0 (the single-evaluation kernel) adds a phasor table of that many
 // slots: V of the own buses in block floating point and 2^62 (cos, sin), each
-// a pair of 64-bit integers, and (v, 1/v), and the ord and w2 arrays
+// a pair of 64-bit integers, and (v, 1/v), and the ord array
 __host__ __device__ inline EwSmem ew_smem_plan(int max_nbus, int max_nt, int max_L, bool jac, int max_nph = 0)
 {
     EwSmem p;
@@ -171,8 +170,7 @@ __host__ __device__ inline EwSmem ew_smem_plan(int max_nbus, int max_nt, int max
     p.pq = p.jst + (jac ? 16u * (uint32_t)max_L : 0u);
     p.ph = p.pq + 16u * p.pqs;
     p.ord = p.ph + 48u * (uint32_t)max_nph;
-    p.w2 = p.ord + (max_nph > 0 ? (4u * (uint32_t)max_nbus + 15u) & ~15u : 0u);
-    p.total = p.w2 + (max_nph > 0 ? 16u * (uint32_t)max_nbus : 0u);
+    p.total = p.ord + (max_nph > 0 ? (4u * (uint32_t)max_nbus + 15u) & ~15u : 0u);
     return p;
 }
 constexpr uint32_t kMaxSmem = 227u * 1024u;
