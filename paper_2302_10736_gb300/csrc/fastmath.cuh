@@ -2,10 +2,9 @@
 // flips on the integer pipe (the GB300 FP64 pipe is the binding resource of
 // this library; the sine and cosine are in isincos.cuh).
 //
-// rcp: the hardware's approximate reciprocal y (about 20 correct bits) corrected
-// by the geometric series of e = 1 - v y up to e^2 (e^3 is below 2^-57): 3 FMAs,
-// where two Newton-Raphson steps take 4.  Zero or subnormal v is not supported
-// (flushed).
+// rcp: the hardware's approximate reciprocal refined by two Newton-Raphson
+// steps y <- y + y (1 - v y) (quadratic convergence from ~23 correct bits);
+// 4 FMAs.  Zero or subnormal v is not supported (flushed).
 #pragma once
 
 #include <cstdint>
@@ -28,8 +27,10 @@ __device__ __forceinline__ double fast_rcp(double v)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    const double e = fma(-v, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    double e = fma(-v, y, 1.0);
+    y = fma(y, e, y);
+    e = fma(-v, y, 1.0);
+    return fma(y, e, y);
 }
 
 }  // namespace pf

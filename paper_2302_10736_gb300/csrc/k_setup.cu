@@ -119,7 +119,7 @@ __device__ ITrig g_itrig_tab[kITrigCopies * kITrigN];
 // Phasor step (Sec. IV-B.1 step 1): U = e^{j theta} with v and 1/v (gathered
 // by the Jacobian kernels) and V = v U (gathered by the injection kernels and
 // by the element-wise Jacobian for the owner bus).  The sine and cosine run on
-// the integer pipe (isincos.cuh); 5 FP64 instructions per bus (fast_rcp 3 +
+// the integer pipe (isincos.cuh); 6 FP64 instructions per bus (fast_rcp 4 +
 // the hardware approximation, V 2).
 __global__ void __launch_bounds__(256) k_phasor(int nb, const double *__restrict__ vm,
                                                 const double *__restrict__ va, double4_32a *__restrict__ U,
