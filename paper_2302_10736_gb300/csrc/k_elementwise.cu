@@ -129,27 +129,27 @@ __device__ __forceinline__ void store_range(double *x, const double *s, int b0, 
 // An entry of a parallel run holds the run's sum (k_ybus_values writes the
 // values in terminal order, zero for the run's later terminals).  Rows with a
 // magnitude whose products or quotient might leave the range of normal
-// doubles, or with a non-finite angle of their own, take the sum of currents
-// in FP64 instead (ybus_row).
+// doubles, or with a non-finite angle, are evaluated whole from their current in
+// FP64 instead (ybus_row), after the others: one call, with little live around it
+// (calls among the evaluation's products and sums: 10.1 against 9.4 us at 70,000 buses).
 //
 // Why windows: with W lanes per CSR row and the sine and cosine per entry
 // (the earlier one-launch form) every bus was transformed 3.5 times and the
 // row's results left as scattered 8-byte stores; on windows it is 1.7 times,
 // and the results leave as bulk copies.  70,000 buses, Jacobian back to back:
-// 21.2 -> 9.9 us a call (k_ew: 9.1); 410,000: 98.9 -> 51.9; 25,000, injections,
-// on the device: 10.0 -> 6.0.
+// 21.2 -> 9.4 us a call (k_ew: 8.6); 410,000: 98.5 -> 45.2; 25,000, injections,
+// on the device: 9.9 -> 4.8.
 constexpr int kYbusSlowRow = (int)0x80000000;
 
 // a biased exponent within 2^-300 .. 2^300
 __device__ __forceinline__ bool ybus_mid(int e) { return (unsigned)(e - 723) <= 600u; }
 
-// Y_oq of the entry whose parallel run starts at sorted terminal p (zero for a
-// later terminal of a run), summed as k_ybus_values sums it
-__device__ __noinline__ double2 ybus_entry(const EwArgs &a, int p, int kpos)
+// Y_oq of the entry whose parallel run starts at sorted terminal p, summed as
+// k_ybus_values sums it
+__device__ __forceinline__ double2 ybus_entry(const EwArgs &a, int p)
 {
     double2 y = make_double2(0.0, 0.0);
-    if (kpos & EW_ACCUM) return y;
-    const int o = a.town[p], pe = a.tp[o + 1];
+    const int pe = a.tp[a.town[p] + 1];
     do {
         const double2 c = a.tcoup[p];
         y.x += c.x;
@@ -159,51 +159,61 @@ __device__ __noinline__ double2 ybus_entry(const EwArgs &a, int p, int kpos)
     return y;
 }
 
-struct YbusRow {
-    double2 S, dT, dV;   // S_o, dS_o/dtheta_o, dS_o/dv_o
-};
-
 // Row o by its current I_o (Eqs. 1, 3, 4) in FP64, in the order of operations of
-// a row kernel's lane (k_jac_ybus_b)
-__device__ __noinline__ YbusRow ybus_row(const EwArgs &a, int o)
+// a row kernel's lane (k_jac_ybus_b): its entries into the window's J slice (row:
+// its P half's first, d entries, the Q half L behind; NULL: the injections alone)
+// and S_o
+__device__ __noinline__ void ybus_row(const EwArgs &a, int o, double *row, int L, int d, double *P, double *Q)
 {
     double so, co;
     int_sincos(a.va[o], a.trig, &so, &co);
     const double v = a.vm[o], Vr = v * co, Vi = v * so;
-    double Ir = 0.0, Ii = 0.0;
-    YbusRow r;
+    double Ir = 0.0, Ii = 0.0, dTr = 0.0, dTi = 0.0, dVr = 0.0, dVi = 0.0;
     const int pe = a.tp[o + 1];
-    bool diag = true;   // still to come
-    for (int p = a.tp[o]; p < pe || diag;) {
+    int k = 0, kd = -1;   // the row's entries in column order; the diagonal's place
+    for (int p = a.tp[o]; p < pe || kd < 0;) {
         const int2 nq = p < pe ? a.tnbr[p] : make_int2(o + 1, 0);
-        const bool own = diag && nq.x > o;   // the diagonal's turn in column order
+        const bool own = kd < 0 && nq.x > o;   // the diagonal's turn
         if (!own && (nq.y & EW_ACCUM)) {
             ++p;
             continue;
         }
         const int j = own ? o : nq.x;
-        const double2 y = own ? a.yd[o] : ybus_entry(a, p, nq.y);
+        const double2 y = own ? a.yd[o] : ybus_entry(a, p);
         double s, c;
         int_sincos(a.va[j], a.trig, &s, &c);
         const double vj = a.vm[j];
         const double YUr = fma(y.x, c, -y.y * s), YUi = fma(y.x, s, y.y * c);
+        const double sVr = fma(Vr, YUr, Vi * YUi), sVi = fma(Vi, YUr, -Vr * YUi);   // V conj(YU)
+        const double sTr = vj * sVi, sTi = -vj * sVr;
         Ir = fma(vj, YUr, Ir);
         Ii = fma(vj, YUi, Ii);
         if (own) {
-            const double sVr = fma(Vr, YUr, Vi * YUi), sVi = fma(Vi, YUr, -Vr * YUi);   // V conj(YU)
-            r.dT = make_double2(vj * sVi, -vj * sVr);
-            r.dV = make_double2(sVr, sVi);
-            diag = false;
+            kd = k;
+            dTr = sTr;
+            dTi = sTi;
+            dVr = sVr;
+            dVi = sVi;
         } else {
             ++p;
+            if (row) {
+                row[k] = sTr;
+                row[k + d] = sVr;
+                row[L + k] = sTi;
+                row[L + k + d] = sVi;
+            }
         }
+        ++k;
     }
-    r.S = make_double2(fma(Vr, Ir, Vi * Ii), fma(Vi, Ir, -Vr * Ii));
-    r.dT.x -= r.S.y;   // + j S
-    r.dT.y += r.S.x;
-    r.dV.x += fma(Ir, co, Ii * so);   // + conj(I) U
-    r.dV.y += fma(Ir, so, -Ii * co);
-    return r;
+    const double Sr = fma(Vr, Ir, Vi * Ii), Si = fma(Vi, Ir, -Vr * Ii);
+    if (row) {
+        row[kd] = dTr - Si;                                   // + j S
+        row[kd + d] = dVr + fma(Ir, co, Ii * so);             // + conj(I) U
+        row[L + kd] = dTi + Sr;
+        row[L + kd + d] = dVi + fma(Ir, so, -Ii * co);
+    }
+    *P = Sr;
+    *Q = Si;
 }
 
 // One window per CTA; with PERSIST the CTAs loop over the windows
@@ -362,16 +372,20 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
             const longlong2 A = sA[ol], uq = sU[nq.x];
             const double vo = sW[ol].x, vq = sW[nq.x].x;
             double Gr, Gi;
-            if (A.x == kFixNaN || uq.x == kFixNaN || ey == 0 ||
-                !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, yf.x, yf.y, ey, &Gr, &Gi)) {
+            if (YBUS) {
+                // magnitudes whose products might leave the doubles' range, and
+                // non-finite angles: the row goes the general way
+                if (!(ybus_mid(ey) && ybus_mid(fix_vexp(vq)) && uq.x != kFixNaN) || A.x == kFixNaN ||
+                    !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, yf.x, yf.y, ey, &Gr, &Gi)) {
+                    Gr = Gi = 0.0;
+                    sbm[ol].z |= kYbusSlowRow;
+                }
+            } else if (A.x == kFixNaN || uq.x == kFixNaN || ey == 0 ||
+                       !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, yf.x, yf.y, ey, &Gr, &Gi)) {
                 const longlong2 uo = sU[ol];
-                const double2 yc = YBUS ? ybus_entry(a, t0 + i, nq.y) : a.tcoup[t0 + i];
+                const double2 yc = a.tcoup[t0 + i];
                 fix_G(A.x, A.y, vo, uo.x, uo.y, uq.x, uq.y, 0, 0, 0, yc.x, yc.y, &Gr, &Gi);
-                if (YBUS && (nq.y & EW_ACCUM)) Gr = Gi = 0.0;   // in the entry of its run's first terminal
             }
-            // magnitudes whose products might leave the doubles' range: the
-            // row's sums go the general way (ybus_row)
-            if (YBUS && !(ybus_mid(ey) && ybus_mid(fix_vexp(vq)))) sbm[ol].z |= kYbusSlowRow;
             const double Kr = vq * Gr, Ki = vq * Gi;   // K_t = v_q G
             if (JAC) {
                 skg[2 * i] = make_double2(Kr, Ki);
@@ -428,23 +442,15 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 }
                 const double2 vy = syd[b], vw = sW[b];   // v conj(Yd); v, 1/v
                 const double vc = im ? vy.y : vy.x;
-                const int pos = bm.x + (YBUS ? bm.z & ~kYbusSlowRow : bm.z);
+                if (YBUS && bm.z < 0) {   // below
+                    slow_row = true;
+                    continue;
+                }
+                const int pos = bm.x + bm.z;
                 jst[(im ? 0 : L) + pos] = neg_if(sK, im);                  // Re / Im of j sum K
                 jst[(im ? L : 0) + pos + d] = fma(sK, vw.y, fix_twice(vc));   // 2 v conj(Yd) + sum K / v
                 spq[(im ? pqs : 0) + b + par] = fma(vw.x, vc, sK);            // S = v^2 conj(Yd) + sum K
-                if (YBUS) slow_row |= bm.z < 0;
             }
-            if (YBUS && slow_row)
-                for (int x = tid; x < 2 * nbus; x += TB) {
-                    const int b = sord[x >> 1], im = x & 1;
-                    const int4 bm = sbm[b];
-                    if (bm.z >= 0) continue;
-                    const YbusRow r = ybus_row(a, b0 + b);
-                    const int pos = bm.x + (bm.z & ~kYbusSlowRow);
-                    jst[(im ? 0 : L) + pos] = im ? r.dT.x : r.dT.y;
-                    jst[(im ? L : 0) + pos + bm.y] = im ? r.dV.y : r.dV.x;
-                    spq[(im ? pqs : 0) + b + par] = im ? r.S.y : r.S.x;
-                }
         } else {
             // two threads per bus as above
             const double *k1 = reinterpret_cast<const double *>(skg);   // K.x, K.y per terminal
@@ -458,17 +464,19 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 for (; i < tend; ++i) sK += k1[2 * i + im];
                 const double2 y = syd[b];
                 const double v = sW[b].x;
-                spq[(im ? pqs : 0) + b + par] = fma(v, v * (im ? neg(y.y) : y.x), sK);   // S = v^2 conj(Yd) + sum K
-                if (YBUS) slow_row |= bm.z < 0;
+                if (YBUS && bm.z < 0)   // below
+                    slow_row = true;
+                else
+                    spq[(im ? pqs : 0) + b + par] = fma(v, v * (im ? neg(y.y) : y.x), sK);   // S = v^2 conj(Yd) + sum K
             }
-            if (YBUS && slow_row)
-                for (int x = tid; x < 2 * nbus; x += TB) {
-                    const int b = sord[x >> 1], im = x & 1;
-                    if (sbm[b].z >= 0) continue;
-                    const YbusRow r = ybus_row(a, b0 + b);
-                    spq[(im ? pqs : 0) + b + par] = im ? r.S.y : r.S.x;
-                }
         }
+        if (YBUS && slow_row)   // their entries, over those that the evaluation wrote
+            for (int x = tid; x < 2 * nbus; x += TB) {
+                const int b = sord[x >> 1];
+                const int4 bm = sbm[b];
+                if (bm.z < 0 && !(x & 1))
+                    ybus_row(a, b0 + b, JAC ? jst + bm.x : nullptr, L, bm.y, spq + b + par, spq + pqs + b + par);
+            }
 
         // ---- stores ----
         if (RED) {
@@ -559,7 +567,7 @@ __global__ void __launch_bounds__(256, 5) k_ew(EwArgs a)
 
 // the same by the Ybus method (one launch)
 template <bool JAC>
-__global__ void __launch_bounds__(256, 5) k_ybus_win(EwArgs a)
+__global__ void __launch_bounds__(256, 5) k_ybus_win(const __grid_constant__ EwArgs a)
 {
     ew_windows<JAC, false, false, true>(a);
 }
