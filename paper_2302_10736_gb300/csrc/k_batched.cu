@@ -316,9 +316,9 @@ __global__ void __launch_bounds__(256, 4) k_ewb(BatchArgs a)
                     sKr += skg[i].x;
                     sKi += skg[i].y;
                 }
-                const double v = x == tid ? vb : a.vm[sb + b0 + b];
-                spq[b + par] = fma(v, v * y.x, sKr);
-                spq[pqs + b + par] = fma(v, neg(v * y.y), sKi);
+                const double v = x == tid ? vb : a.vm[sb + b0 + b], v2 = v * v;
+                spq[b + par] = fma(v2, y.x, sKr);
+                spq[pqs + b + par] = fma(-v2, y.y, sKi);
             }
         }
         double *Js = JAC ? a.J + a.joff[s] : nullptr;

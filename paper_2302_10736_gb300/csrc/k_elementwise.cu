@@ -467,7 +467,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 if (YBUS && bm.z < 0)   // below
                     slow_row = true;
                 else
-                    spq[(im ? pqs : 0) + b + par] = fma(v, v * (im ? neg(y.y) : y.x), sK);   // S = v^2 conj(Yd) + sum K
+                    spq[(im ? pqs : 0) + b + par] = fma(v * v, im ? neg(y.y) : y.x, sK);   // S = v^2 conj(Yd) + sum K
             }
         }
         if (YBUS && slow_row)   // their entries, over those that the evaluation wrote
