@@ -29,9 +29,13 @@
 //   dL/dtheta_q = sum over q's terminals t (other bus o, mirror terminal m):
 //                 <r_q, j K_t> + <r_o, -j K_m>
 //   dL/dv_q     = <r_q, 2 v_q conj(Yd_q)> + (sum_t <r_q, K_t> + <r_o, K_m>) / v_q
-// with K_t = conj(Yc_t) V_q conj(V_o), K_m = conj(Yc_m) V_o conj(V_q): each bus
-// sums over its own terminals only (no scatter, fixed order).  Branch
-// parameter gradients come from the partials of Eqs. (5)-(6) by g, b, b_sh and
+// with K_t = conj(Yc_t) V_q conj(V_o), K_m = conj(Yc_m) V_o conj(V_q) = v_q G_m: each
+// bus sums over its own terminals only (no scatter, fixed order).  The K_t enter
+// through their sum alone, which the injections formed, and v_q is common to
+// the K_m, so a terminal's share is <r_o, -j G_m> and <r_o, G_m>:
+//   dL/dtheta_q = <r_q, j sum K> + v_q sum_t <r_o, -j G_m>
+//   dL/dv_q     = <r_q, 2 v_q conj(Yd_q)> + <r_q, sum K> / v_q + sum_t <r_o, G_m>.
+// Branch parameter gradients come from the partials of Eqs. (5)-(6) by g, b, b_sh and
 // the tap, one thread per branch summing the scenarios in ascending order.
 #include "fastmath.cuh"
 #include "fixrot.cuh"
@@ -63,7 +67,7 @@ struct BatchArgs {
     int *err;
     // adjoint
     const double *Ps, *Qs, *wP, *wQ;
-    double2 *r;
+    double2 *r, *sk;   // residuals; sum K of every bus
     double *lpart, *L, *gvm, *gva, *gg, *gb, *gbsh, *gtap;
     const double *Lbar;      // upstream gradient (device scalar; NULL = 1): scales every gradient
     double *Ltot;            // sum_s L_s (may be NULL)
@@ -420,13 +424,20 @@ __device__ __forceinline__ void batch_loss(const BatchArgs &a)
 
 // Branch-parameter gradients: the partials of Eqs. (5)-(6) by g, b, b_sh and
 // the tap m of branch (h, k), paired with the end residuals.  With
-// B = V_h conj(V_k) e^{-j phi}, A_h = v_h^2 / m^2, s_x = r_h.x + r_k.x,
-// d_x = r_h.x - r_k.x (likewise s_y, d_y), Q1 = B.x s_x + B.y d_y,
-// Q2 = B.x s_y - B.y d_x and S_sh = r_h.y A_h + r_k.y v_k^2, one scenario adds
-//   dL/dg    += r_h.x A_h + r_k.x v_k^2 - Q1 / m
-//   dL/db    += Q2 / m - S_sh
+// V' = V_h e^{-j phi} / m, B = V' conj(V_k), X_h = |V'|^2 r_h.x, Y_h = |V'|^2 r_h.y,
+// S_sh = Y_h + v_k^2 r_k.y,
+// Q1 = B.x (r_h.x + r_k.x) + B.y (r_h.y - r_k.y), Q2 = B.x (r_h.y + r_k.y) - B.y (r_h.x - r_k.x),
+// one scenario adds
+//   dL/dg    += X_h + v_k^2 r_k.x - Q1
+//   dL/db    += Q2 - S_sh
 //   dL/db_sh += -S_sh / 2
-//   dL/dm    += (-2 A_h (r_h.x g + r_h.y c1i) + (g Q1 - b Q2) / m) / m,  c1i = -(b + b_sh/2).
+//   dL/dm    += (g (Q1 - 2 X_h) - (b Q2 + 2 c1i Y_h)) / m,  c1i = -(b + b_sh/2).
+// Bound by the FP64 pipe (over a batch).  Taking the tap and the shift into V'
+// first leaves a line (V' = V_h, the warp skips the turn) 33 FP64 operations a
+// scenario instead of 48, a transformer 39: 250,000 buses x 16 states, the whole
+// adjoint 1,119 -> 1,086 us.  Each scenario's terms are joined before they are
+// added: summing X_h, Y_h and Q apart and joining them at the end (26 operations,
+// 1,031 us) loses the digits in which a scenario's terms cancel.
 struct BranchConst {
     int h, k;
     double g, bb, im, cphi, sphi, c1i;
@@ -439,56 +450,51 @@ __device__ __forceinline__ BranchConst branch_const(const BatchArgs &a, int l)
     return BranchConst{hk.x, hk.y, a.pg[l], a.pb[l], aux.x, aux.y, aux.z, aux.w};
 }
 
-template <bool ACC>
+struct BranchSums {
+    double g, b, sh, m;   // dL/dg, dL/db, -2 dL/db_sh, m dL/dm
+};
+
 __device__ __forceinline__ void branch_terms(const BranchConst &c, double2 Vh, double2 Vk, double2 rh, double2 rk,
-                                             double &agg, double &agb, double &agsh, double &agt)
+                                             BranchSums &t)
 {
-    const double im = c.im;
+    if (c.im != 1.0 || c.cphi != 1.0 || c.sphi != 0.0) {   // V'
+        const double x = Vh.x;
+        Vh.x = c.im * fma(x, c.cphi, Vh.y * c.sphi);
+        Vh.y = c.im * fma(Vh.y, c.cphi, -x * c.sphi);
+    }
     const double vh2 = fma(Vh.x, Vh.x, Vh.y * Vh.y), vk2 = fma(Vk.x, Vk.x, Vk.y * Vk.y);
-    const double Wr = fma(Vh.x, Vk.x, Vh.y * Vk.y), Wi = fma(Vh.y, Vk.x, -Vh.x * Vk.y);   // V_h conj(V_k)
-    const double Br = fma(Wr, c.cphi, Wi * c.sphi), Bi = fma(Wi, c.cphi, -Wr * c.sphi);   // W e^{-j phi}
+    const double Br = fma(Vh.x, Vk.x, Vh.y * Vk.y), Bi = fma(Vh.y, Vk.x, -Vh.x * Vk.y);   // V' conj(V_k)
     const double sx = rh.x + rk.x, dx = rh.x - rk.x, sy = rh.y + rk.y, dy = rh.y - rk.y;
     const double Q1 = fma(Br, sx, Bi * dy), Q2 = fma(Br, sy, -Bi * dx);
-    const double Ah = vh2 * (im * im);
-    const double Ssh = fma(rh.y, Ah, rk.y * vk2);
-    const double tg = fma(-im, Q1, fma(rh.x, Ah, rk.x * vk2));
-    const double tb = fma(im, Q2, -Ssh);
-    const double tsh = -0.5 * Ssh;
-    const double C = fma(rh.x, c.g, rh.y * c.c1i);
-    const double tt = im * fma(-2.0 * Ah, C, im * fma(c.g, Q1, -c.bb * Q2));
-    if (ACC) {
-        agg += tg;
-        agb += tb;
-        agsh += tsh;
-        agt += tt;
-    } else {
-        agg = tg;
-        agb = tb;
-        agsh = tsh;
-        agt = tt;
-    }
+    const double Xh = vh2 * rh.x, Yh = vh2 * rh.y, Ssh = fma(vk2, rk.y, Yh);
+    t.g += fma(vk2, rk.x, Xh) - Q1;
+    t.b += Q2 - Ssh;
+    t.sh += Ssh;
+    t.m += fma(c.g, fma(-2.0, Xh, Q1), -fma(c.bb, Q2, 2.0 * c.c1i * Yh));
+}
+
+__device__ __forceinline__ void branch_out(const BatchArgs &a, int l, const BranchConst &c, const BranchSums &t)
+{
+    a.gg[l] = t.g;
+    a.gb[l] = t.b;
+    a.gbsh[l] = -0.5 * t.sh;
+    a.gtap[l] = c.im * t.m;
 }
 
 // one thread per branch summing the scenarios in ascending order, from the
-// phasors V and the residuals r of every scenario in global memory
+// phasors V and the residuals r of every scenario in global memory (two
+// scenarios' loads in flight)
 __device__ __forceinline__ void branch_grad(const BatchArgs &a, int l, const BranchConst &c)
 {
-    double agg = 0.0, agb = 0.0, agsh = 0.0, agt = 0.0;
-    bool first = true;
+    BranchSums t{0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
     for (int s = 0; s < a.S; ++s) {
-        if (a.sc[s].l == l) continue;   // removed in this scenario
+        const bool out = a.sc[s].l == l;   // removed in this scenario
         const long long sb = (long long)s * a.nb;
         const double2 Vh = a.V[sb + c.h], Vk = a.V[sb + c.k], rh = a.r[sb + c.h], rk = a.r[sb + c.k];
-        if (first)
-            branch_terms<false>(c, Vh, Vk, rh, rk, agg, agb, agsh, agt);
-        else
-            branch_terms<true>(c, Vh, Vk, rh, rk, agg, agb, agsh, agt);
-        first = false;
+        if (!out) branch_terms(c, Vh, Vk, rh, rk, t);
     }
-    a.gg[l] = agg;
-    a.gb[l] = agb;
-    a.gbsh[l] = agsh;
-    a.gtap[l] = agt;
+    branch_out(a, l, c, t);
 }
 
 // This CTA's branches: a contiguous range of ceil(nl / gridDim.x), so that
@@ -565,7 +571,10 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
             const double dP = fma(v2, y.x, sKr) - a.Ps[o];
             const double dQ = fma(-v2, y.y, sKi) - a.Qs[o];
             const double wp = a.wP[o], wq = a.wQ[o];
-            if (GRAD) a.r[sb + o] = make_double2(tl * wp * dP, tl * wq * dQ);
+            if (GRAD) {
+                a.r[sb + o] = make_double2(tl * wp * dP, tl * wq * dQ);
+                a.sk[sb + o] = make_double2(sKr, sKi);
+            }
             spq[x] = fma(wp * dP, dP, wq * dQ * dQ);
         }
         __syncthreads();
@@ -587,16 +596,10 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
         for (int i = tid; i < nt; i += TB) {
             const int p = t0 + i;
             const int q = a.town[p], o = a.tnbr[p].x;   // q owns the terminal, o is the other end
-            const double2 rq = a.r[sb + q], ro = a.r[sb + o];
-            // K_t = conj(Yc_t) V_q conj(V_o) = v_o G_t and the mirror's K_m =
-            // conj(Yc_m) V_o conj(V_q) = v_q G_m, the G on the integer pipe
-            double gtr, gti, gmr, gmi, vo, vq;
-            batch_G(a, a.U + sb, p, q, o, &gtr, &gti, &vo);
+            const double2 ro = a.r[sb + o];
+            double gmr, gmi, vq;   // G_m, the mirror's, on the integer pipe
             batch_G(a, a.U + sb, a.tmir[p], o, q, &gmr, &gmi, &vq);
-            const double Kr = vo * gtr, Ki = vo * gti;
-            const double Mr = vq * gmr, Mi = vq * gmi;
-            double th = fma(-rq.x, Ki, rq.y * Kr) + fma(ro.x, Mi, -ro.y * Mr);
-            double vv = fma(rq.x, Kr, rq.y * Ki) + fma(ro.x, Mr, ro.y * Mi);
+            double th = fma(ro.x, gmi, -ro.y * gmr), vv = fma(ro.x, gmr, ro.y * gmi);
             if (p == sc.ph || p == sc.pk) th = vv = 0.0;
             skg[i] = make_double2(th, vv);
         }
@@ -620,12 +623,12 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
             }
             const int q = b0 + b;
             const double4_32a uq = a.U[sb + q];
-            const double2 rq = a.r[sb + q];
+            const double2 rq = a.r[sb + q], sk = a.sk[sb + q];
             const double2 y = syd[b];
-            const double tv = uq.z + uq.z;
-            // <r_q, 2 v_q conj(Yd)> + (sum) / v_q
-            spq[b + par] = gth;
-            spq[pqs + b + par] = fma(gv, uq.w, tv * fma(rq.x, y.x, -rq.y * y.y));
+            // <r_q, j sum K> + v_q (sum), and <r_q, 2 v_q conj(Yd)> + <r_q, sum K> / v_q + (sum)
+            spq[b + par] = fma(uq.z, gth, fma(-rq.x, sk.y, rq.y * sk.x));
+            spq[pqs + b + par] = fma(fix_twice(uq.z), fma(rq.x, y.x, -rq.y * y.y),
+                                     fma(uq.w, fma(rq.x, sk.x, rq.y * sk.y), gv));
         }
         if (a.aligned) {
             fence_proxy_async_smem();
@@ -656,15 +659,14 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
 // Small-batch adjoint: one (scenario, window) item per CTA (the launch has a
 // CTA for every item) and one grid barrier.  Before the barrier the item
 // forms the phasors of its own and ghost buses (slot j's bus in slotbus),
-// both flows of every terminal (o owns the terminal): K_t = conj(Yc_t) V_o
-// conj(V_q) and the mirror's K_m = conj(Yc_m) V_q conj(V_o), the complex
-// products in fixed point on the integer pipe (fixrot.cuh), then its buses'
-// injections and residuals.  All of it stays in shared
+// for every terminal (o owns it) its flow K_t = conj(Yc_t) V_o conj(V_q) and the
+// mirror's G_m = conj(Yc_m) V_q conj(U_o), the complex products in fixed point on
+// the integer pipe (fixrot.cuh), then its buses' injections and residuals.  All of it stays in shared
 // memory, so after the barrier the item reads back only its ghost buses'
 // residuals (one L2 round trip) before the state gradients (and, for a single
 // scenario, the gradients of the branches whose from-terminal it owns)
-//   dL/dtheta_o = sum_t <r_o, j K_t> + <r_q, -j K_m>
-//   dL/dv_o     = <r_o, 2 v_o conj(Yd_o)> + (sum_t <r_o, K_t> + <r_q, K_m>) / v_o.
+//   dL/dtheta_o = <r_o, j sum K> + v_o sum_t <r_q, -j G_m>
+//   dL/dv_o     = <r_o, 2 v_o conj(Yd_o)> + <r_o, sum K> / v_o + sum_t <r_q, G_m>.
 // GRAD = false: the loss alone (no mirror flows, residuals or gradients).
 template <bool GRAD>
 __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
@@ -675,7 +677,8 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
     int4 *sbm = reinterpret_cast<int4 *>(smem + sp.bm);
     double2 *syd = reinterpret_cast<double2 *>(smem + sp.yd);
     double2 *sK = reinterpret_cast<double2 *>(smem + sp.K);
-    double2 *sM = reinterpret_cast<double2 *>(smem + sp.M);
+    double2 *sM = reinterpret_cast<double2 *>(smem + sp.M);       // G_m of every terminal
+    double2 *sSK = reinterpret_cast<double2 *>(smem + sp.sk);     // sum K of the own buses
     int2 *sloc = reinterpret_cast<int2 *>(smem + sp.loc);   // per terminal: {owner slot, other-bus slot}
     __shared__ double swl[32];                                 // per-warp loss partials
     double *spq = reinterpret_cast<double *>(smem + sp.pq);
@@ -809,8 +812,8 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
                 loc = make_int2(a.town[p], a.tloc[p].x);
             }
             loc.x -= b0;
-            // K_t = conj(Yc_t) V_o conj(V_q) = v_q G_t and the mirror's K_m =
-            // conj(Yc_m) V_q conj(V_o) = v_o G_m, the G on the integer pipe
+            // K_t = conj(Yc_t) V_o conj(V_q) = v_q G_t and the mirror's G_m =
+            // conj(Yc_m) V_q conj(U_o), the G on the integer pipe
             const longlong2 Ao = sAf[loc.x], Uq = sUf[loc.y];
             const double vo = svs[loc.x], vq = svs[loc.y];
             double gr, gi;
@@ -831,9 +834,8 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
                     const double2 ym = a.tcoup[tm];
                     fix_G(Aq.x, Aq.y, vq, Uq.x, Uq.y, Uo.x, Uo.y, 0, 0, 0, ym.x, ym.y, &mr, &mi);
                 }
-                double Mr = vo * mr, Mi = vo * mi;
-                if (p == sc.ph || p == sc.pk) Mr = Mi = 0.0;
-                sM[i] = make_double2(Mr, Mi);
+                if (p == sc.ph || p == sc.pk) mr = mi = 0.0;
+                sM[i] = make_double2(mr, mi);
                 sloc[i] = loc;
             }
         }
@@ -870,6 +872,7 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
                     const double r = tl * wt * d;   // 2 Lbar w dS
                     gr[2 * b + im] = r;
                     rr[2 * b + im] = r;
+                    reinterpret_cast<double *>(sSK)[2 * b + im] = sk;
                 }
                 lt = fma(wt * d, d, lt);
             }
@@ -923,12 +926,8 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
         __syncthreads();
         // ---- state-gradient terms of every terminal ----
         for (int i = tid; i < nt; i += TB) {
-            const double2 K = sK[i], M = sM[i];
-            const int2 loc = sloc[i];
-            const double2 ro = sR[loc.x], rq = sR[loc.y];
-            const double th = fma(-ro.x, K.y, ro.y * K.x) + fma(rq.x, M.y, -rq.y * M.x);
-            const double vv = fma(ro.x, K.x, ro.y * K.y) + fma(rq.x, M.x, rq.y * M.y);
-            sK[i] = make_double2(th, vv);
+            const double2 M = sM[i], rq = sR[sloc[i].y];
+            sK[i] = make_double2(fma(rq.x, M.y, -rq.y * M.x), fma(rq.x, M.x, rq.y * M.y));
         }
         // the window's branches: h = the from-terminal's owner, k = its other bus
         for (int j = tid; j < nbr; j += TB) {
@@ -941,12 +940,9 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
                 c = branch_const(a, l);
             }
             const int2 loc = sloc[i];
-            double agg = 0.0, agb = 0.0, agsh = 0.0, agt = 0.0;
-            if (l != sc.l) branch_terms<false>(c, sV[loc.x], sV[loc.y], sR[loc.x], sR[loc.y], agg, agb, agsh, agt);
-            a.gg[l] = agg;
-            a.gb[l] = agb;
-            a.gbsh[l] = agsh;
-            a.gtap[l] = agt;
+            BranchSums bt{0.0, 0.0, 0.0, 0.0};
+            if (l != sc.l) branch_terms(c, sV[loc.x], sV[loc.y], sR[loc.x], sR[loc.y], bt);
+            branch_out(a, l, c, bt);
         }
         __syncthreads();
         const int pqs = (int)sp.pqs;
@@ -961,10 +957,11 @@ __global__ void __launch_bounds__(kAdj1Threads, 1) k_adj1(BatchArgs a)
                 double g = 0.0;
                 if (i < tend) g = kk[2 * i++ + im];
                 for (; i < tend; ++i) g += kk[2 * i + im];
-                if (im) {   // <r_o, 2 v_o conj(Yd)> + (sum) / v_o
-                    const double2 vw = sW[b], ro = sR[b], y = syd[b];
-                    g = fma(g, vw.y, (vw.x + vw.x) * fma(ro.x, y.x, -ro.y * y.y));
-                }
+                const double2 vw = sW[b], ro = sR[b], sk = sSK[b], y = syd[b];
+                if (im)   // <r_o, 2 v_o conj(Yd)> + <r_o, sum K> / v_o + (sum)
+                    g = fma(fix_twice(vw.x), fma(ro.x, y.x, -ro.y * y.y), fma(vw.y, fma(ro.x, sk.x, ro.y * sk.y), g));
+                else      // <r_o, j sum K> + v_o (sum)
+                    g = fma(vw.x, g, fma(-ro.x, sk.y, ro.y * sk.x));
                 spq[(im ? pqs : 0) + b + par] = g;
             }
         }
@@ -1033,6 +1030,7 @@ static BatchArgs batch_args(Batch *b)
     a.bar = g->bar;
     a.err = g->err;
     a.r = b->r;
+    a.sk = b->sk;
     a.lpart = b->lpart;
     a.pg = g->p_g;
     a.pb = g->p_b;

@@ -188,7 +188,7 @@ constexpr int kLossCountWord = 96;
 // form), residual and bus-name tables of the own and ghost slots, (v, 1/v) of
 // the own buses, the sine/cosine table.
 struct Adj1Smem {
-    uint32_t bm, yd, K, M, loc, pq, V, R, W, uf, af, vs, slot, tab, total, pqs;
+    uint32_t bm, yd, K, M, loc, pq, V, R, W, uf, af, vs, slot, sk, tab, total, pqs;
 };
 __host__ __device__ inline Adj1Smem adj1_smem_plan(int max_nbus, int max_nt, int max_nph)
 {
@@ -208,7 +208,8 @@ __host__ __device__ inline Adj1Smem adj1_smem_plan(int max_nbus, int max_nt, int
     p.af = p.uf + 16u * nph;
     p.vs = p.af + 16u * nph;
     p.slot = p.vs + 8u * ((nph + 1u) & ~1u);
-    p.tab = p.slot + ((4u * nph + 15u) & ~15u);
+    p.sk = p.slot + ((4u * nph + 15u) & ~15u);   // sum K of the own buses
+    p.tab = p.sk + 16u * nbus;
     p.total = p.tab + kTrigSmem;
     return p;
 }
@@ -443,6 +444,7 @@ struct Batch {
     double4_32a *U = nullptr;        // [S][nb]
     double2 *V = nullptr;            // [S][nb]
     double2 *r = nullptr;            // [S][nb] loss residual (2 wP dP, 2 wQ dQ)
+    double2 *sk = nullptr;           // [S][nb] sum of the bus's flows K (adjoint)
     double *lpart = nullptr;         // [S][nwin] per-window loss partial sums
     double *lscen = nullptr;         // [S] per-scenario losses when the caller wants only their total
     // co-resident CTAs of the batched kernels (inj, jac, adjoint, k_adj1, and
