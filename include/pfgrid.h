@@ -526,7 +526,7 @@ pf_status loss_elementwise(pf_batch *batch, const double *vm, const double *va, 
  * is involved): moves the arrival counter of the grid barrier that the
  * batched element-wise and adjoint kernels of this grid's batches share out
  * of range, so in the next such launch no CTA ever sees the last arrival;
- * each CTA gives up after 2 s, skips its work and sets the device error word,
+ * each waiting CTA gives up after 2 s (in the adjoint it skips its work) and sets the device error word,
  * and grid_check_error then returns PF_ETIMEOUT and resets the barrier.
  * (The single-scenario kernels have no grid-wide wait.)  Synchronizes
  * `stream`.

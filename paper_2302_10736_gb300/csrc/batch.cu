@@ -38,8 +38,9 @@ namespace pf {
 // The window plan of a batch: windows of at most tb buses and tfac x tb
 // terminals (tfac = 0: the largest of 3, 2, 1 at which four CTAs of the
 // batched Jacobian kernel share an SM's shared memory - its register budget
-// allows four; with three, barrier and load stalls leave more of the FP64
-// pipe idle: 1.53 against 1.47 ms for 1,024 N-1 scenarios of the 10,000-bus
+// allows four; larger windows have fewer ghost buses, but with three CTAs the
+// barriers show: 862 us at 2 against 907 at 3 and 1,016 at 1 for 1,024 N-1
+// scenarios of the 10,000-bus
 // grid - else the largest at which one fits).  When the batch has fewer
 // (scenario, window) items than the GPU has SMs, the windows are cut at equal
 // cost into about one item per SM (more CTAs would only make the grid
@@ -52,7 +53,8 @@ pf_status batch_plan(const Grid *g, int nscen, int tb, int tfac, HostEw &E, bool
         cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
         return set_error(PF_ECUDA, "batch: cannot query the device");
     auto smem_of = [](const HostEw &L) {
-        return ew_smem_plan(L.max_nbus, L.max_nt, L.max_L, true).total + kTrigSmem;
+        return std::max(ewb_smem_plan(L.max_nbus, L.max_nt, L.max_L, L.max_nph, true).total,
+                        ew_smem_plan(L.max_nbus, L.max_nt, 0, false).total + kTrigSmem);
     };
     const size_t kCtaReserve = 1024;   // shared memory the runtime keeps per resident CTA
     bool have = false;
@@ -131,15 +133,13 @@ pf_status batch_upload(Batch *b, HostEw &E, bool ghost, cudaStream_t st)
         (e = b->arena.alloc(&b->rorder, E.rorder.size())) ||
         (e = cudaMemcpyAsync(b->rorder, E.rorder.data(), sizeof(int) * E.rorder.size(), cudaMemcpyHostToDevice,
                              st)) ||
-        (ghost && ((e = b->arena.alloc(&b->desc, E.desc.size())) || (e = b->arena.alloc(&b->slotbus, E.slotbus.size())) ||
-                   (e = b->arena.alloc(&b->tloc, E.tloc.size())) ||
-                   (e = cudaMemcpyAsync(b->desc, E.desc.data(), sizeof(int4) * E.desc.size(), cudaMemcpyHostToDevice,
-                                        st)) ||
-                   (e = cudaMemcpyAsync(b->slotbus, E.slotbus.data(), sizeof(int) * E.slotbus.size(),
-                                        cudaMemcpyHostToDevice, st)) ||
-                   (e = cudaMemcpyAsync(b->tloc, E.tloc.data(), sizeof(int2) * E.tloc.size(), cudaMemcpyHostToDevice,
-                                        st)) ||
-                   (e = b->arena.alloc(&b->brl, std::max<size_t>(brl.size(), 1))) ||
+        (e = b->arena.alloc(&b->desc, E.desc.size())) || (e = b->arena.alloc(&b->slotbus, E.slotbus.size())) ||
+        (e = b->arena.alloc(&b->tloc, E.tloc.size())) ||
+        (e = cudaMemcpyAsync(b->desc, E.desc.data(), sizeof(int4) * E.desc.size(), cudaMemcpyHostToDevice, st)) ||
+        (e = cudaMemcpyAsync(b->slotbus, E.slotbus.data(), sizeof(int) * E.slotbus.size(), cudaMemcpyHostToDevice,
+                             st)) ||
+        (e = cudaMemcpyAsync(b->tloc, E.tloc.data(), sizeof(int2) * E.tloc.size(), cudaMemcpyHostToDevice, st)) ||
+        (ghost && ((e = b->arena.alloc(&b->brl, std::max<size_t>(brl.size(), 1))) ||
                    (!brl.empty() &&
                     (e = cudaMemcpyAsync(b->brl, brl.data(), sizeof(int2) * brl.size(), cudaMemcpyHostToDevice, st))))) ||
         (e = b->arena.alloc(&b->lpart, nw)) || (e = cudaStreamSynchronize(st)))
@@ -210,7 +210,8 @@ PF_API pf_status batch_create(pf_grid *grid, int32_t nscen, const int32_t *outag
     const size_t n = (size_t)nscen * g->nb;
     cudaError_t e = cudaSuccess;
     if ((e = b->arena.alloc(&b->sc, std::max(nscen, 1))) || (e = b->arena.alloc(&b->joff, nscen + 1)) ||
-        (e = b->arena.alloc(&b->U, n)) || (e = b->arena.alloc(&b->V, n)) || (e = b->arena.alloc(&b->r, n)) || (e = b->arena.alloc(&b->sk, n)) ||
+        (e = b->arena.alloc(&b->U, n)) || (e = b->arena.alloc(&b->V, n)) || (e = b->arena.alloc(&b->r, n)) ||
+        (e = b->arena.alloc(&b->sk, n)) ||
         (e = b->arena.alloc(&b->lscen, std::max(nscen, 1))) ||
         (nscen && (e = cudaMemcpyAsync(b->sc, b->h_sc.data(), sizeof(ScenOut) * nscen, cudaMemcpyHostToDevice, st))) ||
         (e = cudaMemcpyAsync(b->joff, b->h_joff.data(), sizeof(long long) * (nscen + 1), cudaMemcpyHostToDevice,

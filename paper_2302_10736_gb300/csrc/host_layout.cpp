@@ -92,6 +92,7 @@ pf_status host_topology(int nb, int nl, const int *from, const int *to, HostTopo
         H.tpos[t] = p;
         H.tnbr[p] = make_int2(H.other(t), H.tkpos[t] | (H.taccum[t] ? EW_ACCUM : 0));
         H.town[p] = H.owner(t);
+        if (p > 0 && H.taccum[t]) H.tnbr[p - 1].y |= EW_MORE;
     }
     for (int p = 0; p < T; ++p) H.tmir[p] = H.tpos[H.tsort[p] ^ 1];
     const int nnz = H.nnz;
@@ -278,6 +279,8 @@ pf_status host_selfcheck(const HostTopo &H, const HostEw &E)
         CHECK(kp >= 0 && kp < H.rp[o + 1] - H.rp[o] && kp != H.kd[o], "slot of sorted terminal %d", p);
         const bool acc = (H.tnbr[p].y & EW_ACCUM) != 0;
         CHECK(acc == (p > H.tp[o] && H.tnbr[p - 1].x == q), "parallel-run flag of sorted terminal %d", p);
+        CHECK(((H.tnbr[p].y & EW_MORE) != 0) == (p + 1 < H.tp[o + 1] && H.tnbr[p + 1].x == q),
+              "parallel-run continuation of sorted terminal %d", p);
         const int m = H.tmir[p];
         CHECK(m >= 0 && m < T && H.town[m] == q && H.tnbr[m].x == o && H.tmir[m] == p, "mirror of terminal %d", p);
     }

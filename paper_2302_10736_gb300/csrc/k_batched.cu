@@ -1,15 +1,14 @@
 // k_batched.cu - element-wise method over many scenarios in one persistent
-// cooperative launch: N-1 contingency batches and the adjoint of the mismatch
-// loss.  (The paper evaluates one state of one grid; batching and
+// cooperative launch: N-1 contingency batches and the adjoint of the mismatch loss.  (The paper evaluates one state of one grid; batching and
 // differentiation are the two extensions this library adds around the same
 // per-terminal evaluation and reduction, see k_elementwise.cu.)
 //
-// Work items are (scenario, window) pairs in scenario-major order, handed to
-// the resident CTAs round-robin, so the CTAs active at any time share a few
-// scenarios' phasors in L2.  Phase 1 forms every scenario's phasors (flat
-// chunks of blockDim.x buses, every lane busy); a grid barrier follows; phase
-// 2 evaluates.  The adjoint (k_adj) adds a residual phase and a second
-// barrier.  A small batch (about one item per SM) runs k_adj1 instead: one
+// Work items are (scenario, window) pairs.  Jacobians and injections (k_ewb)
+// take all scenarios of a window in turn and form each item's phasors in the
+// item.  The adjoint (k_adj) takes scenario-major order, round-robin
+// over the resident CTAs, which so share a few scenarios' phasors in L2: phase 1
+// forms every scenario's phasors (flat chunks of blockDim.x buses, every lane
+// busy), a grid barrier, then the residuals, a second barrier, the gradients.  A small batch (about one item per SM) runs k_adj1 instead: one
 // item per CTA, each window's own and ghost phasors formed inside the residual
 // phase (as k_elementwise.cu does), one grid barrier, and everything the
 // gradient phase needs kept in shared memory across it.
@@ -145,27 +144,6 @@ __device__ __forceinline__ void batch_G(const BatchArgs &a, const double4_32a *U
     *vq = uq.z;
 }
 
-// phase 1 of the Jacobian and injection batches: the phasors in the
-// fixed-point form of the single evaluation (fixrot.cuh), U[x] = {2^62 cos,
-// 2^62 sin (64-bit integers, stored bit for bit), v, 1/v (Jacobian only)}
-__device__ __forceinline__ void batch_phasors_fix(const BatchArgs &a, const ITrig *tab, bool jac)
-{
-    const int tid = threadIdx.x, TB = blockDim.x;
-    const int nchunk = (a.nb + TB - 1) / TB;
-    const long long nitem = (long long)a.S * nchunk;
-    for (long long it = blockIdx.x; it < nitem; it += gridDim.x) {
-        const int s = (int)(it / nchunk), c = (int)(it % nchunk);
-        const int o = c * TB + tid;
-        if (o < a.nb) {
-            const long long x = (long long)s * a.nb + o;
-            int64_t C, S;
-            int_sincos_q62(a.va[x], tab, &C, &S);
-            const double v = a.vm[x];
-            a.U[x] = make_double4_32a(__longlong_as_double(C), __longlong_as_double(S), v, jac ? fast_rcp(v) : 0.0);
-        }
-    }
-}
-
 // Window metadata of item (s, w) into shared memory, corrected for the
 // scenario's outage: {J-slice row offset, row length, diagonal position,
 // first terminal} per bus and the self sum Yd without the outage branch.
@@ -193,169 +171,253 @@ __device__ __forceinline__ void batch_window_meta(const BatchArgs &a, const Scen
     }
 }
 
+// G = conj(Yc_p) V_o conj(U_q) of terminal p from the window's phasor table:
+// fixed point on the integer pipe where it applies (fixrot.cuh), else FP64 products
+__device__ __forceinline__ void window_G(const BatchArgs &a, int p, longlong2 A, longlong2 uo, double vo, longlong2 uq,
+                                         longlong2 yf, int ey, double *gr, double *gi)
+{
+    if (A.x == kFixNaN || uq.x == kFixNaN || ey == 0 ||
+        !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, yf.x, yf.y, ey, gr, gi)) {
+        const double2 yc = a.tcoup[p];
+        fix_G(A.x, A.y, vo, uo.x, uo.y, uq.x, uq.y, 0, 0, 0, yc.x, yc.y, gr, gi);
+    }
+}
+
+// Jacobians and injections of a batch: persistent CTAs, each over a contiguous
+// run of (window, scenario) items, all scenarios of a window first, so that the
+// window's bus records stay in shared memory and each thread's first two
+// terminals in registers over the run (a scenario whose outage touches the
+// window rewrites the records).  As in the single evaluation the item forms the
+// phasors of the window's own and ghost buses, then its terminals, its bus sums
+// and diagonals, and leaves its J slices to the bulk copy while the next item's
+// phasors are formed.  Against the phasors of all scenarios in a first phase (32
+// bytes a bus written and read back), a grid barrier and scenario-major items
+// that reload the window: 10,000 buses x 1,024 outages 1,027 -> 862 us (with
+// windows of 128 threads 991 -> 851), 2,000 x 16 13.2 -> 10.2.
+//
+// What bounds it: no one unit.  At 10,000 x 128 the FP64 pipe is 46 % busy, the
+// integer ALU 47 %, the integer multiplier 45 %, instruction issue 53 %; warps
+// wait mostly at the three barriers of an item.  Two more CTAs an SM (48
+// registers) change nothing.  The sums of an item and the next one's phasors in
+// one interval between barriers, with two staging buffers: 1,060 us; with one,
+// 988.  The next state's loads in registers across the sums: 869.
+struct EwbTerm {
+    longlong2 yf;
+    int2 nq;   // the other bus's slot, position | flags
+    int ey, ol;
+};
+
 template <bool JAC>
 __global__ void __launch_bounds__(256, 4) k_ewb(BatchArgs a)
 {
     extern __shared__ __align__(16) char smem[];
     const GridBar gbar = grid_barrier_begin(a.bar);
-    const EwSmem sp = ew_smem_plan(a.max_nbus, a.max_nt, JAC ? a.max_L : 0, JAC);
+    const unsigned int arrived = grid_arrive(gbar);
+    const EwbSmem sp = ewb_smem_plan(a.max_nbus, a.max_nt, a.max_L, a.max_nph, JAC);
     int4 *sbm = reinterpret_cast<int4 *>(smem + sp.bm);
     double2 *syd = reinterpret_cast<double2 *>(smem + sp.yd);
-    double2 *skg = reinterpret_cast<double2 *>(smem + sp.kg);
-    int *skp = reinterpret_cast<int *>(smem + sp.kp);
+    longlong2 *sA = reinterpret_cast<longlong2 *>(smem + sp.A);   // own buses: V in block floating point
+    longlong2 *sU = reinterpret_cast<longlong2 *>(smem + sp.U);   // 2^62 (cos, sin)
+    double *sv = reinterpret_cast<double *>(smem + sp.v);         // v
+    double *siv = reinterpret_cast<double *>(smem + sp.iv);       // own buses: 1/v
+    int *sord = reinterpret_cast<int *>(smem + sp.ord);           // reduction thread -> bus
+    double2 *sK = reinterpret_cast<double2 *>(smem + sp.K);       // injections alone: K of every terminal
     double *jst = reinterpret_cast<double *>(smem + sp.jst);
     double *spq = reinterpret_cast<double *>(smem + sp.pq);
-    ITrig *tab = reinterpret_cast<ITrig *>(smem + sp.total);
-    const int tid = threadIdx.x, TB = blockDim.x;
+    ITrig *tab = reinterpret_cast<ITrig *>(smem + sp.tab);
+    const int tid = threadIdx.x, TB = blockDim.x, pqs = (int)sp.pqs;
     const ITrig *trig = a.trig + (blockIdx.x % kITrigCopies) * kITrigN;
     for (int k = tid; k < kITrigN; k += TB) tab[k] = trig[k];
     __syncthreads();
-    batch_phasors_fix(a, tab, JAC);
-    if (!grid_barrier(gbar, a.bar, gridDim.x, 0, a.err, DEV_TIMEOUT, kBatchBarrierNs)) return;
 
     const long long nitem = (long long)a.S * a.nwin;
-    for (long long it = blockIdx.x; it < nitem; it += gridDim.x) {
-        const int s = (int)(it / a.nwin), w = (int)(it % a.nwin);
+    long long it = nitem * blockIdx.x / gridDim.x;
+    const long long last = nitem * (blockIdx.x + 1) / gridDim.x;
+    int w = (int)(it / a.S), s = (int)(it % a.S);
+    constexpr int NT = 2;   // terminals per thread kept in registers
+    EwbTerm tr[NT];
+    bool fresh = true, dirty = true;   // a window not yet seen; bus records of another scenario
+    for (; it < last; ++it) {
+        const int *sbus = a.slotbus + (long long)w * a.max_nph;
+        const int4 d0 = a.desc[2 * w], d1 = a.desc[2 * w + 1];
+        const int b0 = d0.x, nbus = d0.y, b1 = b0 + nbus, t0 = d0.z, nt = d0.w, nph = d1.z;
         const ScenOut sc = a.sc[s];
-        const int b0 = a.win_bus[w], b1 = a.win_bus[w + 1], nbus = b1 - b0;
-        const int t0 = a.tp[b0], nt = a.tp[b1] - t0;
         const int del = sc.del;
+        const bool touched = (sc.h >= b0 && sc.h < b1) || (sc.k >= b0 && sc.k < b1);
         const int ndb = del * ((sc.h >= 0 && sc.h < b0) + (sc.k >= 0 && sc.k < b0));
         const int ndw = del * ((sc.h >= b0 && sc.h < b1) + (sc.k >= b0 && sc.k < b1));
-        const int r0s = a.rp[b0] - ndb;
-        const int Ls = JAC ? 2 * (a.rp[b1] - a.rp[b0]) - 2 * ndw : 0;
-        const int nnzs = a.nnz - 2 * del;
+        const int r0s = d1.x - ndb, Ls = JAC ? d1.y - 2 * ndw : 0;
         const long long sb = (long long)s * a.nb;
-        __syncthreads();   // previous item's shared-memory readers are done
-        batch_window_meta(a, sc, b0, b1, t0, sbm, syd);
-        // the reduction thread's bus: the window's buses by decreasing terminal count
-        double4_32a ub = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-        double vb = 0.0;
-        int bo = 0;
-        if (tid < nbus) {
-            bo = a.rorder[b0 + tid];
-            if (JAC)
-                ub = a.U[sb + b0 + bo];
-            else
-                vb = a.vm[sb + b0 + bo];
+        if (fresh) {
+#pragma unroll
+            for (int r = 0; r < NT; ++r) {
+                const int p = t0 + tid + r * TB;
+                if (tid + r * TB < nt) tr[r] = EwbTerm{a.tcfx[p], a.tloc[p], a.tce[p], a.town[p]};
+            }
         }
+
+        // ---- phasors of the own and ghost buses ----
+        for (int j = tid; j < nph; j += TB) {
+            const int o = sbus[j];
+            const double th = a.va[sb + o], v = a.vm[sb + o];
+            int64_t C, S;
+            int_sincos_q62(th, tab, &C, &S);
+            sU[j] = make_longlong2(C, S);
+            sv[j] = v;
+            if (j < nbus) {
+                int64_t ar, ai;
+                fix_phasor(C, S, v, &ar, &ai);
+                sA[j] = make_longlong2(ar, ai);
+                if (JAC) siv[j] = fast_rcp(v);
+            }
+        }
+        if (fresh)
+            for (int b = tid; b < nbus; b += TB) sord[b] = a.rorder[b0 + b];
+        if (dirty || touched) batch_window_meta(a, sc, b0, b1, t0, sbm, syd);
+        fresh = false;
+        dirty = touched;
+        if (tid == 0) bulk_wait_read();   // the previous item's slices
         __syncthreads();
-        for (int i = tid; i < nt; i += TB) {
-            const int p = t0 + i;
-            const int2 nq = a.tnbr[p];
-            const int ol = a.town[p] - b0, o = b0 + ol;
-            const bool masked = p == sc.ph || p == sc.pk;
-            // G = conj(Yc) V_o conj(U_q) on the integer pipe, as in the single evaluation
-            double Gr, Gi, vq;
-            batch_G(a, a.U + sb, p, o, nq.x, &Gr, &Gi, &vq);
+
+        // ---- evaluation: one terminal per thread ----
+        int runs = 0;
+        auto terminal = [&](int i, const EwbTerm &x) {
+            const int p = t0 + i, ol = x.ol - b0, ey = x.ey;
+            const int2 nq = x.nq;
+            const longlong2 yf = x.yf;
+            if (JAC && (nq.y & EW_ACCUM)) return;   // with the first branch of its parallel run
+            double Gr, Gi;
+            window_G(a, p, sA[ol], sU[ol], sv[ol], sU[nq.x], yf, ey, &Gr, &Gi);
+            if (p == sc.ph || p == sc.pk) Gr = Gi = 0.0;   // outage branch
+            const double vq = sv[nq.x], Kr = vq * Gr, Ki = vq * Gi;   // K_t = v_q G
             if (JAC) {
-                if (masked) Gr = Gi = 0.0;
-                const double Kr = vq * Gr, Ki = vq * Gi;
-                const int kp = nq.y & EW_KMASK;
-                const int kps = kp - del * ((o == sc.h && kp > sc.kh) + (o == sc.k && kp > sc.kk));
-                const bool gone = del && ((o == sc.h && kp == sc.kh) || (o == sc.k && kp == sc.kk));
-                skg[2 * i] = make_double2(Kr, Ki);
-                skg[2 * i + 1] = make_double2(Gr, Gi);
-                skp[i] = gone ? 0 : (kps | (nq.y & EW_ACCUM));
-                if (!gone && !(nq.y & EW_ACCUM)) {
-                    const int4 bm = sbm[ol];
-                    const int pos = bm.x + kps, d = bm.y;
-                    jst[pos] = Ki;
-                    jst[pos + d] = Gr;
-                    jst[Ls + pos] = neg(Kr);
-                    jst[Ls + pos + d] = Gi;
+                runs |= nq.y;
+                const int4 bm = sbm[ol];
+                int kp = nq.y & EW_KMASK;
+                if (touched && del) {
+                    const int o = b0 + ol;
+                    if ((o == sc.h && kp == sc.kh) || (o == sc.k && kp == sc.kk)) return;   // its pair is gone
+                    kp -= (o == sc.h && kp > sc.kh) + (o == sc.k && kp > sc.kk);
                 }
+                double *e = jst + bm.x + kp;
+                e[0] = Ki;              // J11 = Re(-j K)
+                e[bm.y] = Gr;           // J12
+                e[Ls] = neg(Kr);        // J21 = Im(-j K)
+                e[Ls + bm.y] = Gi;      // J22
             } else {
-                double Kr = vq * Gr, Ki = vq * Gi;
-                if (masked) Kr = Ki = 0.0;
-                skg[i] = make_double2(Kr, Ki);
+                sK[i] = make_double2(Kr, Ki);
             }
+        };
+#pragma unroll
+        for (int r = 0; r < NT; ++r)
+            if (tid + r * TB < nt) terminal(tid + r * TB, tr[r]);
+        for (int i = tid + NT * TB; i < nt; i += TB) {
+            const int p = t0 + i;
+            terminal(i, EwbTerm{a.tcfx[p], a.tloc[p], a.tce[p], a.town[p]});
         }
-        __syncthreads();
-        const int pqs = (int)sp.pqs;
-        const int par = (int)((sb + b0) & 1);
-        for (int x = tid; x < nbus; x += TB) {
-            const int b = x == tid ? bo : a.rorder[b0 + x];
-            const int4 bm = sbm[b];
-            const int tend = b + 1 < nbus ? sbm[b + 1].w : nt;
-            const double2 y = syd[b];
-            // sums start from the first terminal (never EW_ACCUM: it starts its run)
-            double sKr = 0.0, sKi = 0.0;
-            int i1 = bm.w;
-            if (i1 < tend) {
-                const double2 K = skg[JAC ? 2 * i1 : i1];
-                sKr = K.x;
-                sKi = K.y;
-                ++i1;
+        // the later branches of parallel runs onto the entries that this thread wrote
+        if (JAC && (runs & EW_MORE))
+            for (int i = tid; i < nt; i += TB) {
+                int p = t0 + i;
+                const int2 f = a.tloc[p];
+                if ((f.y & EW_ACCUM) || !(f.y & EW_MORE)) continue;
+                const int x = a.town[p] - b0, o = b0 + x;
+                const int4 bm = sbm[x];
+                int kp = f.y & EW_KMASK, more;
+                kp -= del * ((o == sc.h && kp > sc.kh) + (o == sc.k && kp > sc.kk));
+                double *e = jst + bm.x + kp;
+                do {
+                    ++p;
+                    more = a.tloc[p].y & EW_MORE;
+                    if (p == sc.ph || p == sc.pk) continue;   // outage branch
+                    double Gr, Gi;
+                    window_G(a, p, sA[x], sU[x], sv[x], sU[f.x], a.tcfx[p], a.tce[p], &Gr, &Gi);
+                    const double vq = sv[f.x];
+                    e[0] += vq * Gi;
+                    e[bm.y] += Gr;
+                    e[Ls] -= vq * Gr;
+                    e[Ls + bm.y] += Gi;
+                } while (more);
             }
+        __syncthreads();
+
+        // the next item's state towards L2 meanwhile
+        if (it + 1 < last && s + 1 < a.S)
+            for (int j = tid; j < nph; j += TB) {
+                const long long x = sb + a.nb + sbus[j];
+                prefetch_l2(a.va + x);
+                prefetch_l2(a.vm + x);
+            }
+
+        // ---- bus sums, diagonal entries, S: two threads per bus, x = 2b' + im
+        // (the single evaluation's order of operations) ----
+        const int par = (int)((sb + b0) & 1);
+        for (int x = tid; x < 2 * nbus; x += TB) {
+            const int b = sord[x >> 1], im = x & 1;
+            const int4 bm = sbm[b];
+            const double2 y = syd[b];
+            const double v = sv[b];
+            double sum = 0.0;
             if (JAC) {
                 const int d = bm.y;
-                for (int i = i1; i < tend; ++i) {
-                    const double2 K = skg[2 * i];
-                    sKr += K.x;
-                    sKi += K.y;
-                    const int kp = skp[i];
-                    if (kp & EW_ACCUM) {
-                        const double2 G = skg[2 * i + 1];
-                        const int pos = bm.x + (kp & EW_KMASK);
-                        jst[pos] += K.y;
-                        jst[pos + d] += G.x;
-                        jst[Ls + pos] -= K.x;
-                        jst[Ls + pos + d] += G.y;
-                    }
-                }
-                const double4_32a uo = x == tid ? ub : a.U[sb + b0 + b];
-                const double v = uo.z, iv = uo.w, vyr = v * y.x, vyi = neg(v * y.y);   // v conj(Yd)
-                const int pos = bm.x + bm.z;
-                // 2 v conj(Yd) + sum K / v and S = v^2 conj(Yd) + sum K, in the
-                // single evaluation's order of operations
-                jst[pos] = neg(sKi);
-                jst[pos + d] = fma(sKr, iv, fix_twice(vyr));
-                jst[Ls + pos] = sKr;
-                jst[Ls + pos + d] = fma(sKi, iv, fix_twice(vyi));
-                spq[b + par] = fma(v, vyr, sKr);
-                spq[pqs + b + par] = fma(v, vyi, sKi);
+                double *row = jst + (im ? 0 : Ls) + bm.x;   // K along the staged row, past the diagonal
+                if (d > 1) sum = row[bm.z == 0];
+#pragma unroll 1
+                for (int k = 1; k < d - 1; ++k) sum += row[k + (k >= bm.z)];
+                sum = neg_if(sum, !im);
+                const double vc = v * (im ? neg(y.y) : y.x);   // v conj(Yd)
+                double *e = jst + bm.x + bm.z;
+                e[im ? 0 : Ls] = neg_if(sum, im);                                // Re / Im of j sum K
+                e[(im ? Ls : 0) + d] = fma(sum, siv[b], fix_twice(vc));          // 2 v conj(Yd) + sum K / v
+                spq[(im ? pqs : 0) + b + par] = fma(v, vc, sum);                 // S = v^2 conj(Yd) + sum K
             } else {
-                for (int i = i1; i < tend; ++i) {
-                    sKr += skg[i].x;
-                    sKi += skg[i].y;
-                }
-                const double v = x == tid ? vb : a.vm[sb + b0 + b], v2 = v * v;
-                spq[b + par] = fma(v2, y.x, sKr);
-                spq[pqs + b + par] = fma(-v2, y.y, sKi);
+                const double *k1 = reinterpret_cast<const double *>(sK);
+                const int tend = b + 1 < nbus ? sbm[b + 1].w : nt;
+                int i = bm.w;
+                if (i < tend) sum = k1[2 * i++ + im];
+                for (; i < tend; ++i) sum += k1[2 * i + im];
+                spq[(im ? pqs : 0) + b + par] = fma(v * v, im ? neg(y.y) : y.x, sum);
             }
         }
-        double *Js = JAC ? a.J + a.joff[s] : nullptr;
+
+        // ---- stores ----
+        double *Jp = JAC ? a.J + a.joff[s] + 2 * (long long)r0s : nullptr;
+        double *Jq = JAC ? Jp + 2 * (long long)(a.nnz - 2 * del) : nullptr;
         if (a.aligned) {
             fence_proxy_async_smem();
             __syncthreads();
             if (tid == 0) {
                 if (JAC) {
-                    bulk_s2g(Js + 2 * (long long)r0s, jst, 8u * (uint32_t)Ls);
-                    bulk_s2g(Js + 2 * (long long)nnzs + 2 * (long long)r0s, jst + Ls, 8u * (uint32_t)Ls);
+                    bulk_s2g(Jp, jst, 8u * (uint32_t)Ls);
+                    bulk_s2g(Jq, jst + Ls, 8u * (uint32_t)Ls);
                 }
                 if (a.P) {
                     store_range_ll(a.P, spq, sb + b0, sb + b1);
                     store_range_ll(a.Q, spq + pqs, sb + b0, sb + b1);
                 }
                 bulk_commit();
-                bulk_wait_read();
             }
         } else {
             __syncthreads();
-            if (JAC) {
+            if (JAC)
                 for (int x = tid; x < Ls; x += TB) {
-                    Js[2 * (long long)r0s + x] = jst[x];
-                    Js[2 * (long long)nnzs + 2 * (long long)r0s + x] = jst[Ls + x];
+                    Jp[x] = jst[x];
+                    Jq[x] = jst[Ls + x];
                 }
-            }
             if (a.P)
                 for (int b = tid; b < nbus; b += TB) {
                     a.P[sb + b0 + b] = spq[b + par];
                     a.Q[sb + b0 + b] = spq[pqs + b + par];
                 }
         }
+        if (++s == a.S) {
+            s = 0;
+            ++w;
+            fresh = dirty = true;
+        }
     }
+    grid_arrive_end(gbar, arrived, a.bar, gridDim.x, a.err, DEV_TIMEOUT, kBatchBarrierNs);
+    if (tid == 0) bulk_wait_read();   // shared memory stays allocated until the copies have read it
 }
 
 // ------------------------------------------------------------ adjoint ----
@@ -1095,8 +1157,7 @@ cudaError_t launch_ew_batched(Batch *b, bool jac, const double *vm, const double
     a.Q = Q;
     a.J = J;
     a.aligned = (!J || al16(J)) && (!P || (al16(P) && al16(Q)));
-    const EwSmem sp = ew_smem_plan(a.max_nbus, a.max_nt, jac ? a.max_L : 0, jac);
-    const size_t smem = sp.total + kTrigSmem;
+    const size_t smem = ewb_smem_plan(a.max_nbus, a.max_nt, a.max_L, a.max_nph, jac).total;
     const long long items = (long long)b->S * b->nwin;
     const long long cap = (long long)b->cfg.ctas_per_sm * b->nsm;
     if (jac) return coop_launch(k_ewb<true>, b->resident[1], b->tb, smem, items, s, a, cap);

@@ -28,11 +28,12 @@
 // Reduction step (Eq. 7 and the copy-add of Fig. 2, without atomics).
 // Terminals are stored sorted by (owner, other bus), so a CTA owns a window of
 // consecutive buses together with all of their terminals: the off-diagonal
-// slot (o, q) is written by the terminal's thread (parallel branches,
-// adjacent in the sorted order, are added by the owner's thread below), and
-// two threads per bus (the real and the imaginary parts; the window's buses
+// slot (o, q) is written by the terminal's thread (the first of a run of
+// parallel branches, which are adjacent in the sorted order, adds the others),
+// and two threads per bus (the real and the imaginary parts; the window's buses
 // taken by decreasing terminal count, so that a warp's lanes loop equally
-// long) sum its terminals' K in a fixed order:
+// long) sum K in a fixed order, with a Jacobian along the bus's staged row, whose
+// J11 and J21 entries are the K, else over its terminals:
 //     S_o           = v_o^2 conj(Yd_o) + sum K
 //     dS_o/dtheta_o = j sum K
 //     dS_o/dv_o     = 2 v_o conj(Yd_o) + (sum K) / v_o
@@ -228,7 +229,6 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
     int4 *sbm = reinterpret_cast<int4 *>(smem + sp.bm);
     double2 *syd = reinterpret_cast<double2 *>(smem + sp.yd);   // Yd, or (Jacobian) v conj(Yd)
     double2 *skg = reinterpret_cast<double2 *>(smem + sp.kg);
-    int *skp = reinterpret_cast<int *>(smem + sp.kp);
     double *jst = reinterpret_cast<double *>(smem + sp.jst);
     double *spq = reinterpret_cast<double *>(smem + sp.pq);
     longlong2 *sA = reinterpret_cast<longlong2 *>(smem + sp.ph);             // own buses: V in block floating point
@@ -358,7 +358,12 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
         __syncthreads();
         PF_PROBE_MARK(1);
 
-        // ---- evaluation: one terminal per thread ----
+        // ---- evaluation: one terminal per thread.  With a Jacobian nothing but
+        // the staged entries is kept for the sums (a second copy of K and G and
+        // the slot positions were 36 bytes a terminal and three more stores; with
+        // them and the parallel runs in the sums' loop 70,000 buses took 8.55 us,
+        // 410,000 42.9, without 7.5 and 38.7) ----
+        int runs = 0;
         for (int i = tid; i < nt; i += TB) {
             if (i != tid) {
                 yf = a.tcfx[t0 + i];
@@ -367,6 +372,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 ol = a.town[t0 + i];
             }
             ol -= b0;
+            if (JAC && (nq.y & EW_ACCUM)) continue;   // with the first branch of its parallel run
             // G = conj(Yc) V_o conj(U_q) = dS_t/dv_q on the integer pipe (FP64
             // products for the values the fixed-point form does not hold)
             const longlong2 A = sA[ol], uq = sU[nq.x];
@@ -388,21 +394,49 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
             }
             const double Kr = vq * Gr, Ki = vq * Gi;   // K_t = v_q G
             if (JAC) {
-                skg[2 * i] = make_double2(Kr, Ki);
-                skg[2 * i + 1] = make_double2(Gr, Gi);
-                skp[i] = nq.y;
-                if (!(nq.y & EW_ACCUM)) {
-                    const int4 bm = sbm[ol];
-                    const int pos = bm.x + (nq.y & EW_KMASK), d = bm.y;
-                    jst[pos] = Ki;           // J11 = Re(-j K)
-                    jst[pos + d] = Gr;       // J12
-                    jst[L + pos] = neg(Kr);  // J21 = Im(-j K)
-                    jst[L + pos + d] = Gi;   // J22
-                }
+                runs |= nq.y;
+                const int4 bm = sbm[ol];
+                const int pos = bm.x + (nq.y & EW_KMASK), d = bm.y;
+                jst[pos] = Ki;           // J11 = Re(-j K)
+                jst[pos + d] = Gr;       // J12
+                jst[L + pos] = neg(Kr);  // J21 = Im(-j K)
+                jst[L + pos + d] = Gi;   // J22
             } else {
                 skg[i] = make_double2(Kr, Ki);
             }
         }
+        // the later branches of parallel runs, in their order, onto the entries
+        // that this thread wrote (apart from the loop above, which has no
+        // registers to spare for them)
+        if (JAC && !YBUS && (runs & EW_MORE))
+            for (int i = tid; i < nt; i += TB) {
+                int p = t0 + i;
+                const int2 f = a.tloc[p];
+                if ((f.y & EW_ACCUM) || !(f.y & EW_MORE)) continue;
+                const int o = a.town[p] - b0;
+                const longlong2 A = sA[o], uq = sU[f.x];
+                const double vo = sW[o].x, vq = sW[f.x].x;
+                const int4 bm = sbm[o];
+                double *e = jst + bm.x + (f.y & EW_KMASK);
+                int more;
+                do {
+                    ++p;
+                    const longlong2 y = a.tcfx[p];
+                    const int ye = a.tce[p];
+                    more = a.tloc[p].y & EW_MORE;
+                    double Gr, Gi;
+                    if (A.x == kFixNaN || uq.x == kFixNaN || ye == 0 ||
+                        !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, y.x, y.y, ye, &Gr, &Gi)) {
+                        const longlong2 uo = sU[o];
+                        const double2 yc = a.tcoup[p];
+                        fix_G(A.x, A.y, vo, uo.x, uo.y, uq.x, uq.y, 0, 0, 0, yc.x, yc.y, &Gr, &Gi);
+                    }
+                    e[0] += vq * Gi;
+                    e[bm.y] += Gr;
+                    e[L] -= vq * Gr;
+                    e[L + bm.y] += Gi;
+                } while (more);
+            }
         __syncthreads();
         PF_PROBE_MARK(2);
 
@@ -415,37 +449,23 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
             // depend on them only; the arithmetic is uniform across the pair (no
             // divergence), and with the buses taken by decreasing terminal count
             // the lanes of a warp loop about equally long
-            const double *kg = reinterpret_cast<const double *>(skg);   // K.x, K.y, G.x, G.y per terminal
             for (int x = tid; x < 2 * nbus; x += TB) {
                 const int b = sord[x >> 1], im = x & 1;
                 const int4 bm = sbm[b];
-                const int tend = b + 1 < nbus ? sbm[b + 1].w : nt;
-                const int d = bm.y;
-                // the sum starts from the first terminal (which starts its
-                // parallel run, so it is never EW_ACCUM): one addition fewer
-                int i = bm.w;
-                double sK = 0.0;
-                if (i < tend) sK = kg[4 * i++ + im];
-                for (; i < tend; ++i) {
-                    sK += kg[4 * i + im];
-                    const int kp = skp[i];
-                    if (!YBUS && (kp & EW_ACCUM)) {   // later branch of a parallel run: add into the run's slot
-                        const int pos = bm.x + (kp & EW_KMASK);
-                        if (im) {
-                            jst[pos] += kg[4 * i + 1];           // J11 += Re(-j K)
-                            jst[L + pos + d] += kg[4 * i + 3];   // J22 += Im G
-                        } else {
-                            jst[pos + d] += kg[4 * i + 2];       // J12 += Re G
-                            jst[L + pos] -= kg[4 * i];           // J21 += Im(-j K)
-                        }
-                    }
-                }
-                const double2 vy = syd[b], vw = sW[b];   // v conj(Yd); v, 1/v
-                const double vc = im ? vy.y : vy.x;
                 if (YBUS && bm.z < 0) {   // below
                     slow_row = true;
                     continue;
                 }
+                const int d = bm.y;
+                // K along the staged row, past the diagonal; the sum starts from the first entry
+                const double *row = jst + (im ? 0 : L) + bm.x;
+                double sK = 0.0;
+                if (d > 1) sK = row[bm.z == 0];
+#pragma unroll 1
+                for (int k = 1; k < d - 1; ++k) sK += row[k + (k >= bm.z)];
+                sK = neg_if(sK, !im);
+                const double2 vy = syd[b], vw = sW[b];   // v conj(Yd); v, 1/v
+                const double vc = im ? vy.y : vy.x;
                 const int pos = bm.x + bm.z;
                 jst[(im ? 0 : L) + pos] = neg_if(sK, im);                  // Re / Im of j sum K
                 jst[(im ? L : 0) + pos + d] = fma(sK, vw.y, fix_twice(vc));   // 2 v conj(Yd) + sum K / v

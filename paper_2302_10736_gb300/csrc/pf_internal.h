@@ -77,7 +77,8 @@ inline cudaError_t alloc_all(DevArena &a, double **const (&out)[K], const size_t
 
 // ------------------------------------------------ host index structures --
 // Topology-only structures, built once on the host (host_layout.cpp).
-enum : int { EW_ACCUM = 0x40000000, EW_KMASK = 0x3fffffff };
+// flags beside a terminal's slot position: a later branch of a parallel run; followed by one
+enum : int { EW_ACCUM = 0x40000000, EW_MORE = 0x20000000, EW_KMASK = 0x1fffffff };
 
 struct HostTopo {
     int nb = 0, nl = 0, nnz = 0;
@@ -146,14 +147,13 @@ pf_status host_window_branches(const HostTopo &H, const HostEw &E, std::vector<i
 // Shared-memory plan of the element-wise kernels (byte offsets, 16-aligned):
 //   bm  int4    [max_nbus]   per bus {J-slice row offset, row length, diagonal position, first terminal}
 //   yd  double2 [max_nbus]   per bus self sum (the single evaluation's Jacobian: v conj of it)
-//   kg  double2 [2 max_nt]   per terminal K and G (injection kernel: K only)
-//   kp  int     [max_nt]     per terminal slot position | EW_ACCUM (Jacobian kernel)
+//   kg  double2 [max_nt]     per terminal K (without a Jacobian)
 //   jst double  [2 max_L]    the window's J slice (P half, then Q half)
 //   pq  double  [2 pqs]      P then Q of the window, parity-aligned with global memory
 //   ph                       phasor table (below)
 //   ord int     [max_nbus]   the reduction's thread-to-bus map (HostEw::rorder)      (max_nph > 0)
 struct EwSmem {
-    uint32_t bm, yd, kg, kp, jst, pq, pqs, ph, ord, total;
+    uint32_t bm, yd, kg, jst, pq, pqs, ph, ord, total;
 };
 // max_nph > 0 (the single-evaluation kernel) adds a phasor table of that many
 // slots: V of the own buses in block floating point and 2^62 (cos, sin), each
@@ -165,8 +165,7 @@ __host__ __device__ inline EwSmem ew_smem_plan(int max_nbus, int max_nt, int max
     p.bm = 0;
     p.yd = p.bm + 16u * (uint32_t)max_nbus;
     p.kg = p.yd + 16u * (uint32_t)max_nbus;
-    p.kp = p.kg + (jac ? 32u : 16u) * (uint32_t)max_nt;
-    p.jst = p.kp + (jac ? ((4u * (uint32_t)max_nt + 15u) & ~15u) : 0u);
+    p.jst = p.kg + (jac ? 0u : 16u * (uint32_t)max_nt);   // a Jacobian's K are summed from its staged rows
     p.pq = p.jst + (jac ? 16u * (uint32_t)max_L : 0u);
     p.ph = p.pq + 16u * p.pqs;
     p.ord = p.ph + 48u * (uint32_t)max_nph;
@@ -181,6 +180,33 @@ constexpr uint32_t kTrigSmem = kITrigN * (uint32_t)sizeof(ITrig);
 // own lines, and the loss total's arrival count (k_batched.cu) on a fourth
 constexpr int kBarWords = 128;
 constexpr int kLossCountWord = 96;
+
+// Shared memory of the batched Jacobian and injection kernel (k_ewb): bus
+// records, self sums, phasors and reduction order of the window's own buses,
+// phasors of its own and ghost buses, the J slices (injections alone: K of
+// every terminal), P and Q, the sine/cosine table.
+struct EwbSmem {
+    uint32_t bm, yd, A, U, v, iv, ord, K, jst, pq, pqs, tab, total;
+};
+__host__ __device__ inline EwbSmem ewb_smem_plan(int max_nbus, int max_nt, int max_L, int max_nph, bool jac)
+{
+    EwbSmem p;
+    const uint32_t nbus = (uint32_t)max_nbus, nph = (uint32_t)max_nph;
+    p.pqs = (nbus + 3u) & ~1u;   // even, >= max_nbus + 2
+    p.bm = 0;
+    p.yd = p.bm + 16u * nbus;
+    p.A = p.yd + 16u * nbus;
+    p.U = p.A + 16u * nbus;
+    p.v = p.U + 16u * nph;
+    p.iv = p.v + ((8u * nph + 15u) & ~15u);
+    p.ord = p.iv + (jac ? (8u * nbus + 15u) & ~15u : 0u);
+    p.K = p.ord + ((4u * nbus + 15u) & ~15u);
+    p.jst = p.K + (jac ? 0u : 16u * (uint32_t)max_nt);
+    p.pq = p.jst + (jac ? 16u * (uint32_t)max_L : 0u);
+    p.tab = p.pq + 16u * p.pqs;
+    p.total = p.tab + kTrigSmem;
+    return p;
+}
 
 // Shared memory of the small-batch adjoint (k_adj1, one item per CTA): bus
 // metadata and self sums, both flows of every terminal and its two phasor

@@ -154,6 +154,36 @@ __device__ __forceinline__ bool grid_barrier(const GridBar &b, unsigned int *sta
     return s_ok != 0;
 }
 
+// The barrier's arrival alone, for cooperative kernels without a phase that needs
+// it: every CTA arrives as it starts, thread 0 of CTA 0 looks as it ends whether
+// all have (by then they have, so it does not wait).  Broken barrier state is so
+// reported as by the kernels that wait.
+__device__ __forceinline__ unsigned int grid_arrive(const GridBar &b)
+{
+    unsigned int arrived = 0u;
+    if (threadIdx.x == 0)
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(b.cnt) : "memory");
+    return arrived;
+}
+
+__device__ __forceinline__ void grid_arrive_end(const GridBar &b, unsigned int arrived, unsigned int *state,
+                                                unsigned int nblocks, int *err, int timeout_code, uint64_t limit_ns)
+{
+    if (threadIdx.x != 0) return;
+    if (arrived + 1u == nblocks) *(volatile unsigned int *)state = b.parity ^ 1u;   // every CTA has read the parity
+    if (blockIdx.x != 0) return;
+    const uint64_t t0 = global_timer_ns();
+    for (;;) {
+        unsigned int c;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(b.cnt) : "memory");
+        if ((int)(c - nblocks) >= 0) break;
+        if (global_timer_ns() - t0 > limit_ns) {
+            atomicExch(err, timeout_code);
+            break;
+        }
+    }
+}
+
 // programmatic dependent launch: let the next kernel in the stream start its
 // prologue now / wait until the previous kernel's results are visible
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
