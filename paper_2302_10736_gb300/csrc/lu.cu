@@ -350,8 +350,9 @@ struct MfGroup {
     {
         if (NC > 1)
             for (int q = 0; q < NC; ++q) {
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rrow[q]) : "r"(smem_addr(row)), "r"(q));
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar[q]) : "r"(smem_addr(bar)), "r"(q));
+                const int to = (rank + 1 + q) % NC;   // the CTA that owns the next row first
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rrow[q]) : "r"(smem_addr(row)), "r"(to));
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar[q]) : "r"(smem_addr(bar)), "r"(to));
             }
     }
 
@@ -523,7 +524,8 @@ __device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr
         }
     mf_slots<NC, C2>(g, 0, min(p, rows));
     double m[R][C2];
-    constexpr int G = R * C2 % 4 == 0 ? 4 : 3;   // elements at a time
+    constexpr int G = R * C2 % 4 == 0 ? 4 : R * C2 % 3 == 0 ? 3 : 2;   // elements at a time
+    static_assert(R * C2 % G == 0);
     uint32_t rest = 0;
 #pragma unroll
     for (int t = 0; t < R * C2; t += G) {
@@ -618,7 +620,15 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
     for (int s; (s = mf_next(a, 2, g, &s_next)) >= 0;)
         for (;;) {
             const MfFront fr = a.fr[s];
-            if (fr.f < 128)
+            // the owner's chain takes and scales every column block it is compiled
+            // for: with 4 blocks for all fronts below 128 unknowns this kernel took
+            // 140 us at 10,000 buses and 316 at 25,000, with 2, 3 and 4 (and rows sent
+            // to the next row's CTA first) 105 and 279
+            if (fr.f < 64)
+                mf_tile_front<kMfWideCtas, NW, 1, 2>(a, fr, g, (int)(kMfWideRowBytes / 512));
+            else if (fr.f < 96)
+                mf_tile_front<kMfWideCtas, NW, 2, 3>(a, fr, g, (int)(kMfWideRowBytes / 768));
+            else if (fr.f < 128)
                 mf_tile_front<kMfWideCtas, NW, 2, 4>(a, fr, g, (int)(kMfWideRowBytes / 1024));
             else if (fr.f < 192)
                 mf_tile_front<kMfWideCtas, NW, 3, 6>(a, fr, g, (int)(kMfWideRowBytes / 1536));
