@@ -373,6 +373,7 @@ PF_API void grid_destroy(pf_grid *grid)
     if (!grid) return;
     trace_free(&grid->g);
     grid->g.arena.free_all();
+    if (grid->g.nt_res) cudaFreeHost(grid->g.nt_res);
     delete grid;
 }
 

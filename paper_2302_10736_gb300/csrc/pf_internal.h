@@ -264,6 +264,12 @@ struct alignas(16) MfFront {
     long long m0, pad2;                // place in global memory (the last class)
 };
 
+// what the Newton loop reads of an iteration: the bits of max |F|, the error word
+struct NewtonResult {
+    unsigned long long bits;
+    int err;
+};
+
 struct Grid {
     int nb = 0, nl = 0, nnz = 0;
     pf_config cfg{};
@@ -339,7 +345,8 @@ struct Grid {
     std::vector<int> red_h_colptr, red_h_rowidx, red_h_fmap;
     // Newton-Raphson workspace (powerflow_newton): F, J_r (CSC), step, max |F|
     double *nt_F = nullptr, *nt_J = nullptr, *nt_dx = nullptr;
-    unsigned long long *nt_max = nullptr;
+    unsigned long long *nt_max = nullptr;   // {running max |F|, CTAs done}
+    NewtonResult *nt_res = nullptr;         // page-locked host memory
     // sparse LU of the reduced system (lu.cu): the plan of the current bus types
     // (HostLu), its pivot rows, updates, solution and counters
     int lu_ready = 0, lu_n = 0, lu_nf = 0, lu_backmax = 0, lu_bigp = 0;
