@@ -47,12 +47,13 @@
 // k_mf_back_small: the backward solve; a CTA or warp follows one heavy path of the
 // tree down and waits (bounded) only at its head.
 //
-// One solve (CUDA-profiled kernels, us): 2,000 buses 378 -> 172, 10,000 962 -> 350,
-// 25,000 1,752 -> 560, 70,000 3,111 -> 937, against a left-looking factorization
+// One solve (CUDA-profiled kernels, us): 2,000 buses 378 -> 160, 10,000 962 -> 300,
+// 25,000 1,752 -> 490, 70,000 3,111 -> 857, against a left-looking factorization
 // by columns whose every level cost a chain of L2 round trips, with the top of the
 // tree as one dense block of a cluster and an FP64 reciprocal in each of its warps.
-// Of the 560 us at 25,000 buses, small 34, mid 88, wide 295 (0.75 us per pivot row
-// of the top ten fronts), backward 130.
+// Of the 300 us at 10,000 buses, small 19, mid 108 (4.5 us a level of the tree, of
+// which the update's way to the parent through L2, by atomic and back, is half),
+// wide 105, backward 64.
 //
 // Every sum has a fixed order (children in order of their pivots, lane-strided
 // partial sums joined by a fixed shuffle tree): the results are bitwise
@@ -79,8 +80,9 @@ constexpr int kMfSmallLd = 13;        // row stride of a small front (odd: no ba
 constexpr int kMfSmallWarps = 16;     // warps per CTA of k_mf_small and k_mf_back_small
 constexpr int kMfMidWarps = 8;        // warps per CTA of the second class
 constexpr int kMfWideWarps = 8, kMfWideCtas = 8;           // of the third
+constexpr int kMfBackSmall = kMfSmall * kMfSmall + kMfSmall;   // doubles of a small front's pivot rows and y
 constexpr int kMfHugeThreads = 512, kMfBackThreads = 512;
-constexpr int kMfBackRows = 160;      // most pivots of a front whose pivot block the backward solve copies to shared memory
+constexpr int kMfBackRows = 160;      // in the limit on the largest front (back_smem)
 constexpr int kMfMidRows = kMfMid;    // pivot rows kept in shared memory at a time: all of a front of the second class
 constexpr size_t kMfWideRowBytes = 200u * 1024u;           // ... and what fits, of the third
 constexpr size_t kMfMaxSmem = 220u * 1024u;
@@ -88,6 +90,7 @@ constexpr size_t kMfMaxSmem = 220u * 1024u;
 struct MfArgs {
     int n, nf, nnzA;
     int backmax;            // unknowns of the largest front but the small ones
+    int backp, backw;       // its pivots in whole warps; doubles of the backward solve's copies of U
     int nleaf[kMfClasses];  // fronts without children of their class
     int npath[2];           // backward paths of the small fronts, of the others
     const MfFront *fr;
@@ -96,6 +99,7 @@ struct MfArgs {
     const int2 *el;         // per element of a front: {its first source (mf_source; kMfNone), its further ones in ext (-1: none)}
     const int4 *ext;        // {how many, the first three}, then the others
     const int *bidx;        // per border unknown: its number
+    const int *rel;         // ... and its place in the parent (pivots, border)
     const int *perm;        // unknown -> reduced index
     const double *A, *F;
     double *U, *cb, *x, *dx, *mat;   // pivot rows and y; updates; solution; fronts beyond shared memory
@@ -694,84 +698,118 @@ __global__ void __launch_bounds__(kMfHugeThreads) k_mf_huge(MfArgs a)
 // ------------------------------------------------------ backward solve ----
 
 // The other fronts: x_p of the fronts of one path, from its head down, by one CTA.
-// t = y - U_pr x_r (a warp per row), then U_pp x_p = t (unit diagonal) from the
-// bottom in blocks of 32 rows: a block's triangle by one warp (a lane per row), its
-// terms out of the rows above by a thread per row.  U_pp is copied to shared
-// memory before the wait.
+// t = y - U_pr x_r (a thread per row and quarter of the border), then U_pp x_p = t
+// (unit diagonal) from the bottom in blocks of 32 rows: a block's triangle by one
+// warp (a lane per row), its terms out of the rows above by a thread per row.
+// The chain from front to front is what counts: a front's x stays in shared memory,
+// where the next front of the path finds its border (a child's border is among its
+// parent's pivots and border), and that front's pivot rows are copied there while
+// the triangle is solved, by the other warps (before the wait, for a path's head).
+// The border's products by a warp per row, each with a shuffle tree of 5 additions
+// (FP64 instructions like the products), and every load behind the front before
+// took 65 us at 10,000 buses and 192 at 70,000; so 44 and 138 (the small fronts, by
+// the same means, 24 -> 20 and 38 -> 32).
 __global__ void __launch_bounds__(kMfBackThreads) k_mf_back_big(MfArgs a)
 {
     extern __shared__ __align__(16) double msm[];
     __shared__ int s_next, s_ok;
-    // the border's x, the pivots' right-hand side, U_pp (of at most kMfBackRows pivots)
-    double *xr = msm, *tv = msm + a.backmax, *T = tv + a.backmax;
+    // x of the front (pivots, border) and of the one before; partial sums; pivot rows and y
+    double *const sp = msm + 2 * a.backmax, *const Wm = sp + 4 * a.backp;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     constexpr int TB = kMfBackThreads, nw = TB / 32;
     int *next = a.cnt + 2 * a.nf + kMfClasses + 1, *done = a.cnt + a.nf;
+    auto room = [](const MfFront &f) { return f.p * (f.f | 1) + f.p; };   // doubles of its copy
+    auto stage = [&](const MfFront &f, double *W, int w0, int w1) {   // by warps w0 .. w1 - 1
+        const int ld = f.f | 1;
+        const double *U = a.U + f.u0;
+        for (int i = wid - w0; i < f.p; i += w1 - w0)
+            for (int j = i + 1 + lane; j < f.f; j += 32) cp_async8(W + i * ld + j, U + (size_t)i * f.f + j);
+        for (int i = tid - 32 * w0; i < f.p; i += 32 * (w1 - w0)) cp_async8(W + f.p * ld + i, U + (size_t)f.p * f.f + i);
+    };
     for (;;) {
         if (tid == 0) s_next = atomicAdd(next, 1);
         __syncthreads();
         const int t = s_next;
         __syncthreads();
         if (t >= a.npath[1]) break;
-        int s = a.path[1][t];
-        bool head = true;
-        while (s >= 0) {
-            const MfFront fr = a.fr[s];
-            const int p = fr.p, f = fr.f, r = f - p, ldt = p | 1;
-            const double *U = a.U + fr.u0;
-            const bool whole = p <= kMfBackRows;
-            const int bj = tid < r ? a.bidx[fr.b0 + tid] : 0;
-            if (whole)
-                for (int i = wid; i < p; i += nw)
-                    for (int j = i + 1 + lane; j < p; j += 32) T[i * ldt + j] = U[(size_t)i * f + j];
-            if (head && fr.wait) {
-                if (tid == 0) s_ok = mf_wait(a, done + fr.parent);
-                __syncthreads();
-                if (!s_ok) return;
+        int s = a.path[1][t], cur = 0;
+        MfFront fr = a.fr[s];
+        bool head = true, staged = false;   // staged: its copy was begun with the front before
+        double *W = Wm;
+        int rl = 0;   // the place of the thread's first border unknown
+        for (;;) {
+            const int p = fr.p, f = fr.f, r = f - p, own = room(fr);
+            const bool in = own <= a.backw;
+            if (!staged) {
+                W = Wm;
+                if (in) stage(fr, W, 0, nw);
             }
-            head = false;
-            for (int j = tid; j < r; j += TB) xr[j] = __ldcg(a.x + (j == tid ? bj : a.bidx[fr.b0 + j]));
+            // the next front, of which nothing is used before this one's border products
+            const MfFront nx = a.fr[fr.heavy >= 0 ? fr.heavy : s];
+            double *X = msm + cur * a.backmax;
+            const double *Xp = msm + (cur ^ 1) * a.backmax;
+            if (head) {
+                const int bj = tid < r ? a.bidx[fr.b0 + tid] : 0;
+                if (fr.wait) {
+                    if (tid == 0) s_ok = mf_wait(a, done + fr.parent);
+                    __syncthreads();
+                    if (!s_ok) {
+                        cp_async_wait_all();
+                        return;
+                    }
+                }
+                for (int j = tid; j < r; j += TB) X[p + j] = __ldcg(a.x + (j == tid ? bj : a.bidx[fr.b0 + j]));
+            } else {
+                for (int j = tid; j < r; j += TB) X[p + j] = Xp[j == tid ? rl : a.rel[fr.b0 + j]];
+            }
+            cp_async_wait_all();
             __syncthreads();
-            for (int i = wid; i < p; i += 2 * nw) {   // two rows at a time
-                const int i2 = i + nw < p ? i + nw : i;
-                double s0 = 0.0, s1 = 0.0;
-#pragma unroll 2
-                for (int j = lane; j < r; j += 32) {
-                    const double x = xr[j];
-                    s0 = fma(U[(size_t)i * f + p + j], x, s0);
-                    s1 = fma(U[(size_t)i2 * f + p + j], x, s1);
-                }
-                s0 = warp_sum_d(s0);
-                s1 = warp_sum_d(s1);
-                if (lane == 0) {
-                    tv[i] = U[(size_t)p * f + i] - s0;
-                    if (i2 != i) tv[i2] = U[(size_t)p * f + i2] - s1;
-                }
+            const double *T = in ? W : a.U + fr.u0;
+            const int ld = in ? f | 1 : f;
+            for (int u = wid; u < (p + 31) / 32 * 4; u += nw) {
+                const int i = (u >> 2) * 32 + lane;
+                double sum = 0.0;
+                if (i < p)
+#pragma unroll 4
+                    for (int j = u & 3; j < r; j += 4) sum = fma(T[(size_t)i * ld + p + j], X[p + j], sum);
+                sp[32 * u + lane] = sum;
+            }
+            __syncthreads();
+            // the next front's copy at the other end of the room, if both fit
+            const bool ahead = fr.heavy >= 0 && own + room(nx) <= a.backw;
+            double *const Wn = W == Wm ? Wm + (a.backw - room(nx)) : Wm;
+            if (ahead && wid > 0) stage(nx, Wn, 1, nw);
+            rl = fr.heavy >= 0 && tid < nx.f - nx.p ? a.rel[nx.b0 + tid] : 0;
+            for (int i = tid; i < p; i += TB) {
+                const double *q = sp + 128 * (i >> 5) + (i & 31);
+                X[i] = T[(size_t)p * ld + i] - ((q[0] + q[32]) + (q[64] + q[96]));
             }
             __syncthreads();
             for (int b1 = p; b1 > 0; b1 -= 32) {
                 const int b0 = b1 > 32 ? b1 - 32 : 0, w = b1 - b0;
                 if (wid == 0) {
-                    const double *Ti = whole ? T + (size_t)(b0 + lane) * ldt + b0 : U + (size_t)(b0 + lane) * f + b0;
-                    double x = lane < w ? tv[b0 + lane] : 0.0;
+                    const double *Ti = T + (size_t)(b0 + min(lane, w - 1)) * ld + b0;
+                    double x = lane < w ? X[b0 + lane] : 0.0;
+#pragma unroll 4
                     for (int k = w - 1; k > 0; --k) {
                         const double uk = lane < k ? Ti[k] : 0.0;
                         const double xk = __shfl_sync(0xffffffffu, x, k);
                         if (lane < k) x = fma(-uk, xk, x);
                     }
                     if (lane < w) {
-                        tv[b0 + lane] = x;
+                        X[b0 + lane] = x;
                         a.x[fr.e0 + b0 + lane] = x;
                         a.dx[a.perm[fr.e0 + b0 + lane]] = x;
                     }
                 }
                 __syncthreads();
+                if (b0 == 0) break;
                 for (int i = tid; i < b0; i += TB) {
-                    const double *Ti = whole ? T + (size_t)i * ldt + b0 : U + (size_t)i * f + b0;
-                    double y = tv[i];
+                    const double *Ti = T + (size_t)i * ld + b0;
+                    double y = X[i];
 #pragma unroll 4
-                    for (int k = 0; k < w; ++k) y = fma(-Ti[k], tv[b0 + k], y);
-                    tv[i] = y;
+                    for (int k = 0; k < w; ++k) y = fma(-Ti[k], X[b0 + k], y);
+                    X[i] = y;
                 }
                 __syncthreads();
             }
@@ -779,38 +817,52 @@ __global__ void __launch_bounds__(kMfBackThreads) k_mf_back_big(MfArgs a)
                 __threadfence();
                 atomicExch(done + s, 1);
             }
+            if (fr.heavy < 0) break;
             s = fr.heavy;
+            fr = nx;
+            cur ^= 1;
+            head = false;
+            staged = ahead;
+            if (ahead) W = Wn;
         }
     }
 }
 
 // Small fronts: the same by one warp; the lanes are (row, part) pairs that split
-// the row's border terms, joined by a shuffle tree.  What does not depend on the
-// fronts above is loaded before the wait.
+// the row's border terms, joined by a shuffle tree.  The path's next front is
+// loaded while this one is solved, its border's x come from this one's lanes.
 __global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_back_small(MfArgs a)
 {
     extern __shared__ __align__(16) double msm[];
     const int lane = threadIdx.x & 31;
-    double *W = msm + (size_t)(threadIdx.x >> 5) * (kMfSmall * kMfSmall + kMfSmall);   // pivot rows and y
+    double *const Wm = msm + (size_t)(threadIdx.x >> 5) * (2 * kMfBackSmall);   // pivot rows and y of two fronts
     int *next = a.cnt + 2 * a.nf + kMfClasses, *done = a.cnt + a.nf;
+    auto stage = [&](const MfFront &f, double *W) {
+        for (int q = lane; q < f.p * f.f + f.p; q += 32) cp_async8(W + q, a.U + f.u0 + q);
+    };
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(next, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= a.npath[0]) break;
         int s = a.path[0][t];
-        bool head = true;
-        while (s >= 0) {
-            const MfFront fr = a.fr[s];
+        MfFront fr = a.fr[s];
+        double *W = Wm;
+        stage(fr, W);
+        const int bj = lane < fr.f - fr.p ? a.bidx[fr.b0 + lane] : 0;
+        int pm = lane < fr.p ? a.perm[fr.e0 + lane] : 0;
+        // the head of a path waits for its parent unless an earlier launch wrote it
+        if (fr.wait && !__all_sync(0xffffffffu, mf_wait(a, done + fr.parent))) {
+            cp_async_wait_all();
+            return;
+        }
+        __syncwarp();
+        double xb = lane < fr.f - fr.p ? __ldcg(a.x + bj) : 0.0;
+        for (;;) {
             const int p = fr.p, f = fr.f, r = f - p;
-            for (int q = lane; q < p * f + p; q += 32) W[q] = a.U[fr.u0 + q];
-            const int bj = lane < r ? a.bidx[fr.b0 + lane] : 0;
-            const int pm = lane < p ? a.perm[fr.e0 + lane] : 0;
-            // the head of a path waits for its parent unless an earlier launch wrote it
-            if (head && fr.wait && !__all_sync(0xffffffffu, mf_wait(a, done + fr.parent))) return;
-            head = false;
+            const MfFront nx = a.fr[fr.heavy >= 0 ? fr.heavy : s];
+            cp_async_wait_all();
             __syncwarp();
-            const double xb = lane < r ? __ldcg(a.x + bj) : 0.0;
             // lane = row i + p2 * part g
             const int p2 = p <= 1 ? 1 : 1 << (32 - __clz(p - 1)), g = lane / p2, i = lane & (p2 - 1), ng = 32 / p2;
             double sum = 0.0;
@@ -820,6 +872,13 @@ __global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_back_small(MfArgs a)
                 if (j < r && i < p) sum = fma(W[i * f + p + j], xj, sum);
             }
             for (int off = p2; off < 32; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            double *const Wn = W == Wm ? Wm + kMfBackSmall : Wm;
+            int rl = 0, pn = 0;
+            if (fr.heavy >= 0) {
+                stage(nx, Wn);
+                rl = lane < nx.f - nx.p ? a.rel[nx.b0 + lane] : 0;
+                pn = lane < nx.p ? a.perm[nx.e0 + lane] : 0;
+            }
             double x = 0.0;
             if (i < p) x = W[p * f + i] - sum;
             for (int k = p - 1; k > 0; --k) {
@@ -835,7 +894,14 @@ __global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_back_small(MfArgs a)
                 __threadfence();
                 atomicExch(done + s, 1);
             }
+            if (fr.heavy < 0) break;
+            // a border unknown of the next front is a pivot or border unknown of this one
+            const double u = __shfl_sync(0xffffffffu, x, rl & 31), v = __shfl_sync(0xffffffffu, xb, (rl - p) & 31);
+            xb = rl < p ? u : v;
             s = fr.heavy;
+            fr = nx;
+            pm = pn;
+            W = Wn;
         }
     }
 }
@@ -1109,7 +1175,8 @@ pf_status host_lu(int nb, int n, int npvpq, const std::vector<int> &colptr, cons
         return f.p + (int)(std::lower_bound(b, e, x) - b);
     };
     // the place of every border unknown in the parent (both borders ascend)
-    std::vector<int> rel(std::max<long long>(b0, 1), 0);
+    std::vector<int> &rel = L.rel;
+    rel.assign(std::max<long long>(b0, 1), 0);
     std::vector<std::vector<int>> kids(nf);
     for (int s = 0; s < nf; ++s) {
         const MfFront &f = L.fr[s];
@@ -1227,11 +1294,24 @@ pf_status host_lu(int nb, int n, int npvpq, const std::vector<int> &colptr, cons
     return PF_OK;
 }
 
-// shared memory of the backward solve
+// the limit on a front: the shared memory of its x and pivot block
 static size_t back_smem(int fmax, int pmax)
 {
     const size_t p = (size_t)std::min(pmax, kMfBackRows);
     return sizeof(double) * (2 * (size_t)fmax + p * (p | 1));
+}
+
+// doubles of the backward solve's copies: what a front and the next of its path
+// take, as far as it fits
+static int back_room(const HostLu &L)
+{
+    auto room = [](const MfFront &f) { return (long long)f.p * (f.f | 1) + f.p; };
+    long long most = 0;
+    for (int h : L.path[1])
+        for (int s = h; s >= 0; s = L.fr[s].heavy)
+            most = std::max(most, room(L.fr[s]) + (L.fr[s].heavy >= 0 ? room(L.fr[L.fr[s].heavy]) : 0));
+    const long long left = (long long)(kMfMaxSmem / sizeof(double)) - 2 * L.backmax - 4 * ((L.bigp + 31) / 32 * 32);
+    return (int)std::max(0LL, std::min(most, left));
 }
 
 // Upload the plan of the grid's current bus types and size its workspace.
@@ -1260,7 +1340,7 @@ pf_status lu_prepare(Grid *g, cudaStream_t s)
     if ((e = up(&g->lu_fr, L.fr)) || (e = up(&g->lu_leaf[0], L.leaf[0])) || (e = up(&g->lu_leaf[1], L.leaf[1])) ||
         (e = up(&g->lu_leaf[2], L.leaf[2])) || (e = up(&g->lu_leaf[3], L.leaf[3])) || (e = up(&g->lu_path[0], L.path[0])) ||
         (e = up(&g->lu_path[1], L.path[1])) || (e = up(&g->lu_el, L.el)) || (e = up(&g->lu_ext, L.ext)) ||
-        (e = up(&g->lu_bidx, L.bidx)) || (e = up(&g->lu_perm, L.perm)) ||
+        (e = up(&g->lu_bidx, L.bidx)) || (e = up(&g->lu_rel, L.rel)) || (e = up(&g->lu_perm, L.perm)) ||
         (e = g->arena.alloc(&g->lu_U, (size_t)std::max<long long>(L.nU, 1))) ||
         (e = g->arena.alloc(&g->lu_cb, (size_t)std::max<long long>(L.nC, 1))) ||
         (e = g->arena.alloc(&g->lu_x, (size_t)std::max(L.n, 1))) ||
@@ -1274,7 +1354,8 @@ pf_status lu_prepare(Grid *g, cudaStream_t s)
     for (int c = 0; c < kMfClasses; ++c) g->lu_nleaf[c] = (int)L.leaf[c].size();
     for (int c = 0; c < 2; ++c) g->lu_npath[c] = (int)L.path[c].size();
     g->lu_backmax = L.backmax;
-    g->lu_bigp = L.bigp;
+    g->lu_backp = (L.bigp + 31) / 32 * 32;
+    g->lu_backw = back_room(L);
     g->lu_ready = 1;
     return PF_OK;
 }
@@ -1283,7 +1364,7 @@ void lu_release(Grid *g)
 {
     for (void *p : {(void *)g->lu_fr, (void *)g->lu_leaf[0], (void *)g->lu_leaf[1], (void *)g->lu_leaf[2], (void *)g->lu_leaf[3],
                     (void *)g->lu_path[0], (void *)g->lu_path[1], (void *)g->lu_el, (void *)g->lu_ext,
-                    (void *)g->lu_bidx, (void *)g->lu_perm, (void *)g->lu_U, (void *)g->lu_cb, (void *)g->lu_x,
+                    (void *)g->lu_bidx, (void *)g->lu_rel, (void *)g->lu_perm, (void *)g->lu_U, (void *)g->lu_cb, (void *)g->lu_x,
                     (void *)g->lu_mat, (void *)g->lu_cnt})
         g->arena.release(p);
     g->lu_fr = nullptr;
@@ -1291,7 +1372,7 @@ void lu_release(Grid *g)
     for (int *&p : g->lu_path) p = nullptr;
     g->lu_el = nullptr;
     g->lu_ext = nullptr;
-    g->lu_bidx = g->lu_perm = g->lu_cnt = nullptr;
+    g->lu_bidx = g->lu_rel = g->lu_perm = g->lu_cnt = nullptr;
     g->lu_U = g->lu_cb = g->lu_x = g->lu_mat = nullptr;
     g->lu_ready = 0;
 }
@@ -1316,6 +1397,9 @@ cudaError_t launch_lu_solve(Grid *g, const double *Jr, const double *F, double *
     a.el = g->lu_el;
     a.ext = g->lu_ext;
     a.bidx = g->lu_bidx;
+    a.rel = g->lu_rel;
+    a.backp = g->lu_backp;
+    a.backw = g->lu_backw;
     a.perm = g->lu_perm;
     a.A = Jr;
     a.F = F;
@@ -1333,9 +1417,9 @@ cudaError_t launch_lu_solve(Grid *g, const double *Jr, const double *F, double *
             return e;
     }
     const size_t sm_small = sizeof(double) * kMfSmallWarps * kMfSmall * kMfSmallLd;
-    const size_t sm_bsmall = sizeof(double) * kMfSmallWarps * (kMfSmall * kMfSmall + kMfSmall);
+    const size_t sm_bsmall = sizeof(double) * kMfSmallWarps * 2 * kMfBackSmall;
     const size_t sm_wide = sizeof(double) * (kMfWide + 1) + kMfWideRowBytes;
-    const size_t sm_bbig = back_smem(g->lu_backmax, g->lu_bigp);
+    const size_t sm_bbig = sizeof(double) * (2 * (size_t)g->lu_backmax + 4 * (size_t)g->lu_backp + g->lu_backw);
     if ((e = ensure_dyn_smem(reinterpret_cast<const void *>(k_mf_wide), sm_wide)) ||
         (e = ensure_dyn_smem(reinterpret_cast<const void *>(k_mf_back_big), sm_bbig)))
         return e;

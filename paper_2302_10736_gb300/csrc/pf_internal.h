@@ -349,13 +349,13 @@ struct Grid {
     NewtonResult *nt_res = nullptr;         // page-locked host memory
     // sparse LU of the reduced system (lu.cu): the plan of the current bus types
     // (HostLu), its pivot rows, updates, solution and counters
-    int lu_ready = 0, lu_n = 0, lu_nf = 0, lu_backmax = 0, lu_bigp = 0;
+    int lu_ready = 0, lu_n = 0, lu_nf = 0, lu_backmax = 0, lu_backp = 0, lu_backw = 0;
     int lu_nleaf[kMfClasses] = {}, lu_npath[2] = {};
     MfFront *lu_fr = nullptr;
     int *lu_leaf[kMfClasses] = {}, *lu_path[2] = {};
     int2 *lu_el = nullptr;
     int4 *lu_ext = nullptr;
-    int *lu_bidx = nullptr, *lu_perm = nullptr, *lu_cnt = nullptr;
+    int *lu_bidx = nullptr, *lu_rel = nullptr, *lu_perm = nullptr, *lu_cnt = nullptr;
     double *lu_U = nullptr, *lu_cb = nullptr, *lu_x = nullptr, *lu_mat = nullptr;
     // tracer: events [2 * capacity], kernel id per record
     std::vector<cudaEvent_t> tr_ev;
@@ -439,7 +439,7 @@ struct HostLu {
     int n = 0, backmax = 0, bigp = 0;
     long long nU = 0, nC = 0;
     std::vector<MfFront> fr;
-    std::vector<int> perm, bidx;
+    std::vector<int> perm, bidx, rel;   // rel: per border unknown, its place in the parent (pivots, border)
     std::vector<int2> el;
     std::vector<int4> ext;
     std::vector<int> leaf[kMfClasses], path[2];

@@ -12,6 +12,13 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)
 // Bring the line of a valid global address into L2 (a hint: no data returned,
 // no ordering; L2 is the point of coherence, so a later load after a
 // programmatic-dependent-launch wait still sees what the previous grid wrote)
+// 8 bytes to shared memory without a register; the thread's copies are done after cp_async_wait_all
+__device__ __forceinline__ void cp_async8(double *smem, const double *gmem)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
