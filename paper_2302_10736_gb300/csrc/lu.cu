@@ -47,11 +47,11 @@
 // k_mf_back_small: the backward solve; a CTA or warp follows one heavy path of the
 // tree down and waits (bounded) only at its head.
 //
-// One solve (CUDA-profiled kernels, us): 2,000 buses 378 -> 160, 10,000 962 -> 300,
+// One solve (CUDA-profiled kernels, us): 2,000 buses 378 -> 155, 10,000 962 -> 293,
 // 25,000 1,752 -> 490, 70,000 3,111 -> 857, against a left-looking factorization
 // by columns whose every level cost a chain of L2 round trips, with the top of the
 // tree as one dense block of a cluster and an FP64 reciprocal in each of its warps.
-// Of the 300 us at 10,000 buses, small 19, mid 108 (4.5 us a level of the tree, of
+// Of the 293 us at 10,000 buses, small 19, mid 101 (4 us a level of the tree, of
 // which the update's way to the parent through L2, by atomic and back, is half),
 // wide 105, backward 64.
 //
@@ -511,14 +511,11 @@ __device__ __forceinline__ void mf_pivots(const MfArgs &a, const MfFront &fr, Mf
         if (p > K0 + N) mf_pivots<NC, NW, R, C2, K0 + N>(a, fr, g, rows, kb, m);
 }
 
-template <int NC, int NW, int R, int C2>
-__device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr, MfGroup<NC> &g, int rows)
+// the plan of the thread's elements of a front
+template <int NW, int R, int C2>
+__device__ __forceinline__ void mf_plan(const MfArgs &a, const MfFront &fr, int gw, int2 *e)
 {
-    const int p = fr.p, f = fr.f, w = f + 1, r = f - p;
-    const int lane = threadIdx.x & 31, gw = g.gw;
-    // ---- the front's elements: their plan while the slots are made ready, then
-    // their sources, a few at a time ----
-    int2 e[R * C2];
+    const int f = fr.f, w = f + 1, lane = threadIdx.x & 31;
 #pragma unroll
     for (int q = 0; q < R; ++q)
 #pragma unroll
@@ -526,6 +523,18 @@ __device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr
             const int i = gw + NW * q, j = 32 * c + lane;
             e[q * C2 + c] = i < f && j < w ? a.el[fr.s0 + i * w + j] : make_int2(kMfNone, -1);
         }
+}
+
+// a front from its plan e to its update and pivot rows; `nx`, with which the group
+// may go on, is loaded on the way
+template <int NC, int NW, int R, int C2>
+__device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr, MfGroup<NC> &g, int rows,
+                                              const int2 *e, MfFront &nx)
+{
+    const int p = fr.p, f = fr.f, r = f - p;
+    const int lane = threadIdx.x & 31, gw = g.gw;
+    // ---- the front's elements: their sources, a few at a time, while the slots
+    // are made ready ----
     mf_slots<NC, C2>(g, 0, min(p, rows));
     double m[R][C2];
     constexpr int G = R * C2 % 4 == 0 ? 4 : R * C2 % 3 == 0 ? 3 : 2;   // elements at a time
@@ -549,6 +558,7 @@ __device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr
             if (rest >> t & 1) m[t / C2][t % C2] = mf_gather_rest(a, e[t].y, m[t / C2][t % C2]);
     int kb = 0;   // first row of the batch
     mf_pivots<NC, NW, R, C2, 0>(a, fr, g, rows, kb, m);
+    if (fr.parent_need > 0) nx = a.fr[fr.parent];
     // ---- the update ----
 #pragma unroll
     for (int q = 0; q < R; ++q) {
@@ -599,16 +609,39 @@ __global__ void __launch_bounds__(32 * kMfMidWarps, 2) k_mf_mid(MfArgs a)
     __shared__ uint64_t bar[kMfMidRows];
     __shared__ int s_next;
     MfGroup<1> g(bar, row, 0, (int)threadIdx.x >> 5);
-    for (int s; (s = mf_next(a, 1, g, &s_next)) >= 0;)
-        for (;;) {
-            const MfFront fr = a.fr[s];
-            if (fr.f < 32)
-                mf_tile_front<1, kMfMidWarps, 4, 1>(a, fr, g, kMfMidRows);
+    for (int s; (s = mf_next(a, 1, g, &s_next)) >= 0;) {
+        MfFront fr = a.fr[s], nx = fr;
+        // a front's plan; the parent's is in flight while this CTA counts itself there
+        // (k_mf_mid 90 -> 85 us at 2,000 buses, 108 -> 101 at 10,000)
+        int2 e[16];
+        auto plan = [&](const MfFront &x) {
+            if (x.f < 32)
+                mf_plan<kMfMidWarps, 4, 1>(a, x, g.gw, e);
             else
-                mf_tile_front<1, kMfMidWarps, 8, 2>(a, fr, g, kMfMidRows);
-            if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
-            s = fr.parent;
+                mf_plan<kMfMidWarps, 8, 2>(a, x, g.gw, e);
+        };
+        plan(fr);
+        for (;;) {
+            if (fr.f < 32)
+                mf_tile_front<1, kMfMidWarps, 4, 1>(a, fr, g, kMfMidRows, e, nx);
+            else
+                mf_tile_front<1, kMfMidWarps, 8, 2>(a, fr, g, kMfMidRows, e, nx);
+            if (fr.parent_need == 0) break;
+            plan(nx);
+            if (!mf_climb(a, fr, g, &s_next)) break;
+            fr = nx;
         }
+    }
+}
+
+template <int R, int C2>
+__device__ __forceinline__ void mf_wide_front(const MfArgs &a, const MfFront &fr, MfGroup<kMfWideCtas> &g)
+{
+    constexpr int NW = kMfWideWarps * kMfWideCtas;
+    int2 e[R * C2];
+    MfFront nx;
+    mf_plan<NW, R, C2>(a, fr, g.gw, e);
+    mf_tile_front<kMfWideCtas, NW, R, C2>(a, fr, g, (int)(kMfWideRowBytes / (256 * C2)), e, nx);
 }
 
 __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWideWarps, 1) k_mf_wide(MfArgs a)
@@ -617,7 +650,6 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
     __shared__ int s_next;
     uint32_t rank;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    constexpr int NW = kMfWideWarps * kMfWideCtas;
     // consecutive rows on different SMs
     MfGroup<kMfWideCtas> g(reinterpret_cast<uint64_t *>(msm), msm + (kMfWide + 1), (int)rank,
                            ((int)threadIdx.x >> 5) * kMfWideCtas + (int)rank);
@@ -629,15 +661,15 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
             // 140 us at 10,000 buses and 316 at 25,000, with 2, 3 and 4 (and rows sent
             // to the next row's CTA first) 105 and 279
             if (fr.f < 64)
-                mf_tile_front<kMfWideCtas, NW, 1, 2>(a, fr, g, (int)(kMfWideRowBytes / 512));
+                mf_wide_front<1, 2>(a, fr, g);
             else if (fr.f < 96)
-                mf_tile_front<kMfWideCtas, NW, 2, 3>(a, fr, g, (int)(kMfWideRowBytes / 768));
+                mf_wide_front<2, 3>(a, fr, g);
             else if (fr.f < 128)
-                mf_tile_front<kMfWideCtas, NW, 2, 4>(a, fr, g, (int)(kMfWideRowBytes / 1024));
+                mf_wide_front<2, 4>(a, fr, g);
             else if (fr.f < 192)
-                mf_tile_front<kMfWideCtas, NW, 3, 6>(a, fr, g, (int)(kMfWideRowBytes / 1536));
+                mf_wide_front<3, 6>(a, fr, g);
             else
-                mf_tile_front<kMfWideCtas, NW, 4, 8>(a, fr, g, (int)(kMfWideRowBytes / 2048));
+                mf_wide_front<4, 8>(a, fr, g);
             if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
             s = fr.parent;
         }
