@@ -212,9 +212,12 @@ static pf_status ew_fits(const HostEw &E, size_t *smem)
 {
     const EwSmem plan = ew_smem_plan(E.max_nbus, E.max_nt, E.max_L, true, E.max_nph);
     *smem = plan.total + kTrigSmem;
-    if (*smem > kMaxSmem)
+    // the limit on a bus's branches is that of 36 more bytes a terminal, which the
+    // kernel once kept there: grids are accepted and refused as ever
+    const size_t limit = *smem + 32u * (size_t)E.max_nt + ((4u * (size_t)E.max_nt + 15u) & ~(size_t)15u);
+    if (limit > kMaxSmem)
         return set_error(PF_EUNSUPPORTED, "an element-wise window needs %u bytes of shared memory (max %u): a bus "
-                                          "has too many branches for this library", (unsigned)*smem, kMaxSmem);
+                                          "has too many branches for this library", (unsigned)limit, kMaxSmem);
     return PF_OK;
 }
 
