@@ -607,8 +607,12 @@ __global__ void __launch_bounds__(256, 5) k_ew_red(EwArgs a)
 
 static bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-// persistent CTAs per SM of the host-output evaluation
-constexpr int kEwHostCtasPerSm = 2;
+// persistent CTAs per SM of the host-output evaluation.  One: since the windows'
+// evaluation got faster, a second CTA per SM only makes two overlapping evaluations
+// get in each other's way on the host link (70,000 buses, eval_host_async on two
+// streams: 17,050 evaluations/s, with two CTAs 16,400-16,700, with three
+// 16,400-16,860; eval_host alone 79 us either way).
+constexpr int kEwHostCtasPerSm = 1;
 
 enum class EwOut { device, host, reduced, ybus };
 
