@@ -49,12 +49,12 @@ EW_OPS_PER_TERMINAL = 12   # E = V_o conj(U_q) 4, G = conj(Yc) E 4, K = v_q G 2,
 EW_OPS_PER_BUS = 16        # phasor (1/v 4, V 2, v^2 1, 2v 1; sin/cos on the integer pipe) + diagonal entries and S (8)
 # of which the kernel runs E, G, V and 2v in fixed point on the integer pipes: what is left on the FP64 pipe
 EW_FP64_PIPE_PER_TERMINAL = 4   # K = v_q G 2, sum K 2
-EW_FP64_PIPE_PER_BUS = 13       # 1/v 4, v^2 1, diagonal entries and S 8
+EW_FP64_PIPE_PER_BUS = 10       # 1/v 4, v conj(Yd) 2, diagonal entries and S 4
 YB_OPS_PER_NNZ = 16
 YB_OPS_PER_ROW = 16
 # DRAM bytes of one k_ew<1> launch on the 70k-bus grid (dram__bytes_read.sum + dram__bytes_write.sum
 # of an ncu capture of that launch); None whenever the kernel changes, until it is captured again
-EW_TRAFFIC_BYTES = 9941504
+EW_TRAFFIC_BYTES = 10014976
 
 
 def parse_args(argv=None):
@@ -1016,7 +1016,7 @@ def main():
             "unit": "GFP64op/s", "frac": achieved / fp64_peak["gdfma_per_s"], "traffic": EW_TRAFFIC_BYTES,
             "ops_per_launch": ops_ew,
             "ops_note": "the method's operations in plain FP64 form (12 per terminal, 16 per bus); the kernel runs "
-                        "8 per terminal and 3 per bus of them in 64-bit fixed point on the integer pipes, %d on "
+                        "8 per terminal and 3 per bus of them in 64-bit fixed point on the integer pipes and shares 3 per bus, %d on "
                         "the FP64 pipe" % (EW_FP64_PIPE_PER_TERMINAL * T + EW_FP64_PIPE_PER_BUS * nb),
             "rate_note": "achieved = operations per evaluation x evaluations per second over the timed region "
                          "(%d CUDA streams, two evaluations' CTAs sharing the SMs); on one stream, launches back "
