@@ -107,6 +107,16 @@ struct MfArgs {
     int *err;
 };
 
+// The kernels of a solve are programmatic dependents of one another: the next
+// one's CTAs start as this one runs out of work, and wait here until it is done
+// (a Newton step at 25,000 buses 520 -> 511 us, four in a power flow at 10,000
+// buses 1,358 -> 1,320).
+__device__ __forceinline__ void mf_begin()
+{
+    pdl_launch_dependents();
+    pdl_wait();
+}
+
 __device__ __forceinline__ int ld_acquire(const int *p)
 {
     int v;
@@ -292,6 +302,7 @@ __device__ __forceinline__ void mf_small_front(const MfArgs &a, const MfFront &f
 
 __global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_small(MfArgs a)
 {
+    mf_begin();
     extern __shared__ __align__(16) double msm[];
     const int lane = threadIdx.x & 31;
     double *S = msm + (size_t)(threadIdx.x >> 5) * (kMfSmall * kMfSmallLd);
@@ -605,6 +616,7 @@ __device__ __forceinline__ int mf_next(const MfArgs &a, int cls, const MfGroup<N
 
 __global__ void __launch_bounds__(32 * kMfMidWarps, 2) k_mf_mid(MfArgs a)
 {
+    mf_begin();
     __shared__ __align__(16) double row[kMfMidRows * 64];
     __shared__ uint64_t bar[kMfMidRows];
     __shared__ int s_next;
@@ -646,6 +658,7 @@ __device__ __forceinline__ void mf_wide_front(const MfArgs &a, const MfFront &fr
 
 __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWideWarps, 1) k_mf_wide(MfArgs a)
 {
+    mf_begin();
     extern __shared__ __align__(16) double msm[];
     __shared__ int s_next;
     uint32_t rank;
@@ -716,6 +729,7 @@ __device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr
 
 __global__ void __launch_bounds__(kMfHugeThreads) k_mf_huge(MfArgs a)
 {
+    mf_begin();
     __shared__ int s_next;
     const MfGroup<1> g(nullptr, nullptr, 0, 0);
     for (int s; (s = mf_next(a, 3, g, &s_next)) >= 0;)
@@ -743,6 +757,7 @@ __global__ void __launch_bounds__(kMfHugeThreads) k_mf_huge(MfArgs a)
 // the same means, 24 -> 20 and 38 -> 32).
 __global__ void __launch_bounds__(kMfBackThreads) k_mf_back_big(MfArgs a)
 {
+    mf_begin();
     extern __shared__ __align__(16) double msm[];
     __shared__ int s_next, s_ok;
     // x of the front (pivots, border) and of the one before; partial sums; pivot rows and y
@@ -865,6 +880,7 @@ __global__ void __launch_bounds__(kMfBackThreads) k_mf_back_big(MfArgs a)
 // loaded while this one is solved, its border's x come from this one's lanes.
 __global__ void __launch_bounds__(32 * kMfSmallWarps) k_mf_back_small(MfArgs a)
 {
+    mf_begin();
     extern __shared__ __align__(16) double msm[];
     const int lane = threadIdx.x & 31;
     double *const Wm = msm + (size_t)(threadIdx.x >> 5) * (2 * kMfBackSmall);   // pivot rows and y of two fronts
@@ -1460,16 +1476,19 @@ cudaError_t launch_lu_solve(Grid *g, const double *Jr, const double *F, double *
     auto ctas = [&](int items, int per_cta, int per_sm) {
         return std::max(1, std::min(per_sm * g->nsm, (items + per_cta - 1) / per_cta));
     };
-    if (a.nleaf[0] > 0)
-        k_mf_small<<<ctas(a.nleaf[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_small, s>>>(a);
-    if (a.nleaf[1] > 0) k_mf_mid<<<ctas(a.nleaf[1], 1, 6), 32 * kMfMidWarps, 0, s>>>(a);
+    bool first = true;
+    auto launch = [&](void (*kernel)(MfArgs), int grid, int block, size_t smem) {
+        if (e == cudaSuccess) e = launch_k(kernel, grid, block, smem, s, !first, a);
+        first = false;
+    };
+    if (a.nleaf[0] > 0) launch(k_mf_small, ctas(a.nleaf[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_small);
+    if (a.nleaf[1] > 0) launch(k_mf_mid, ctas(a.nleaf[1], 1, 6), 32 * kMfMidWarps, 0);
     if (a.nleaf[2] > 0)
-        k_mf_wide<<<kMfWideCtas * std::min(a.nleaf[2], std::max(1, g->nsm / kMfWideCtas)), 32 * kMfWideWarps, sm_wide, s>>>(a);
-    if (a.nleaf[3] > 0) k_mf_huge<<<ctas(a.nleaf[3], 1, 1), kMfHugeThreads, 0, s>>>(a);
-    if (a.npath[1] > 0) k_mf_back_big<<<ctas(a.npath[1], 1, 2), kMfBackThreads, sm_bbig, s>>>(a);
-    if (a.npath[0] > 0)
-        k_mf_back_small<<<ctas(a.npath[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_bsmall, s>>>(a);
-    return cudaGetLastError();
+        launch(k_mf_wide, kMfWideCtas * std::min(a.nleaf[2], std::max(1, g->nsm / kMfWideCtas)), 32 * kMfWideWarps, sm_wide);
+    if (a.nleaf[3] > 0) launch(k_mf_huge, ctas(a.nleaf[3], 1, 1), kMfHugeThreads, 0);
+    if (a.npath[1] > 0) launch(k_mf_back_big, ctas(a.npath[1], 1, 2), kMfBackThreads, sm_bbig);
+    if (a.npath[0] > 0) launch(k_mf_back_small, ctas(a.npath[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_bsmall);
+    return e;
 }
 
 }  // namespace pf
