@@ -609,9 +609,10 @@ static bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // persistent CTAs per SM of the host-output evaluation.  One: since the windows'
 // evaluation got faster, a second CTA per SM only makes two overlapping evaluations
-// get in each other's way on the host link (70,000 buses, eval_host_async on two
-// streams: 17,050 evaluations/s, with two CTAs 16,400-16,700, with three
-// 16,400-16,860; eval_host alone 79 us either way).
+// get in each other's way on the host link.  70,000 buses, evaluations/s of
+// eval_host_async on two streams / of eval_host: bulk stores 17,400-17,600 /
+// 12,900, with two CTAs 16,800 / 12,870; plain stores 16,950-17,140 / 12,670, with
+// two CTAs 16,400-16,700 / 12,650.
 constexpr int kEwHostCtasPerSm = 1;
 
 enum class EwOut { device, host, reduced, ybus };
@@ -662,8 +663,8 @@ static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double
     a.max_nt = L.max_nt;
     a.max_L = L.max_L;
     a.max_nph = max_nph;
-    // bulk (TMA) stores for device outputs; plain coalesced stores for host memory
-    a.aligned = (out == EwOut::device || ybus) && (!J || al16(J)) && (!P || (al16(P) && al16(Q)));
+    // bulk (TMA) stores, to host memory as well; plain coalesced ones where unaligned
+    a.aligned = (!J || al16(J)) && (!P || (al16(P) && al16(Q)));
     a.desc = L.desc;
     a.slotbus = L.slotbus;
     a.bmeta = L.bmeta;
