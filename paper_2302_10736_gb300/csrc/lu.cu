@@ -358,10 +358,11 @@ struct MfGroup {
     int rank;           // this CTA in the cluster
     int gw;             // this warp among the group's
     bool dead;          // a wait ran out: no further waits
+    bool lost;          // ... for a slot to be read out (this thread's)
     uint32_t rrow[NC], rbar[NC];   // row and bar in every CTA of a cluster
 
     __device__ __forceinline__ MfGroup(uint64_t *bar_, double *row_, int rank_, int gw_)
-        : bar(bar_), row(row_), rank(rank_), gw(gw_), dead(false)
+        : bar(bar_), row(row_), rank(rank_), gw(gw_), dead(false), lost(false)
     {
         if (NC > 1)
             for (int q = 0; q < NC; ++q) {
@@ -414,8 +415,23 @@ __device__ __forceinline__ void mf_send(const MfGroup<NC> &g, int slot, int col,
     }
 }
 
-// rows k0 .. k1 - 1 of the batch from their slots to U and y (the CTAs of a group
-// in turn, a warp per row), and the end of their mbarriers
+// Every slot of rows k0 .. k1 - 1 complete in every CTA, before mf_rows_out (every
+// thread; ends with a barrier of the group).  Across a cluster only a slot's own
+// mbarrier tells that its row has arrived: the group's barrier does not order the
+// asynchronous stores, and a warp without later rows has not waited for the slot in
+// the elimination (a root's last row is waited for by none).  So the threads of each
+// CTA look at a slot each; all but the last few have long arrived.
+template <int NC>
+__device__ __forceinline__ void mf_drain(const MfArgs &a, MfGroup<NC> &g, int k0, int k1)
+{
+    if (NC > 1)
+        for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x)
+            if (!g.lost) g.lost = !mf_wait_slot(a, g.bar + (k - k0));
+    g.sync();
+}
+
+// rows k0 .. k1 - 1 of the batch from their slots (drained) to U and y (the CTAs of a
+// group in turn, a warp per row), and the end of their mbarriers
 template <int NC, int C2>
 __device__ __forceinline__ void mf_rows_out(const MfArgs &a, const MfFront &fr, const MfGroup<NC> &g, int k0, int k1)
 {
@@ -484,7 +500,7 @@ __device__ __forceinline__ void mf_pivots(const MfArgs &a, const MfFront &fr, Mf
     const int k1 = min(p, K0 + N);
     for (int k = K0; k < k1; ++k) {
         if (k == kb + rows) {   // the batch's slots are used up
-            g.sync();
+            mf_drain(a, g, kb, k);
             mf_rows_out<NC, C2>(a, fr, g, kb, k);
             g.sync();
             kb = k;
@@ -583,7 +599,7 @@ __device__ __forceinline__ void mf_tile_front(const MfArgs &a, const MfFront &fr
             }
         }
     }
-    g.sync();
+    mf_drain(a, g, kb, p);
     mf_rows_out<NC, C2>(a, fr, g, kb, p);
 }
 
@@ -686,7 +702,7 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
             if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
             s = fr.parent;
         }
-    g.sync();   // no CTA leaves while another may still send to it
+    g.sync();   // every CTA has drained its slots (mf_drain): none is sent to any more
 }
 
 // One front by one CTA in global memory M: any size
