@@ -754,9 +754,11 @@ def _mismatch_loss_function():
 
         @staticmethod
         def forward(ctx, batch, vm, va, g, b, bsh, tap, shift, gs, bs, Pspec, Qspec, wP, wQ):
-            params = [None if x is None else x.contiguous() for x in (g, b, bsh, tap, shift, gs, bs)]
+            # detached: the caller's own objects may hold other values by the time of backward
+            # (p.data = ..., p.set_(...)), these keep the storage that this pass reads
+            params, state = ([None if x is None else x.detach().contiguous() for x in xs]
+                             for xs in ((g, b, bsh, tap, shift, gs, bs), (vm, va, Pspec, Qspec, wP, wQ)))
             grid_set_params(batch.grid, *params)
-            state = [None if x is None else x.contiguous() for x in (vm, va, Pspec, Qspec, wP, wQ)]
             Ltot = torch.empty(1, dtype=torch.float64, device=vm.device)
             loss_elementwise(batch, *state, None, Ltot)
             ctx.batch, ctx.params, ctx.state, ctx.shapes = batch, params, state, (vm.shape, va.shape)
