@@ -614,9 +614,11 @@ pf_status jac_target(pf_grid *grid, int32_t method, const double *vm, const doub
  * asynchronous: a memset of the counters and up to six plain launches (fronts
  * eliminated by a warp, a CTA, a cluster of 8 CTAs, or a CTA in global memory,
  * the forward solve with them; then the backward solve, by CTAs and by warps),
- * fewer where a size does not occur.  Bitwise repeatable.  A zero
- * or non-finite pivot sets the grid's device error word (grid_check_error
- * reports PF_EDEVICE), a wait that runs out (2 s) sets it to a time-out
+ * fewer where a size does not occur.  Bitwise repeatable.  A pattern whose
+ * largest front (dense block of the factorization) has more than about 4,690
+ * unknowns gives PF_EUNSUPPORTED.  A zero or non-finite pivot sets the grid's
+ * device error word (grid_check_error reports PF_EDEVICE), a wait that runs out
+ * (2 s) sets it to a time-out
  * (grid_check_error reports PF_ETIMEOUT and clears it); no pivoting
  * means the matrix must admit LU in that order, which the power-flow Jacobians
  * of this library's grids do (their 2 x 2 bus blocks dominate).

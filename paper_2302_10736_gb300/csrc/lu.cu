@@ -82,7 +82,6 @@ constexpr int kMfMidWarps = 8;        // warps per CTA of the second class
 constexpr int kMfWideWarps = 8, kMfWideCtas = 8;           // of the third
 constexpr int kMfBackSmall = kMfSmall * kMfSmall + kMfSmall;   // doubles of a small front's pivot rows and y
 constexpr int kMfHugeThreads = 512, kMfBackThreads = 512;
-constexpr int kMfBackRows = 160;      // in the limit on the largest front (back_smem)
 constexpr int kMfMidRows = kMfMid;    // pivot rows kept in shared memory at a time: all of a front of the second class
 constexpr size_t kMfWideRowBytes = 200u * 1024u;           // ... and what fits, of the third
 constexpr size_t kMfMaxSmem = 220u * 1024u;
@@ -1358,12 +1357,10 @@ pf_status host_lu(int nb, int n, int npvpq, const std::vector<int> &colptr, cons
     return PF_OK;
 }
 
-// the limit on a front: the shared memory of its x and pivot block
-static size_t back_smem(int fmax, int pmax)
-{
-    const size_t p = (size_t)std::min(pmax, kMfBackRows);
-    return sizeof(double) * (2 * (size_t)fmax + p * (p | 1));
-}
+// doubles of the backward solve without its copies (k_mf_back_big): x of two fronts,
+// four partial sums of every pivot row.  The limit on a front: about 4,690 unknowns,
+// all of them pivots.
+static long long back_fixed(const HostLu &L) { return 2LL * L.backmax + 4LL * ((L.bigp + 31) / 32 * 32); }
 
 // doubles of the backward solve's copies: what a front and the next of its path
 // take, as far as it fits
@@ -1374,7 +1371,7 @@ static int back_room(const HostLu &L)
     for (int h : L.path[1])
         for (int s = h; s >= 0; s = L.fr[s].heavy)
             most = std::max(most, room(L.fr[s]) + (L.fr[s].heavy >= 0 ? room(L.fr[L.fr[s].heavy]) : 0));
-    const long long left = (long long)(kMfMaxSmem / sizeof(double)) - 2 * L.backmax - 4 * ((L.bigp + 31) / 32 * 32);
+    const long long left = (long long)(kMfMaxSmem / sizeof(double)) - back_fixed(L);
     return (int)std::max(0LL, std::min(most, left));
 }
 
@@ -1391,7 +1388,7 @@ pf_status lu_prepare(Grid *g, cudaStream_t s)
             f.m0 = (long long)nmat;
             nmat += (size_t)f.f * ((f.f + 1) | 1);
         }
-    if (back_smem(L.backmax, L.bigp) > kMfMaxSmem)
+    if (back_fixed(L) * (long long)sizeof(double) > (long long)kMfMaxSmem)
         return set_error(PF_EUNSUPPORTED, "jac_reduced_solve: a front of %d unknowns exceeds shared memory", L.backmax);
     const int nf = (int)L.fr.size();
     cudaError_t e = cudaSuccess;
