@@ -612,8 +612,8 @@ pf_status jac_target(pf_grid *grid, int32_t method, const double *vm, const doub
  * the buses, symbolic factorization, fronts), allocates the factor storage and
  * synchronizes; make it before any stream capture.  Every later call is
  * asynchronous: a memset of the counters and up to six plain launches (fronts
- * eliminated by a warp, a CTA, a cluster of 8 CTAs, or a CTA in global memory,
- * the forward solve with them; then the backward solve, by CTAs and by warps),
+ * eliminated by a warp, a CTA, a cluster of 8 CTAs, or, the largest, a cluster in
+ * global memory, the forward solve with them; then the backward solve, by CTAs and by warps),
  * fewer where a size does not occur.  Bitwise repeatable.  A pattern whose
  * largest front (dense block of the factorization) has more than about 4,690
  * unknowns gives PF_EUNSUPPORTED.  A zero or non-finite pivot sets the grid's

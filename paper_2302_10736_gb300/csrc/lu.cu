@@ -43,7 +43,7 @@
 //     backward solve need no FP64 operation of their own.
 // The kernels, by the size of a front (plan_classes): k_mf_small, a warp per front
 // in shared memory; k_mf_mid, a CTA, and k_mf_wide, a cluster of 8 CTAs, with the
-// front in registers; k_mf_huge, a CTA in global memory.  k_mf_back_big,
+// front in registers; k_mf_huge, a cluster in global memory.  k_mf_back_big,
 // k_mf_back_small: the backward solve; a CTA or warp follows one heavy path of the
 // tree down and waits (bounded) only at its head.
 //
@@ -73,7 +73,7 @@ namespace {
 
 constexpr uint64_t kLuWaitNs = 2000000000ull;   // bounded waits (2 s)
 // classes of fronts, by who eliminates them (kMfClasses): a warp, a CTA, a
-// cluster of CTAs, and, beyond those, a CTA with the front in global memory
+// cluster of CTAs, and, beyond those, a cluster with the front in global memory
 constexpr int kMfSmall = 12, kMfMid = 63, kMfWide = 255;   // most unknowns of a front of the first three
 constexpr int kMfNone = (int)0x80000000;   // no source
 constexpr int kMfSmallLd = 13;        // row stride of a small front (odd: no bank conflicts down a column)
@@ -81,7 +81,8 @@ constexpr int kMfSmallWarps = 16;     // warps per CTA of k_mf_small and k_mf_ba
 constexpr int kMfMidWarps = 8;        // warps per CTA of the second class
 constexpr int kMfWideWarps = 8, kMfWideCtas = 8;           // of the third
 constexpr int kMfBackSmall = kMfSmall * kMfSmall + kMfSmall;   // doubles of a small front's pivot rows and y
-constexpr int kMfHugeThreads = 512, kMfBackThreads = 512;
+constexpr int kMfHugeThreads = 512, kMfHugeCtas = 8;       // of the last
+constexpr int kMfBackThreads = 512;
 constexpr int kMfMidRows = kMfMid;    // pivot rows kept in shared memory at a time: all of a front of the second class
 constexpr size_t kMfWideRowBytes = 200u * 1024u;           // ... and what fits, of the third
 constexpr size_t kMfMaxSmem = 220u * 1024u;
@@ -704,12 +705,38 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
     g.sync();   // every CTA has drained its slots (mf_drain): none is sent to any more
 }
 
-// One front by one CTA in global memory M: any size
-__device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr, double *M)
+// One front by a cluster in global memory M, in panels of kMfHugeB pivots:
+//   * every CTA factors the panel's diagonal block for itself, in shared memory (no
+//     barrier of the cluster),
+//   * its pivot rows U and columns L beyond the block, a thread per column or row
+//     of the front (each needs the block only), dealt out over the cluster,
+//   * the rest less L U, in tiles dealt out over the cluster.
+// Every element takes its terms in the order of the pivots, each by one FMA: the
+// result does not depend on the panels.
+// Bound by the cluster's FP64 pipes (2 multiply-adds a cycle and SM: 27 of the 51 ms
+// of 1,598 unknowns) and, at a few hundred unknowns, by the panels' serial steps.
+// One CTA a front, a pivot at a time over all of it, waited for L2 instead.  A solve,
+// ms: complete graphs of 278 / 598 / 1,598 unknowns 4.9 / 47 / 845 -> 1.2 / 4.8 / 51,
+// square meshes of 100 x 100 / 150 x 150 buses (fronts of 304 / 510 unknowns) 16 / 122
+// -> 3.6 / 14.6 (a left-looking factorization by columns: 13 / 59).
+constexpr int kMfHugeB = 32, kMfHugeT = 64;
+constexpr int kMfHugeLd = kMfHugeB + 1;
+
+struct MfHugeSmem {
+    double D[kMfHugeB * kMfHugeLd];    // diagonal block: L, strict upper U
+    double inv[kMfHugeB];              // reciprocals of its pivots
+    double L[kMfHugeT * kMfHugeLd];    // a tile's L and U
+    double U[kMfHugeB * kMfHugeT];
+};
+
+__device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr, double *M,
+                                              const MfGroup<kMfHugeCtas> &g, MfHugeSmem &sm)
 {
-    const int p = fr.p, f = fr.f, ld = (f + 1) | 1, r = f - p;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = kMfHugeThreads >> 5;
-    for (int t = tid; t < f * (f + 1); t += kMfHugeThreads) {
+    constexpr int TB = kMfHugeThreads, B = kMfHugeB, T = kMfHugeT, NW = TB / 32 * kMfHugeCtas;
+    const int p = fr.p, f = fr.f, r = f - p;
+    const size_t ld = (size_t)((f + 1) | 1);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, gt = g.rank * TB + tid;
+    for (int t = gt; t < f * (f + 1); t += kMfHugeCtas * TB) {
         const int2 e[1] = {a.el[fr.s0 + t]};
         double x[1];
         uint32_t rest;
@@ -717,40 +744,125 @@ __device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr
         if (rest) x[0] = mf_gather_rest(a, e[0].y, x[0]);
         M[(size_t)(t / (f + 1)) * ld + t % (f + 1)] = x[0];
     }
-    __syncthreads();
-    for (int k = 0; k < p; ++k) {
-        double *Mk = M + (size_t)k * ld;
-        const double d = Mk[k], inv = fast_rcp(d);
-        __syncthreads();
-        for (int j = k + 1 + tid; j <= f; j += kMfHugeThreads) Mk[j] *= inv;
-        if (tid == 0) pivot_check(a, d);
-        __syncthreads();
-        for (int i = k + 1 + wid; i < f; i += nw) {
-            double *Mi = M + (size_t)i * ld;
-            const double x = -Mi[k];
-            for (int j = k + 1 + lane; j <= f; j += 32) Mi[j] = fma(x, Mk[j], Mi[j]);
+    g.sync();
+    double *U = a.U + fr.u0;
+    for (int k0 = 0; k0 < p; k0 += B) {
+        const int nb = min(B, p - k0), k1 = k0 + nb;
+        // ---- the diagonal block (an identity where the last panel is short) ----
+        for (int t = tid; t < B * B; t += TB) {
+            const int i = t / B, j = t % B;
+            sm.D[i * kMfHugeLd + j] =
+                i < nb && j < nb ? __ldcg(M + (size_t)(k0 + i) * ld + k0 + j) : (i == j ? 1.0 : 0.0);
         }
         __syncthreads();
+        for (int k = 0; k < B; ++k) {
+            if (wid == 0) {
+                const double d = sm.D[k * kMfHugeLd + k], inv = fast_rcp(d);
+                if (lane > k) sm.D[k * kMfHugeLd + lane] *= inv;
+                if (lane == 0) {
+                    sm.inv[k] = inv;
+                    if (g.rank == 0) pivot_check(a, d);
+                }
+            }
+            __syncthreads();
+            for (int i = k + 1 + wid; i < B; i += TB / 32) {
+                double *Di = sm.D + i * kMfHugeLd;
+                if (lane > k) Di[lane] = fma(-Di[k], sm.D[k * kMfHugeLd + lane], Di[lane]);
+            }
+            __syncthreads();
+        }
+        if (g.rank == 0)
+            for (int t = tid; t < B * B; t += TB) {
+                const int i = t / B, j = t % B;
+                if (i < j && j < nb) U[(size_t)(k0 + i) * f + k0 + j] = sm.D[i * kMfHugeLd + j];
+            }
+        // ---- columns k1 .. f of its rows, rows k1 .. f - 1 of its columns ----
+        const int nc = f + 1 - k1, items = nc + f - k1;
+        for (int t = gt; t < items; t += kMfHugeCtas * TB) {
+            double x[B];
+            if (t < nc) {
+                const int j = k1 + t;
+                double *Mj = M + (size_t)k0 * ld + j;
+#pragma unroll
+                for (int k = 0; k < B; ++k) x[k] = k < nb ? __ldcg(Mj + k * ld) : 0.0;
+#pragma unroll
+                for (int k = 0; k < B; ++k) {
+#pragma unroll
+                    for (int m = 0; m < k; ++m) x[k] = fma(-sm.D[k * kMfHugeLd + m], x[m], x[k]);
+                    x[k] *= sm.inv[k];
+                }
+#pragma unroll
+                for (int k = 0; k < B; ++k)
+                    if (k < nb) {
+                        Mj[k * ld] = x[k];
+                        U[j < f ? (size_t)(k0 + k) * f + j : (size_t)p * f + k0 + k] = x[k];
+                    }
+            } else {
+                double *Mi = M + (size_t)(k1 + t - nc) * ld + k0;
+#pragma unroll
+                for (int k = 0; k < B; ++k) x[k] = k < nb ? __ldcg(Mi + k) : 0.0;
+#pragma unroll
+                for (int k = 0; k < B; ++k)
+#pragma unroll
+                    for (int m = 0; m < k; ++m) x[k] = fma(-x[m], sm.D[m * kMfHugeLd + k], x[k]);
+#pragma unroll
+                for (int k = 0; k < B; ++k)
+                    if (k < nb) Mi[k] = x[k];
+            }
+        }
+        g.sync();
+        // ---- the rest, a warp 4 rows of a tile, a lane 2 columns of it ----
+        const int nr = f - k1, tr = (nr + T - 1) / T, tc = (nc + T - 1) / T;
+        for (int t = g.rank; t < tr * tc; t += kMfHugeCtas) {
+            const int i0 = k1 + t / tc * T, j0 = k1 + t % tc * T;
+            double c[4][2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const int i = i0 + 4 * wid + u, j = j0 + lane + 32 * v;
+                    c[u][v] = i < f && j <= f ? __ldcg(M + (size_t)i * ld + j) : 0.0;
+                }
+            for (int x = tid; x < T * B; x += TB) {
+                const int i = i0 + x / B, j = j0 + x % T;
+                sm.L[x / B * kMfHugeLd + x % B] = i < f && x % B < nb ? __ldcg(M + (size_t)i * ld + k0 + x % B) : 0.0;
+                sm.U[x] = j <= f && x / T < nb ? __ldcg(M + (size_t)(k0 + x / T) * ld + j) : 0.0;
+            }
+            __syncthreads();
+            for (int k = 0; k < nb; ++k)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v)
+                        c[u][v] = fma(-sm.L[(4 * wid + u) * kMfHugeLd + k], sm.U[k * T + lane + 32 * v], c[u][v]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const int i = i0 + 4 * wid + u, j = j0 + lane + 32 * v;
+                    if (i < f && j <= f) M[(size_t)i * ld + j] = c[u][v];
+                }
+            __syncthreads();
+        }
+        g.sync();
     }
-    double *U = a.U + fr.u0;
-    for (int i = wid; i < p; i += nw) {
-        for (int j = i + 1 + lane; j < f; j += 32) U[(size_t)i * f + j] = M[(size_t)i * ld + j];
-        if (lane == 0) U[(size_t)p * f + i] = M[(size_t)i * ld + f];
-    }
-    for (int i = wid; i < r; i += nw)
+    for (int i = wid * kMfHugeCtas + g.rank; i < r; i += NW)
         for (int j = lane; j <= r; j += 32)
-            a.cb[fr.c0 + (size_t)i * (r + 1) + j] = M[(size_t)(p + i) * ld + p + j];
+            a.cb[fr.c0 + (size_t)i * (r + 1) + j] = __ldcg(M + (size_t)(p + i) * ld + p + j);
 }
 
-__global__ void __launch_bounds__(kMfHugeThreads) k_mf_huge(MfArgs a)
+__global__ void __cluster_dims__(kMfHugeCtas, 1, 1) __launch_bounds__(kMfHugeThreads, 1) k_mf_huge(MfArgs a)
 {
     mf_begin();
+    __shared__ MfHugeSmem sm;
     __shared__ int s_next;
-    const MfGroup<1> g(nullptr, nullptr, 0, 0);
+    uint32_t rank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const MfGroup<kMfHugeCtas> g(nullptr, nullptr, (int)rank, 0);
     for (int s; (s = mf_next(a, 3, g, &s_next)) >= 0;)
         for (;;) {
             const MfFront fr = a.fr[s];
-            mf_huge_front(a, fr, a.mat + fr.m0);
+            mf_huge_front(a, fr, a.mat + fr.m0, g, sm);
             if (fr.parent_need == 0 || !mf_climb(a, fr, g, &s_next)) break;
             s = fr.parent;
         }
@@ -1498,7 +1610,8 @@ cudaError_t launch_lu_solve(Grid *g, const double *Jr, const double *F, double *
     if (a.nleaf[1] > 0) launch(k_mf_mid, ctas(a.nleaf[1], 1, 6), 32 * kMfMidWarps, 0);
     if (a.nleaf[2] > 0)
         launch(k_mf_wide, kMfWideCtas * std::min(a.nleaf[2], std::max(1, g->nsm / kMfWideCtas)), 32 * kMfWideWarps, sm_wide);
-    if (a.nleaf[3] > 0) launch(k_mf_huge, ctas(a.nleaf[3], 1, 1), kMfHugeThreads, 0);
+    if (a.nleaf[3] > 0)
+        launch(k_mf_huge, kMfHugeCtas * std::min(a.nleaf[3], std::max(1, g->nsm / kMfHugeCtas)), kMfHugeThreads, 0);
     if (a.npath[1] > 0) launch(k_mf_back_big, ctas(a.npath[1], 1, 2), kMfBackThreads, sm_bbig);
     if (a.npath[0] > 0) launch(k_mf_back_small, ctas(a.npath[0], kMfSmallWarps, 2), 32 * kMfSmallWarps, sm_bsmall);
     return e;
