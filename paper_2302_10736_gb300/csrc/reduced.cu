@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(256) k_reduce(int n, int npvpq, int nnz, const
             const long long i = base + u * stride;
             if (i < total) {
                 const double x = ld_after_wait((i < n ? (i < npvpq ? P : Q) : J) + src[u]);
-                val[u] = i < n ? x - (i < npvpq ? Ps : Qs)[src[u]] : x;
+                val[u] = i < n ? x - ld_after_wait((i < npvpq ? Ps : Qs) + src[u]) : x;
             }
         }
 #pragma unroll
