@@ -107,13 +107,16 @@ __device__ __forceinline__ bool scen_yu(const RowOutage &ro, int i, int k, int j
     return true;
 }
 
+// What depends on the parameters (Y, Yf, Ye, tself, tcoup) comes through pointers
+// without __restrict__: loads through a const __restrict__ pointer count as
+// invariant over the kernel and may move above the launch wait.
 template <int W, bool OUT>
 __global__ void __launch_bounds__(512) k_inj_ybus_b(int S, int nb, const int *__restrict__ yrow,
                                                      const int *__restrict__ rp,
-                                                     const int *__restrict__ ci, const double2 *__restrict__ Y,
-                                                     const longlong2 *__restrict__ Yf, const int *__restrict__ Ye,
-                                                     const double2 *__restrict__ tself,
-                                                     const double2 *__restrict__ tcoup,
+                                                     const int *__restrict__ ci, const double2 *Y,
+                                                     const longlong2 *Yf, const int *Ye,
+                                                     const double2 *tself,
+                                                     const double2 *tcoup,
                                                      const ScenOut *__restrict__ sc, const double4_32a *__restrict__ U,
                                                      double *__restrict__ P, double *__restrict__ Q)
 {
@@ -203,10 +206,10 @@ __global__ void __launch_bounds__(512) k_inj_ybus_b(int S, int nb, const int *__
 template <int W, bool OUT>
 __global__ void __launch_bounds__(512) k_jac_ybus_b(int S, int nb, int nnz, const int *__restrict__ yrow,
                                                      const int *__restrict__ rp,
-                                                     const int *__restrict__ ci, const double2 *__restrict__ Y,
-                                                     const longlong2 *__restrict__ Yf, const int *__restrict__ Ye,
-                                                     const double2 *__restrict__ tself,
-                                                     const double2 *__restrict__ tcoup,
+                                                     const int *__restrict__ ci, const double2 *Y,
+                                                     const longlong2 *Yf, const int *Ye,
+                                                     const double2 *tself,
+                                                     const double2 *tcoup,
                                                      const ScenOut *__restrict__ sc,
                                                      const long long *__restrict__ joff,
                                                      const double4_32a *__restrict__ U, double *__restrict__ P,

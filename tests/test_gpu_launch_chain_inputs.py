@@ -1,7 +1,8 @@
-"""Calls issued back to back whose inputs the call just before writes (targets):
-as when each is waited for.  The kernels are launched as programmatic
+"""Calls issued back to back whose inputs the call just before writes (targets,
+parameters): as when each is waited for.  The kernels are launched as programmatic
 dependents of one another, and may start before that call is done.
 """
+import numpy as np
 import pytest
 
 from gridcases import random_grid, random_state
@@ -56,3 +57,24 @@ def test_targets_written_just_before(method, fused):
         pf.jac_reduced(grid, method, *at, Ps, Qs, *out)
 
     _equal_runs(calls, (n, nnz))
+
+
+@pytest.mark.parametrize("jac", [True, False])
+@pytest.mark.parametrize("what", ["batch", "rows", "windows", "elementwise"])
+def test_parameters_set_just_before(what, jac):
+    from paper_2302_10736_gb300 import pfgrid as pf
+    gr = random_grid(NB, NL, 9, shift_max=0.2)
+    grid = pf.ybus_build(gr)
+    pf.grid_set_config(grid, ybus_fused=int(what == "windows"))
+    on = pf.batch_create(grid, 1, np.array([17], np.int32)) if what == "batch" else grid
+    params = [[_dev(gr[k] * f) for k in ("g", "b", "bsh", "tap", "shift", "gs", "bs")] for f in (1.0, 1.01)]
+    at = tuple(_dev(x) for x in random_state(NB, 3))
+    fn = {("batch", True): pf.jac_ybus_batched, ("batch", False): pf.inj_ybus_batched,
+          ("elementwise", True): pf.jac_elementwise, ("elementwise", False): pf.inj_elementwise}.get(
+              (what, jac), pf.jac_ybus if jac else pf.inj_ybus)
+
+    def calls(k, out):
+        pf.grid_set_params(grid, *params[k])
+        fn(on, *at, *out)
+
+    _equal_runs(calls, (NB, NB, on.nnzJ_total if what == "batch" else grid.nnzJ) if jac else (NB, NB))
