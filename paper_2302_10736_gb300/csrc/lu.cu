@@ -713,7 +713,7 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
 //   * the rest less L U, in tiles dealt out over the cluster.
 // Every element takes its terms in the order of the pivots, each by one FMA: the
 // result does not depend on the panels.
-// Bound by the cluster's FP64 pipes (2 multiply-adds a cycle and SM: 27 of the 51 ms
+// Bound by the cluster's FP64 pipes (2 multiply-adds a cycle and SM: 44 of the 51 ms
 // of 1,598 unknowns) and, at a few hundred unknowns, by the panels' serial steps.
 // One CTA a front, a pivot at a time over all of it, waited for L2 instead.  A solve,
 // ms: complete graphs of 278 / 598 / 1,598 unknowns 4.9 / 47 / 845 -> 1.2 / 4.8 / 51,
@@ -1229,7 +1229,9 @@ void plan_classes(std::vector<MfFront> &fr)
                     t[k][q] = std::max(t[k][q], t[k][s]);
                 }
             }
-            // at least the work over what runs at once (warps, CTAs, clusters of 148 SMs)
+            // at least the work over what runs at once (warps, CTAs, clusters), fitted with
+            // the costs above to 148 SMs' worth and 18 clusters: with the part's 152 and 19 a
+            // Newton step at 25,000 buses takes 534 us instead of 512
             const double total = std::max(end[0], work[0] / (148 * 16.0)) + std::max(end[1], work[1] / (148 * 2.0)) +
                                  std::max(end[2], work[2] / 18.0);
             if (total < least) {
