@@ -288,7 +288,8 @@ __global__ void __launch_bounds__(256, 4) k_ewb(BatchArgs a)
             if (JAC && (nq.y & EW_ACCUM)) return;   // with the first branch of its parallel run
             double Gr, Gi;
             window_G(a, p, sA[ol], sU[ol], sv[ol], sU[nq.x], yf, ey, &Gr, &Gi);
-            if (p == sc.ph || p == sc.pk) Gr = Gi = 0.0;   // outage branch
+            const bool out = p == sc.ph || p == sc.pk;   // outage branch
+            if (out) Gr = Gi = 0.0;
             const double vq = sv[nq.x], Kr = vq * Gr, Ki = vq * Gi;   // K_t = v_q G
             if (JAC) {
                 runs |= nq.y;
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(256, 4) k_ewb(BatchArgs a)
                 e[Ls] = neg(Kr);        // J21 = Im(-j K)
                 e[Ls + bm.y] = Gi;      // J22
             } else {
-                sK[i] = make_double2(Kr, Ki);
+                sK[i] = out ? make_double2(0.0, 0.0) : make_double2(Kr, Ki);   // also beside a v_q that is not finite
             }
         };
 #pragma unroll
