@@ -735,29 +735,7 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
     pf_config cfg = g->cfg, keep = g->cfg;
     float best_y = 1e30f, best_e = 1e30f;
     const int lanes[] = {1, 2, 4, 8, 16, 32}, blocks[] = {128, 256, 512};
-    // the row kernels' shape, then the windows (which have none) against it
-    g->cfg.ybus_fused = cfg.ybus_fused = 0;
-    for (int w : lanes)
-        for (int bk : blocks) {
-            g->cfg.ybus_lanes = w;
-            g->cfg.ybus_block = bk;
-            float ms;
-            if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
-            if (ms < best_y) {
-                best_y = ms;
-                cfg.ybus_lanes = w;
-                cfg.ybus_block = bk;
-            }
-        }
-    g->cfg.ybus_lanes = cfg.ybus_lanes;
-    g->cfg.ybus_block = cfg.ybus_block;
-    g->cfg.ybus_fused = 1;
-    {
-        float ms;
-        if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
-        cfg.ybus_fused = ms < best_y;
-    }
-    g->cfg.ybus_fused = cfg.ybus_fused;
+    // the windows first: the Ybus method's one-launch form runs on them too
     for (int win : {128, 256}) {
         pf_config c2 = g->cfg;
         c2.ew_window = win;
@@ -775,8 +753,29 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
             cfg.ew_window = win;
         }
     }
-    st = grid_set_config(grid, &cfg, stream);
-    if (!st) g->ybus_shape_set = 1;
+    if ((st = grid_set_config(grid, &cfg, stream))) goto out;
+    // the row kernels' shape, then the windows (which have none) against it
+    g->cfg.ybus_fused = 0;
+    for (int w : lanes)
+        for (int bk : blocks) {
+            g->cfg.ybus_lanes = w;
+            g->cfg.ybus_block = bk;
+            float ms;
+            if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
+            if (ms < best_y) {
+                best_y = ms;
+                cfg.ybus_lanes = w;
+                cfg.ybus_block = bk;
+            }
+        }
+    g->cfg.ybus_fused = 1;
+    {
+        float ms;
+        if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
+        cfg.ybus_fused = ms < best_y;
+    }
+    g->cfg = cfg;
+    g->ybus_shape_set = 1;
 out:
     if (st) g->cfg = keep;
     cudaFree(ctx.P);
