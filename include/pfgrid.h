@@ -377,7 +377,11 @@ typedef struct {
  * the batch workspaces (phasors, residuals and flow sums, 80 bytes per scenario-bus) and
  * synchronizes `stream`.  If the environment variable PFGRID_TUNE_CACHE names
  * a tuning cache file (written by batch_autotune) that holds a configuration
- * for this GPU and the batch's size class, the batch starts with it.
+ * for this GPU and the batch's size class, the batch starts with it.  Its Ybus
+ * row kernels else start with the grid's ybus_lanes and ybus_block if
+ * grid_set_config has changed these from their initial 4 and 256, and with a
+ * shape by nscen * nb if they are the initial or grid_autotune's (which are
+ * for a single state).
  */
 pf_status batch_create(pf_grid *grid, int32_t nscen, const int32_t *outage, pf_stream stream, pf_batch **out);
 

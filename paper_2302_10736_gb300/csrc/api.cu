@@ -312,6 +312,8 @@ PF_API pf_status pf_debug_fail_allocations(int32_t after)
     return PF_OK;
 }
 
+static constexpr pf_config kDefaultConfig{4, 256, 256, 1};   // lanes, block, ew_window, fused
+
 PF_API pf_status ybus_build(const pf_grid_desc *d, pf_stream stream, pf_grid **out)
 {
     if (!out) return set_error(PF_EINVAL, "ybus_build: out is NULL");
@@ -324,10 +326,7 @@ PF_API pf_status ybus_build(const pf_grid_desc *d, pf_stream stream, pf_grid **o
     Grid *g = &pg->g;
     g->nb = d->nb;
     g->nl = d->nl;
-    g->cfg.ybus_lanes = 4;
-    g->cfg.ybus_block = 256;
-    g->cfg.ew_window = 256;
-    g->cfg.ybus_fused = 1;
+    g->cfg = kDefaultConfig;
     if ((st = host_topology(d->nb, d->nl, d->from, d->to, g->topo))) {
         delete pg;
         return st;
@@ -651,7 +650,10 @@ PF_API pf_status grid_set_config(pf_grid *grid, const pf_config *cfg, pf_stream 
         if (st) return st;
         PF_CUDA(cudaStreamSynchronize(s));
     }
-    if (cfg->ybus_lanes != g->cfg.ybus_lanes || cfg->ybus_block != g->cfg.ybus_block) g->ybus_shape_set = 1;
+    // a shape other than the initial one is the program's choice for batches too
+    if (cfg->ybus_lanes != g->cfg.ybus_lanes || cfg->ybus_block != g->cfg.ybus_block)
+        g->ybus_shape_set =
+            cfg->ybus_lanes != kDefaultConfig.ybus_lanes || cfg->ybus_block != kDefaultConfig.ybus_block;
     g->cfg = *cfg;
     return PF_OK;
 }
@@ -775,7 +777,7 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
         cfg.ybus_fused = ms < best_y;
     }
     g->cfg = cfg;
-    g->ybus_shape_set = 1;
+    g->ybus_shape_set = 0;   // fastest for one state: no choice for a batch's many rows
 out:
     if (st) g->cfg = keep;
     cudaFree(ctx.P);

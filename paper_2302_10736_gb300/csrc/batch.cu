@@ -192,7 +192,7 @@ PF_API pf_status batch_create(pf_grid *grid, int32_t nscen, const int32_t *outag
     b->cfg.terminals_per_thread = 0;   // chosen by batch_plan
     b->cfg.ctas_per_sm = 0;
     b->cfg.adjoint_form = 0;
-    // the grid's row-kernel shape where the program chose one, else by size
+    // the grid's row-kernel shape where the program set another than the initial one, else by size
     b->cfg.ybus_lanes = g->cfg.ybus_lanes;
     b->cfg.ybus_block = g->cfg.ybus_block;
     if (!g->ybus_shape_set) ybus_rows_shape((long long)nscen * g->nb, b->cfg);

@@ -273,7 +273,7 @@ struct NewtonResult {
 struct Grid {
     int nb = 0, nl = 0, nnz = 0;
     pf_config cfg{};
-    int ybus_shape_set = 0;   // cfg's row-kernel shape was set or tuned (batches then start from it)
+    int ybus_shape_set = 0;   // cfg's row-kernel shape is one that the program set (batches then start from it)
     DevArena arena;
     HostTopo topo;
     // Ybus (device)

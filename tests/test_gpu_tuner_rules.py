@@ -26,3 +26,35 @@ def test_ybus_form_is_timed_on_the_windows_kept():
     assert max(i for i, k in enumerate(names) if k == "jac_ew") < names.index("jac_ybus")
     assert pf.grid_get_config(grid) == best
     assert max(pf.grid_ew_windows(grid)[:, 3]) <= best["ew_window"]   # the layout in place is the one named
+
+
+def test_shape_a_batch_starts_from():
+    """By size unless the program has set another shape than the initial one,
+    however it came to the present one."""
+    from paper_2302_10736_gb300 import pfgrid as pf
+    nb = 700
+    grid = pf.ybus_build(random_grid(nb, 930, 9))
+
+    def shape():
+        c = pf.batch_get_config(pf.batch_create(grid, 3))
+        return c["ybus_lanes"], c["ybus_block"]
+
+    by_size = shape()
+    assert by_size[1] == 64
+    first = pf.grid_get_config(grid)
+    pf.grid_set_config(grid, **first)   # the initial shape, named
+    assert shape() == by_size
+    pf.grid_set_config(grid, ybus_lanes=16, ybus_block=128)
+    assert shape() == (16, 128)
+    pf.grid_set_config(grid, ew_window=128)   # something else
+    assert shape() == (16, 128)
+    pf.grid_set_config(grid, **first)   # and back
+    assert shape() == by_size
+    pf.grid_set_config(grid, ybus_lanes=16, ybus_block=128)
+    pf.grid_autotune(grid, *(_dev(x) for x in random_state(nb, 1)), reps=1)   # one state's shape
+    assert shape() == by_size
+    pf.grid_set_config(grid, ew_window=128)
+    assert shape() == by_size
+    lanes = 32 if pf.grid_get_config(grid)["ybus_lanes"] != 32 else 16   # another than the tuner's
+    pf.grid_set_config(grid, ybus_lanes=lanes, ybus_block=512)
+    assert shape() == (lanes, 512)
