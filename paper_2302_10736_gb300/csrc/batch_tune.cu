@@ -460,25 +460,27 @@ PF_API pf_status batch_autotune(pf_batch *batch, const double *vm, const double 
         }
         if (st) break;
     }
-    // the batched Ybus method: lanes per row x CTA size (independent of the windows)
+    // the batched Ybus method: the present shape, then lanes per row x CTA size (independent of the windows)
     if (st == PF_OK && (st = batch_apply_config(b, win, s)) == PF_OK && (kernels & PF_TUNE_YBUS)) {
         float yb_best = 0.0f;
         bool yhave = false;
         pf_batch_config ywin = win;
-        for (int lanes : {1, 2, 4, 8, 16, 32}) {
-            for (int blk : {128, 256, 512}) {
-                b->cfg.ybus_lanes = lanes;
-                b->cfg.ybus_block = blk;
-                float ms = 0.0f;
-                if ((st = time_launches(yb, reps, s, e0, e1, &ms))) break;
-                if (!yhave || ms < yb_best) {
-                    yb_best = ms;
-                    ywin = b->cfg;
-                    yhave = true;
-                }
+        auto shape = [&](int lanes, int blk) -> pf_status {
+            b->cfg.ybus_lanes = lanes;
+            b->cfg.ybus_block = blk;
+            float ms = 0.0f;
+            if (pf_status e = time_launches(yb, reps, s, e0, e1, &ms)) return e;
+            if (!yhave || ms < yb_best) {
+                yb_best = ms;
+                ywin = b->cfg;
+                yhave = true;
             }
-            if (st) break;
-        }
+            return PF_OK;
+        };
+        st = shape(cur.ybus_lanes, cur.ybus_block);
+        for (int lanes : {1, 2, 4, 8, 16, 32})
+            for (int blk : {64, 128, 256, 512})
+                if (st == PF_OK) st = shape(lanes, blk);
         win.ybus_lanes = ywin.ybus_lanes;
         win.ybus_block = ywin.ybus_block;
     }

@@ -58,3 +58,19 @@ def test_shape_a_batch_starts_from():
     lanes = 32 if pf.grid_get_config(grid)["ybus_lanes"] != 32 else 16   # another than the tuner's
     pf.grid_set_config(grid, ybus_lanes=lanes, ybus_block=512)
     assert shape() == (lanes, 512)
+
+
+def test_batch_tuner_times_the_present_shape_and_64_threads():
+    """batch_autotune's Ybus candidates: the shape in place, and 6 lane counts by 4
+    CTA sizes, the default one (64 threads) among them; each is launched once and
+    then timed."""
+    from paper_2302_10736_gb300 import pfgrid as pf
+    nb, S, reps = 300, 4, 3
+    grid = pf.ybus_build(random_grid(nb, 420, 9))
+    batch = pf.batch_create(grid, S)
+    pf.batch_set_config(batch, ybus_lanes=2, ybus_block=96)
+    vm, va = random_state(nb, 1, S)
+    pf.grid_trace_enable(grid, 1 << 12)
+    pf.batch_autotune(batch, _dev(vm.ravel()), _dev(va.ravel()), reps=reps, kernels=2)
+    names = [k for k, _ in pf.grid_trace_read(grid)]
+    assert names == ["jac_ybus_batched"] * ((1 + 6 * 4) * (1 + reps))
