@@ -213,7 +213,8 @@ static pf_status ew_fits(const HostEw &E, size_t *smem)
     const EwSmem plan = ew_smem_plan(E.max_nbus, E.max_nt, E.max_L, true, E.max_nph);
     *smem = plan.total + kTrigSmem;
     // the limit on a bus's branches is that of 36 more bytes a terminal, which the
-    // kernel once kept there: grids are accepted and refused as ever
+    // kernel once kept there (a star of 1,879 branches; with what it also kept per bus,
+    // 1,844)
     const size_t limit = *smem + 32u * (size_t)E.max_nt + ((4u * (size_t)E.max_nt + 15u) & ~(size_t)15u);
     if (limit > kMaxSmem)
         return set_error(PF_EUNSUPPORTED, "an element-wise window needs %u bytes of shared memory (max %u): a bus "
@@ -231,19 +232,12 @@ static pf_status build_ew_layout(Grid *g, int tb, cudaStream_t s)
     PF_CUDA(cudaGetDevice(&dev));
     PF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     PF_CUDA(ew_blocks_per_sm(tb, smem, &per_sm));
-    for (int pass = 0; pass < 2 && per_sm > 0 && E.nwin > 1; ++pass) {
-        const long long wave = (long long)nsm * per_sm;
-        const int target = ew_target_windows(E.nwin, nsm, wave);
-        if (target == 0) break;
-        HostEw B;
-        size_t smem_b = 0;
-        if ((st = host_ew(g->topo, tb, B, 1, target)) || (st = ew_fits(B, &smem_b))) return st;
-        int per_sm_b = 0;
-        PF_CUDA(ew_blocks_per_sm(tb, smem_b, &per_sm_b));
-        E = std::move(B);
-        if (per_sm_b >= per_sm) break;   // the balanced windows still fit as planned
-        per_sm = per_sm_b;               // fewer fit: balance again for the smaller wave
-    }
+    if (per_sm > 0 && E.nwin > 1)
+        if (const int target = ew_target_windows(E.nwin, nsm, (long long)nsm * per_sm)) {
+            HostEw B;
+            if ((st = host_ew(g->topo, tb, B, 1, target)) || (st = ew_fits(B, &smem))) return st;
+            E = std::move(B);
+        }
 #ifdef PF_SELFCHECK
     if ((st = host_selfcheck(g->topo, E))) return st;
 #endif
