@@ -78,10 +78,6 @@ struct EwArgs {
     const int2 *binv;
     const double *Ps, *Qs;
     double *F, *Jr;
-    // the Ybus method's general row (ybus_row): terminals of every bus and
-    // their {other bus, slot position | flags}
-    const int *tp;
-    const int2 *tnbr;
 };
 
 #ifdef PF_PHASE_PROBE
@@ -131,8 +127,16 @@ __device__ __forceinline__ void store_range(double *x, const double *s, int b0, 
 // values in terminal order, zero for the run's later terminals).  Rows with a
 // magnitude whose products or quotient might leave the range of normal
 // doubles, or with a non-finite angle, are evaluated whole from their current in
-// FP64 instead (ybus_row), after the others: one call, with little live around it
-// (calls among the evaluation's products and sums: 10.1 against 9.4 us at 70,000 buses).
+// FP64 instead (ybus_row), after the others (calls among the evaluation's products
+// and sums, with their spills: 10.1 against 9.4 us at 70,000 buses).  So is a row whose
+// own magnitude is zero, since its conj(I_i) U_i is no quotient; zero entries (branches
+// out of service) and zero magnitudes of other buses are ordinary factors.
+// The rows of a window that go that way are listed first and taken a lane each:
+// an FP64 instruction costs a warp the same for one lane as for 32.  70,000 buses, a
+// Jacobian, us: 1 % of the branches out of service 8.3, as without; 1 % / 10 % of the
+// buses dead 17.3 / 20.2 (34.3, and 33.5 / 50.2, with zeros among the extreme values,
+// each row by the two threads of its bus and its phasors formed anew; row kernels with
+// the sine and cosine per entry 21).
 //
 // Why windows: with W lanes per CSR row and the sine and cosine per entry
 // (the earlier one-launch form) every bus was transformed 3.5 times and the
@@ -145,66 +149,66 @@ constexpr int kYbusSlowRow = (int)0x80000000;
 // a biased exponent within 2^-300 .. 2^300
 __device__ __forceinline__ bool ybus_mid(int e) { return (unsigned)(e - 723) <= 600u; }
 
-// Y_oq of the entry whose parallel run starts at sorted terminal p, summed as
-// k_ybus_values sums it
-__device__ __forceinline__ double2 ybus_entry(const EwArgs &a, int p)
+// or zero: a product with it is exact
+__device__ __forceinline__ bool ybus_mid_or_zero(double v)
 {
-    double2 y = make_double2(0.0, 0.0);
-    const int pe = a.tp[a.town[p] + 1];
-    do {
-        const double2 c = a.tcoup[p];
-        y.x += c.x;
-        y.y += c.y;
-        ++p;
-    } while (p < pe && (a.tnbr[p].y & EW_ACCUM));
-    return y;
+    return ybus_mid(fix_vexp(v)) || (dbl_bits(v) << 1) == 0;
 }
 
 // Row o by its current I_o (Eqs. 1, 3, 4) in FP64, in the order of operations of
-// a row kernel's lane (k_jac_ybus_b): its entries into the window's J slice (row:
-// its P half's first, d entries, the Q half L behind; NULL: the injections alone)
-// and S_o
-__device__ __noinline__ void ybus_row(const EwArgs &a, int o, double *row, int L, int d, double *P, double *Q)
+// a row kernel's lane (k_jac_ybus_b), from the window's phasors: its sorted terminals
+// from p on, the row's own phasor slot b and diagonal position kd; its d entries into
+// the window's J slice (row: its P half's first, the Q half L behind; NULL: the
+// injections alone) and S_o
+__device__ __noinline__ void ybus_row(const EwArgs &a, const longlong2 *sU, const double2 *sW, int o, int b, int p,
+                                      int kd, double *row, int L, int d, double *P, double *Q)
 {
-    double so, co;
-    int_sincos(a.va[o], a.trig, &so, &co);
-    const double v = a.vm[o], Vr = v * co, Vi = v * so;
+    auto cosine = [&](int j, double &s) {
+        const longlong2 u = sU[j];
+        const double c = fix_q62_or_nan(u.x);
+        s = u.x == kFixNaN ? c : q62_to_double(u.y);
+        return c;
+    };
+    double so;
+    const double co = cosine(b, so);
+    const double v = sW[b].x, Vr = v * co, Vi = v * so;
     double Ir = 0.0, Ii = 0.0, dTr = 0.0, dTi = 0.0, dVr = 0.0, dVi = 0.0;
-    const int pe = a.tp[o + 1];
-    int k = 0, kd = -1;   // the row's entries in column order; the diagonal's place
-    for (int p = a.tp[o]; p < pe || kd < 0;) {
-        const int2 nq = p < pe ? a.tnbr[p] : make_int2(o + 1, 0);
-        const bool own = kd < 0 && nq.x > o;   // the diagonal's turn
-        if (!own && (nq.y & EW_ACCUM)) {
-            ++p;
-            continue;
+#pragma unroll 1
+    for (int k = 0; k < d; ++k) {   // in column order
+        const bool own = k == kd;
+        double2 y;
+        int j = b;
+        if (own) {
+            y = a.yd[o];
+        } else {
+            int2 f = a.tloc[p];
+            j = f.x;
+            y = make_double2(0.0, 0.0);
+            for (;; f = a.tloc[p]) {   // the entry's parallel run, as k_ybus_values sums it
+                const double2 c = a.tcoup[p++];
+                y.x += c.x;
+                y.y += c.y;
+                if (!(f.y & EW_MORE)) break;
+            }
         }
-        const int j = own ? o : nq.x;
-        const double2 y = own ? a.yd[o] : ybus_entry(a, p);
-        double s, c;
-        int_sincos(a.va[j], a.trig, &s, &c);
-        const double vj = a.vm[j];
+        double s;
+        const double c = cosine(j, s), vj = sW[j].x;
         const double YUr = fma(y.x, c, -y.y * s), YUi = fma(y.x, s, y.y * c);
         const double sVr = fma(Vr, YUr, Vi * YUi), sVi = fma(Vi, YUr, -Vr * YUi);   // V conj(YU)
         const double sTr = vj * sVi, sTi = -vj * sVr;
         Ir = fma(vj, YUr, Ir);
         Ii = fma(vj, YUi, Ii);
         if (own) {
-            kd = k;
             dTr = sTr;
             dTi = sTi;
             dVr = sVr;
             dVi = sVi;
-        } else {
-            ++p;
-            if (row) {
-                row[k] = sTr;
-                row[k + d] = sVr;
-                row[L + k] = sTi;
-                row[L + k + d] = sVi;
-            }
+        } else if (row) {
+            row[k] = sTr;
+            row[k + d] = sVr;
+            row[L + k] = sTi;
+            row[L + k + d] = sVi;
         }
-        ++k;
     }
     const double Sr = fma(Vr, Ir, Vi * Ii), Si = fma(Vi, Ir, -Vr * Ii);
     if (row) {
@@ -381,7 +385,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
             if (YBUS) {
                 // magnitudes whose products might leave the doubles' range, and
                 // non-finite angles: the row goes the general way
-                if (!(ybus_mid(ey) && ybus_mid(fix_vexp(vq)) && uq.x != kFixNaN) || A.x == kFixNaN ||
+                if (!(ybus_mid(ey) && ybus_mid_or_zero(vq) && uq.x != kFixNaN) || A.x == kFixNaN ||
                     !fix_G_fast(A.x, A.y, vo, uq.x, uq.y, yf.x, yf.y, ey, &Gr, &Gi)) {
                     Gr = Gi = 0.0;
                     sbm[ol].z |= kYbusSlowRow;
@@ -490,13 +494,29 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                     spq[(im ? pqs : 0) + b + par] = fma(v * v, im ? neg(y.y) : y.x, sK);   // S = v^2 conj(Yd) + sum K
             }
         }
-        if (YBUS && slow_row)   // their entries, over those that the evaluation wrote
-            for (int x = tid; x < 2 * nbus; x += TB) {
-                const int b = sord[x >> 1];
-                const int4 bm = sbm[b];
-                if (bm.z < 0 && !(x & 1))
-                    ybus_row(a, b0 + b, JAC ? jst + bm.x : nullptr, L, bm.y, spq + b + par, spq + pqs + b + par);
+        // everything staged, the rows of the general way (over what the evaluation
+        // wrote of them) last; ends with a barrier
+        auto staged = [&]() {
+            fence_proxy_async_smem();
+            if (!YBUS) {
+                __syncthreads();
+                return;
             }
+            if (!__syncthreads_or(slow_row)) return;
+            __shared__ int nslow;
+            if (tid == 0) nslow = 0;
+            __syncthreads();
+            if (tid < nbus && sbm[tid].z < 0) sord[atomicAdd(&nslow, 1)] = tid;   // the order of the sums is used up
+            __syncthreads();
+            for (int x = tid; x < nslow; x += TB) {
+                const int b = sord[x];
+                const int4 bm = sbm[b];
+                ybus_row(a, sU, sW, b0 + b, b, t0 + bm.w, bm.z & ~kYbusSlowRow, JAC ? jst + bm.x : nullptr, L, bm.y,
+                         spq + b + par, spq + pqs + b + par);
+            }
+            fence_proxy_async_smem();
+            __syncthreads();
+        };
 
         // ---- stores ----
         if (RED) {
@@ -530,8 +550,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                     a.Q[b0 + b] = spq[pqs + b + par];
                 }
         } else if (a.aligned) {
-            fence_proxy_async_smem();
-            __syncthreads();
+            staged();
             PF_PROBE_MARK(3);
             if (tid == 0) {
                 if (JAC) {
@@ -546,7 +565,7 @@ __device__ __forceinline__ void ew_windows(const EwArgs &a)
                 bulk_wait_read();   // shared memory stays allocated until the copies have read it
             }
         } else {
-            __syncthreads();
+            staged();
             if (JAC) {
                 double *Jp = a.J + 2 * (long long)r0;
                 double *Jq = a.J + 2 * (long long)a.nnz + 2 * (long long)r0;
@@ -674,8 +693,6 @@ static cudaError_t launch_ew(Grid *g, const double *vm, const double *va, double
     a.tcoup = g->tcoup;
     a.tcfx = ybus ? g->ytfx : g->tcfx;
     a.tce = ybus ? g->yte : g->tce;
-    a.tp = g->tp;
-    a.tnbr = g->tnbr;
     a.trig = trig_table();
     a.tloc = L.tloc;
     a.vm = vm;

@@ -101,10 +101,11 @@ __global__ void __launch_bounds__(128) k_ybus_values(int nnz, const int *__restr
         yd[d] = acc;
         return;
     }
-    // in terminal order: the entry at its run's first terminal, a zero with a
-    // representable exponent (no slow path) at the later ones
+    // in terminal order: the entry at its run's first terminal, a zero at the later
+    // ones.  A zero (also an entry's: a branch out of service) gets a representable
+    // exponent, which keeps its row on the usual path.
     ytfx[p0] = make_longlong2(fr, fi);
-    yte[p0] = ye;
+    yte[p0] = acc.x == 0.0 && acc.y == 0.0 ? 1023 : ye;
     for (int p = p0 + 1; p < p1; ++p) {
         ytfx[p] = make_longlong2(0, 0);
         yte[p] = 1023;
