@@ -101,9 +101,9 @@ __device__ __forceinline__ double2 fix_V_double(int64_t C, int64_t S, double v)
     return make_double2(v * c, v * s);
 }
 
-// phase 1 of the adjoint: the fixed-point phasors of every scenario as in
-// batch_phasors_fix (1/v with the gradients), and V as doubles for the
-// branch-parameter gradients; chunks of blockDim.x consecutive buses, so that
+// phase 1 of the adjoint: the fixed-point phasors of every scenario, U = {2^62 cos,
+// 2^62 sin (64-bit integers stored bit for bit), v, 1/v with the gradients}, and V as
+// doubles for the branch-parameter gradients; chunks of blockDim.x consecutive buses, so that
 // every lane has a bus
 __device__ __forceinline__ void batch_phasors_adj(const BatchArgs &a, const ITrig *tab, bool grad)
 {

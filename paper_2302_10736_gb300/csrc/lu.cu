@@ -158,12 +158,6 @@ __device__ __forceinline__ bool mf_wait_slot(const MfArgs &a, uint64_t *bar)
     }
 }
 
-__device__ __forceinline__ double warp_sum_d(double x)
-{
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    return x;
-}
-
 __device__ __forceinline__ void pivot_check(const MfArgs &a, double d)
 {
     if (!(fabs(d) > 0.0) || !isfinite(d)) atomicExch(a.err, DEV_SINGULAR);

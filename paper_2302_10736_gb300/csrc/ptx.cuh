@@ -1,6 +1,6 @@
 // ptx.cuh - thin inline-PTX helpers for sm_100+/sm_103a: mbarrier, bulk
-// (TMA, non-tensor) copies between global and shared memory, programmatic
-// dependent launch controls.
+// (TMA, non-tensor) copies from shared to global memory, the grid barrier,
+// programmatic dependent launch controls.
 #pragma once
 
 #include <cstdint>
@@ -9,9 +9,6 @@ namespace pf {
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Bring the line of a valid global address into L2 (a hint: no data returned,
-// no ordering; L2 is the point of coherence, so a later load after a
-// programmatic-dependent-launch wait still sees what the previous grid wrote)
 // 8 bytes to shared memory without a register; the thread's copies are done after cp_async_wait_all
 __device__ __forceinline__ void cp_async8(double *smem, const double *gmem)
 {
@@ -19,6 +16,10 @@ __device__ __forceinline__ void cp_async8(double *smem, const double *gmem)
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Bring the line of a valid global address into L2 (a hint: no data returned,
+// no ordering; L2 is the point of coherence, so a later load after a
+// programmatic-dependent-launch wait still sees what the previous grid wrote)
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
@@ -56,26 +57,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t phase)
         : "r"(smem_addr(bar)), "r"(phase)
         : "memory");
     return ok != 0;
-}
-
-// Bounded wait on phase `phase`: gives up after `limit` polls (each try_wait
-// suspends the thread for a hardware-chosen while), returns false then.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t phase, uint32_t limit)
-{
-    for (uint32_t i = 0; i < limit; ++i) {
-        if (mbar_try_wait(bar, phase)) return true;
-        __nanosleep(64);
-    }
-    return false;
-}
-
-// global -> shared bulk copy completing on `bar` (16-byte aligned, size % 16 == 0)
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
 }
 
 // shared -> global bulk copy in the current bulk group (16-byte aligned, size % 16 == 0)
