@@ -754,9 +754,9 @@ def _mismatch_loss_function():
 
         @staticmethod
         def forward(ctx, batch, vm, va, g, b, bsh, tap, shift, gs, bs, Pspec, Qspec, wP, wQ):
-            # detached: the caller's own objects may hold other values by the time of backward
-            # (p.data = ..., p.set_(...)), these keep the storage that this pass reads
-            params, state = ([None if x is None else x.detach().contiguous() for x in xs]
+            # the caller's own objects may hold other values by the time of backward (p.data = ...,
+            # p.set_(...)); these keep the storage that this pass reads (.data as detach(), in half its time)
+            params, state = ([None if x is None else x.data.contiguous() for x in xs]
                              for xs in ((g, b, bsh, tap, shift, gs, bs), (vm, va, Pspec, Qspec, wP, wQ)))
             grid_set_params(batch.grid, *params)
             Ltot = torch.empty(1, dtype=torch.float64, device=vm.device)
