@@ -707,8 +707,8 @@ __global__ void __cluster_dims__(kMfWideCtas, 1, 1) __launch_bounds__(32 * kMfWi
 //   * the rest less L U, in tiles dealt out over the cluster.
 // Every element takes its terms in the order of the pivots, each by one FMA: the
 // result does not depend on the panels.
-// Bound by the cluster's FP64 pipes (2 multiply-adds a cycle and SM: 44 of the 51 ms
-// of 1,598 unknowns) and, at a few hundred unknowns, by the panels' serial steps.
+// Bound by the cluster's FP64 pipes (at the 528 G multiply-adds a second of all
+// SMs, 49 of the 51 ms of 1,598 unknowns) and, at a few hundred unknowns, by the panels' serial steps.
 // One CTA a front, a pivot at a time over all of it, waited for L2 instead.  A solve,
 // ms: complete graphs of 278 / 598 / 1,598 unknowns 4.9 / 47 / 845 -> 1.2 / 4.8 / 51,
 // square meshes of 100 x 100 / 150 x 150 buses (fronts of 304 / 510 unknowns) 16 / 122
@@ -748,8 +748,9 @@ __device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr
             sm.D[i * kMfHugeLd + j] =
                 i < nb && j < nb ? __ldcg(M + (size_t)(k0 + i) * ld + k0 + j) : (i == j ? 1.0 : 0.0);
         }
+        if (tid >= nb && tid < B) sm.inv[tid] = 1.0;
         __syncthreads();
-        for (int k = 0; k < B; ++k) {
+        for (int k = 0; k < nb; ++k) {
             if (wid == 0) {
                 const double d = sm.D[k * kMfHugeLd + k], inv = fast_rcp(d);
                 if (lane > k) sm.D[k * kMfHugeLd + lane] *= inv;
@@ -759,7 +760,7 @@ __device__ __forceinline__ void mf_huge_front(const MfArgs &a, const MfFront &fr
                 }
             }
             __syncthreads();
-            for (int i = k + 1 + wid; i < B; i += TB / 32) {
+            for (int i = k + 1 + wid; i < nb; i += TB / 32) {
                 double *Di = sm.D + i * kMfHugeLd;
                 if (lane > k) Di[lane] = fma(-Di[k], sm.D[k * kMfHugeLd + lane], Di[lane]);
             }

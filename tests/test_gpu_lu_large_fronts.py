@@ -40,3 +40,22 @@ def test_large_front_below_a_large_front(own, shared):
     bt[0] = 3
     bt[5::7] = 2
     fronts._check(make_grid(nb, br), bt)
+
+
+@pytest.mark.parametrize("core,own,shared", [(3, 150, 2), (9, 140, 1), (40, 131, 5)])
+def test_small_fronts_above_a_large_front(core, own, shared):
+    """A large front whose border reaches small ones: its ancestors are of its class,
+    with panels of a few pivots."""
+    rng = np.random.default_rng(own)
+    br = fronts._clique(list(range(core)), rng)
+    new = list(range(core, core + own))
+    at = list(range(shared))
+    br += [e for e in fronts._clique(at + new, rng) if not (e[0] in at and e[1] in at)]
+    nb = core + own
+    for k in range(5):   # a chain of small cliques off the core
+        ring = list(range(nb, nb + 4))
+        nb += 4
+        br += fronts._clique([core - 1 - k % core] + ring, rng)
+    bt = np.ones(nb, np.int32)
+    bt[nb - 1] = 3
+    fronts._check(make_grid(nb, br), bt)
