@@ -374,7 +374,7 @@ typedef struct {
  * keeps them; its values start at offset joff[s] of the batch's J array
  * (batch_jac_offsets), nnzJ_s = 4 (nnzY - 2 removed).  outage is a host array
  * read during the call; values outside [-1, nl) give PF_EINVAL.  Allocates
- * the batch workspaces (phasors, residuals and flow sums, 80 bytes per scenario-bus) and
+ * the batch workspaces (phasors and residuals, 64 bytes per scenario-bus) and
  * synchronizes `stream`.  If the environment variable PFGRID_TUNE_CACHE names
  * a tuning cache file (written by batch_autotune) that holds a configuration
  * for this GPU and the batch's size class, the batch starts with it.  Its Ybus

@@ -211,7 +211,6 @@ PF_API pf_status batch_create(pf_grid *grid, int32_t nscen, const int32_t *outag
     cudaError_t e = cudaSuccess;
     if ((e = b->arena.alloc(&b->sc, std::max(nscen, 1))) || (e = b->arena.alloc(&b->joff, nscen + 1)) ||
         (e = b->arena.alloc(&b->U, n)) || (e = b->arena.alloc(&b->V, n)) || (e = b->arena.alloc(&b->r, n)) ||
-        (e = b->arena.alloc(&b->sk, n)) ||
         (e = b->arena.alloc(&b->lscen, std::max(nscen, 1))) ||
         (nscen && (e = cudaMemcpyAsync(b->sc, b->h_sc.data(), sizeof(ScenOut) * nscen, cudaMemcpyHostToDevice, st))) ||
         (e = cudaMemcpyAsync(b->joff, b->h_joff.data(), sizeof(long long) * (nscen + 1), cudaMemcpyHostToDevice,

@@ -66,7 +66,7 @@ struct BatchArgs {
     int *err;
     // adjoint
     const double *Ps, *Qs, *wP, *wQ;
-    double2 *r, *sk;   // residuals; sum K of every bus
+    double2 *r;   // residuals
     double *lpart, *L, *gvm, *gva, *gg, *gb, *gbsh, *gtap;
     const double *Lbar;      // upstream gradient (device scalar; NULL = 1): scales every gradient
     double *Ltot;            // sum_s L_s (may be NULL)
@@ -636,7 +636,8 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
             const double wp = a.wP[o], wq = a.wQ[o];
             if (GRAD) {
                 a.r[sb + o] = make_double2(tl * wp * dP, tl * wq * dQ);
-                a.sk[sb + o] = make_double2(sKr, sKi);
+                a.gva[sb + o] = sKr;   // sum K, where the gradients will be (phase 3)
+                a.gvm[sb + o] = sKi;
             }
             spq[x] = fma(wp * dP, dP, wq * dQ * dQ);
         }
@@ -686,7 +687,7 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
             }
             const int q = b0 + b;
             const double4_32a uq = a.U[sb + q];
-            const double2 rq = a.r[sb + q], sk = a.sk[sb + q];
+            const double2 rq = a.r[sb + q], sk = make_double2(a.gva[sb + q], a.gvm[sb + q]);
             const double2 y = syd[b];
             // <r_q, j sum K> + v_q (sum), and <r_q, 2 v_q conj(Yd)> + <r_q, sum K> / v_q + (sum)
             spq[b + par] = fma(uq.z, gth, fma(-rq.x, sk.y, rq.y * sk.x));
@@ -694,7 +695,7 @@ __global__ void __launch_bounds__(256, 4) k_adj(BatchArgs a)
                                      fma(uq.w, fma(rq.x, sk.x, rq.y * sk.y), gv));
         }
         if (a.aligned) {
-            fence_proxy_async_smem();
+            fence_proxy_async();   // the staged gradients, and the sums read where they go
             __syncthreads();
             if (tid == 0) {
                 store_range_ll(a.gva, spq, sb + b0, sb + b1);
@@ -1093,7 +1094,6 @@ static BatchArgs batch_args(Batch *b)
     a.bar = g->bar;
     a.err = g->err;
     a.r = b->r;
-    a.sk = b->sk;
     a.lpart = b->lpart;
     a.pg = g->p_g;
     a.pb = g->p_b;

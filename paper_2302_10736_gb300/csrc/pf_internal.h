@@ -477,7 +477,6 @@ struct Batch {
     double4_32a *U = nullptr;        // [S][nb]
     double2 *V = nullptr;            // [S][nb]
     double2 *r = nullptr;            // [S][nb] loss residual (2 wP dP, 2 wQ dQ)
-    double2 *sk = nullptr;           // [S][nb] sum of the bus's flows K (adjoint)
     double *lpart = nullptr;         // [S][nwin] per-window loss partial sums
     double *lscen = nullptr;         // [S] per-scenario losses when the caller wants only their total
     // co-resident CTAs of the batched kernels (inj, jac, adjoint, k_adj1, and

@@ -74,6 +74,8 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 
 // order this thread's generic-proxy shared-memory writes before later async-proxy reads
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// the same for global memory too, for bulk copies to where this thread's generic accesses were
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
 // Grid-wide barrier for a cooperative launch (every CTA resident).  `state`
 // (zero initially) holds a launch parity at [0] and two arrival counters at
