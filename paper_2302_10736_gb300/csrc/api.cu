@@ -729,9 +729,24 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
     PF_CUDA(cudaMalloc(&ctx.Q, (size_t)g->nb * 8));
     PF_CUDA(cudaMalloc(&ctx.J, (size_t)4 * g->nnz * 8 + 8));
     pf_config cfg = g->cfg, keep = g->cfg;
+    const int keep_set = g->ybus_shape_set;
     float best_y = 1e30f, best_e = 1e30f;
     const int lanes[] = {1, 2, 4, 8, 16, 32}, blocks[] = {128, 256, 512};
-    // the windows first: the Ybus method's one-launch form runs on them too
+    // the row kernels' shape (whatever the windows; and the device is warm after it)
+    g->cfg.ybus_fused = 0;
+    for (int w : lanes)
+        for (int bk : blocks) {
+            g->cfg.ybus_lanes = w;
+            g->cfg.ybus_block = bk;
+            float ms;
+            if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
+            if (ms < best_y) {
+                best_y = ms;
+                cfg.ybus_lanes = w;
+                cfg.ybus_block = bk;
+            }
+        }
+    // the windows, then on those kept the Ybus method's one-launch form against the rows
     for (int win : {128, 256}) {
         pf_config c2 = g->cfg;
         c2.ew_window = win;
@@ -750,20 +765,6 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
         }
     }
     if ((st = grid_set_config(grid, &cfg, stream))) goto out;
-    // the row kernels' shape, then the windows (which have none) against it
-    g->cfg.ybus_fused = 0;
-    for (int w : lanes)
-        for (int bk : blocks) {
-            g->cfg.ybus_lanes = w;
-            g->cfg.ybus_block = bk;
-            float ms;
-            if ((st = time_it(&ms, reps, s, run_jac_ybus, &ctx))) goto out;
-            if (ms < best_y) {
-                best_y = ms;
-                cfg.ybus_lanes = w;
-                cfg.ybus_block = bk;
-            }
-        }
     g->cfg.ybus_fused = 1;
     {
         float ms;
@@ -773,7 +774,10 @@ PF_API pf_status grid_autotune(pf_grid *grid, const double *vm, const double *va
     g->cfg = cfg;
     g->ybus_shape_set = 0;   // fastest for one state: no choice for a batch's many rows
 out:
-    if (st) g->cfg = keep;
+    if (st) {
+        g->cfg = keep;
+        g->ybus_shape_set = keep_set;
+    }
     cudaFree(ctx.P);
     cudaFree(ctx.Q);
     cudaFree(ctx.J);

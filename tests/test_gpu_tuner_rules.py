@@ -14,8 +14,8 @@ def _dev(x):
 
 
 def test_ybus_form_is_timed_on_the_windows_kept():
-    """grid_autotune settles the windows before it times the Ybus forms, one of
-    which runs on them."""
+    """grid_autotune settles the windows before it times the Ybus form that runs on
+    them (one launch; the other form's row kernel comes after a phasor launch)."""
     from paper_2302_10736_gb300 import pfgrid as pf
     grid = pf.ybus_build(random_grid(700, 930, 9))
     vm, va = (_dev(x) for x in random_state(700, 1))
@@ -23,7 +23,8 @@ def test_ybus_form_is_timed_on_the_windows_kept():
     best = pf.grid_autotune(grid, vm, va, reps=2)
     names = [k for k, _ in pf.grid_trace_read(grid)]
     assert "jac_ew" in names and "jac_ybus" in names
-    assert max(i for i, k in enumerate(names) if k == "jac_ew") < names.index("jac_ybus")
+    one = [i for i, k in enumerate(names) if k == "jac_ybus" and (i == 0 or names[i - 1] != "phasor")]
+    assert one and max(i for i, k in enumerate(names) if k == "jac_ew") < one[0]
     assert pf.grid_get_config(grid) == best
     assert max(pf.grid_ew_windows(grid)[:, 3]) <= best["ew_window"]   # the layout in place is the one named
 
