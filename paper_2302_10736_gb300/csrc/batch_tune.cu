@@ -460,7 +460,7 @@ PF_API pf_status batch_autotune(pf_batch *batch, const double *vm, const double 
         }
         if (st) break;
     }
-    // the batched Ybus method: the present shape, then lanes per row x CTA size (independent of the windows)
+    // the batched Ybus method: lanes per row x CTA size (independent of the windows), and the present shape
     if (st == PF_OK && (st = batch_apply_config(b, win, s)) == PF_OK && (kernels & PF_TUNE_YBUS)) {
         float yb_best = 0.0f;
         bool yhave = false;
@@ -477,10 +477,10 @@ PF_API pf_status batch_autotune(pf_batch *batch, const double *vm, const double 
             }
             return PF_OK;
         };
-        st = shape(cur.ybus_lanes, cur.ybus_block);
         for (int lanes : {1, 2, 4, 8, 16, 32})
             for (int blk : {64, 128, 256, 512})
                 if (st == PF_OK) st = shape(lanes, blk);
+        if (st == PF_OK) st = shape(cur.ybus_lanes, cur.ybus_block);   // last: the device is warm
         win.ybus_lanes = ywin.ybus_lanes;
         win.ybus_block = ywin.ybus_block;
     }
