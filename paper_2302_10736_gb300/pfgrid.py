@@ -137,7 +137,7 @@ def header_functions():
 # its caller waits for: torch.cuda.current_stream() builds a Stream object
 # (3 us; the raw handle of the same stream 0.2), and a ctypes argument of type
 # c_void_p takes a plain integer as it is.  jac_elementwise on 118 buses, calls back
-# to back: 10.4 -> 4.8 us; a training step of MismatchLoss at 25,000 buses 394 -> 303.
+# to back: 10.4 -> 4.8 us; a training step of MismatchLoss at 25,000 buses 394 -> 312.
 _Tensor = _f64 = _raw_stream = _device = None
 
 
