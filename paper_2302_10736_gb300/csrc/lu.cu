@@ -853,7 +853,7 @@ __global__ void __cluster_dims__(kMfHugeCtas, 1, 1) __launch_bounds__(kMfHugeThr
     __shared__ int s_next;
     uint32_t rank;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const MfGroup<kMfHugeCtas> g(nullptr, nullptr, (int)rank, 0);
+    const MfGroup<kMfHugeCtas> g(reinterpret_cast<uint64_t *>(sm.inv), sm.D, (int)rank, 0);   // its barrier alone is used
     for (int s; (s = mf_next(a, 3, g, &s_next)) >= 0;)
         for (;;) {
             const MfFront fr = a.fr[s];

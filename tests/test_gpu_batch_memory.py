@@ -9,8 +9,10 @@ pytestmark = pytest.mark.gpu
 
 
 def test_workspace_per_scenario_and_bus():
+    import gc
     import torch
     from paper_2302_10736_gb300 import pfgrid as pf
+    gc.collect()   # nothing of earlier tests is freed meanwhile
     nb, S = 20000, 256
     grid = pf.ybus_build(random_grid(nb, 26400, 9))
     keep = pf.batch_create(grid, 1)   # what any batch holds of the grid's size
